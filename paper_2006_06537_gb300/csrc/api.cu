@@ -100,6 +100,12 @@ static size_t fused_mv_part_doubles(const Plan* P, const fifa_opts& o) {
   return (size_t)std::min(P->nleaf, FS_CTAS_MAX) * std::max(1, std::min(P->L, 10)) * FIFA_CAP_MAX * SWEEP_RHS_MAX;
 }
 
+// Level barriers: one set per rank bucket of every level with CTA groups, so one
+// clear serves a whole factorization.
+static size_t level_bar_bytes(const Plan* P) {
+  return sizeof(unsigned int) * LEVEL_BUCKETS * (size_t)P->lvl_ctas_max * std::max(1, P->lvl_grouped);
+}
+
 // Host part of a plan: bounds, ACA / level / sweep groups, scratch size.
 // aca_cores / lvl_cores[b]: co-resident CTA budgets of the ACA kernel and of
 // the level kernel of rank bucket b.
@@ -220,7 +226,9 @@ static Plan* plan_build(int64_t n, const fifa_opts& o, int aca_cores, const int*
   }
   P->lvl_ctas_max = (int)lvl_ctas;
   add(sizeof(double) * 2 * lvl_ctas * level_part_stride(cap));           // level partials (2 slots)
-  add(sizeof(unsigned int) * LEVEL_BUCKETS * lvl_ctas);                  // level barriers, one set per rank bucket
+  for (int l = 0; l < P->L; ++l)
+    if (std::max({P->lvl_G[0][l], P->lvl_G[1][l], P->lvl_G[2][l]}) > 1) P->lvl_grouped = l + 1;  // a prefix of the levels
+  add(level_bar_bytes(P));                                                // level barriers
   add(sizeof(double) * sweep_ctas * 2 * cap * SWEEP_RHS_MAX);            // sweep partials
   add(sizeof(double) * (size_t)P->nleaf * std::max(1, P->L) * cap * SWEEP_RHS_MAX);  // matvec partials
   add(sizeof(double) * (size_t)std::max(1, P->nnodes) * 2 * cap * SWEEP_RHS_MAX);     // matvec projections
@@ -386,7 +394,7 @@ Scratch carve(fifa_ctx* ctx, Plan* P) {
   S.aca_part = (ArgMax*)take((size_t)3 * sizeof(ArgMax) * std::max(1, P->aca_ncoop));
   S.aca_bar = (unsigned int*)take(sizeof(unsigned int) * std::max(1, P->aca_ncoop));
   S.lvl_part = (double*)take(sizeof(double) * 2 * (size_t)P->lvl_ctas_max * level_part_stride(cap));
-  S.lvl_bar = (unsigned int*)take(sizeof(unsigned int) * LEVEL_BUCKETS * P->lvl_ctas_max);
+  S.lvl_bar = (unsigned int*)take(level_bar_bytes(P));
   int64_t sweep_ctas = 1;
   for (int l = 0; l < P->L; ++l) sweep_ctas = std::max<int64_t>(sweep_ctas, ((int64_t)1 << l) * P->sweep_G[l]);
   S.sweep_part = (double*)take(sizeof(double) * sweep_ctas * 2 * cap * SWEEP_RHS_MAX);
@@ -791,13 +799,17 @@ fifa_status fact_enqueue(fifa_ctx* ctx, fifa_fact* F, const HmatDesc* Hdev) {
   return st == FIFA_OK ? fact_enqueue_part(ctx, F, Hdev, 1) : st;
 }
 
-// The deepest level whose level kernels split no node over a CTA group: levels
-// >= it run with independent CTAs (groups only ever take the top levels).
+// Largest side of a node of level l.
+static int level_side_max(const Plan* P, int l) { return (int)(((n_of(P) + ((int64_t)1 << l) - 1) >> l) + 1) / 2; }
+
+// The deepest level whose level kernels split no node over a waiting CTA group:
+// levels >= it run with independent CTAs or clusters (groups only ever take the
+// top levels).
 int fact_ungrouped_from(const Plan* P) {
   int l = P->L;
   while (l > 0) {
     const int q = l - 1;
-    if (std::max({P->lvl_G[0][q], P->lvl_G[1][q], P->lvl_G[2][q]}) > 1) break;
+    if (q < P->lvl_grouped && !level_clustered(level_side_max(P, q))) break;
     l = q;
   }
   return l;
@@ -819,14 +831,14 @@ fifa_status fact_enqueue_part(fifa_ctx* ctx, fifa_fact* F, const HmatDesc* Hdev,
     CK(launch_leaf_factor(Hdev, F->dev, prec, P->nleaf, P->Bm, P->L, cap, s));
   }
   const int lhi = part == 0 ? P->L - 1 : lsplit - 1, llo = part == 0 ? lsplit : 0;
+  if (llo < P->lvl_grouped && lhi >= llo) {
+    CK(cudaMemsetAsync(S.lvl_bar, 0, level_bar_bytes(P), s));
+    CK(cudaMemsetAsync(S.flags, 0, sizeof(int), s));
+  }
   for (int l = lhi; l >= llo; --l) {
     const int Gb[LEVEL_BUCKETS] = {P->lvl_G[0][l], P->lvl_G[1][l], P->lvl_G[2][l]};
-    if (*std::max_element(Gb, Gb + LEVEL_BUCKETS) > 1) {  // every rank bucket has its own barrier set
-      CK(cudaMemsetAsync(S.lvl_bar, 0, sizeof(unsigned int) * LEVEL_BUCKETS * P->lvl_ctas_max, s));
-      CK(cudaMemsetAsync(S.flags, 0, sizeof(int), s));
-    }
-    const int side_max = (int)(((n_of(P) + ((int64_t)1 << l) - 1) >> l) + 1) / 2;
-    CK(launch_level(F->dev, prec, l, 1 << l, Gb, cap, S.lvl_part, S.lvl_bar, P->lvl_ctas_max, S.flags, side_max, s));
+    unsigned int* bar = S.lvl_bar + (l < P->lvl_grouped ? (size_t)l * LEVEL_BUCKETS * P->lvl_ctas_max : 0);
+    CK(launch_level(F->dev, prec, l, 1 << l, Gb, cap, S.lvl_part, bar, P->lvl_ctas_max, S.flags, level_side_max(P, l), s));
   }
   if (part == 0) return FIFA_OK;
   CK(launch_logdet_reduce(F->dev, s));
@@ -848,15 +860,15 @@ fifa_status fact_enqueue_batched(fifa_ctx* ctx, Plan* P, FactDesc* F0, const Hma
   const int cap = ctx->opts.rank_cap;
   CK(launch_prep_fact(F0, H0, P->nnodes, s, nprob));
   CK(launch_leaf_factor(H0, F0, prec, P->nleaf, P->Bm, P->L, cap, s, nprob));
+  if (P->lvl_grouped > 0) {
+    CK(cudaMemset2DAsync(S.lvl_bar, sstride, 0, level_bar_bytes(P), nprob, s));
+    CK(cudaMemset2DAsync(S.flags, sstride, 0, sizeof(int), nprob, s));
+  }
   for (int l = P->L - 1; l >= 0; --l) {
     int Gb[LEVEL_BUCKETS];
     for (int b = 0; b < LEVEL_BUCKETS; ++b) Gb[b] = std::max(1, P->lvl_G[b][l] / nprob);
-    if (*std::max_element(Gb, Gb + LEVEL_BUCKETS) > 1) {
-      CK(cudaMemset2DAsync(S.lvl_bar, sstride, 0, sizeof(unsigned int) * LEVEL_BUCKETS * P->lvl_ctas_max, nprob, s));
-      CK(cudaMemset2DAsync(S.flags, sstride, 0, sizeof(int), nprob, s));
-    }
-    const int side_max = (int)(((n_of(P) + ((int64_t)1 << l) - 1) >> l) + 1) / 2;
-    CK(launch_level(F0, prec, l, 1 << l, Gb, cap, S.lvl_part, S.lvl_bar, P->lvl_ctas_max, S.flags, side_max, s, nprob,
+    unsigned int* bar = S.lvl_bar + (l < P->lvl_grouped ? (size_t)l * LEVEL_BUCKETS * P->lvl_ctas_max : 0);
+    CK(launch_level(F0, prec, l, 1 << l, Gb, cap, S.lvl_part, bar, P->lvl_ctas_max, S.flags, level_side_max(P, l), s, nprob,
                     sstride));
   }
   CK(launch_logdet_reduce(F0, s, nprob));

@@ -340,7 +340,7 @@ __device__ inline bool group_barrier(unsigned int* counter, unsigned int target,
         ok = 0;
         break;
       }
-      __nanosleep(64);
+      if (spins > 256) __nanosleep(64);  // the others are usually a microsecond away
     }
     __threadfence();
   }

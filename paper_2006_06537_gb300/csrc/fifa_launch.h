@@ -15,23 +15,29 @@ cudaError_t launch_aca(const HmatDesc* Hd, const int4* work, int ncta, bool coop
 int aca_max_coresident_ctas();
 
 size_t leaf_factor_smem(int Bm, int L, int cap, int prec);
-size_t level_smem(int ldm, int cap);
-// Doubles per CTA slot of the level kernel's partial sums: a cap x cap Gram
-// matrix or a 2cap x 8 projection block.
-__host__ __device__ inline size_t level_part_stride(int cap) {
-  // the larger of the packed Gram entries of both sides, r (r + 1) <= cap (cap + 1),
-  // and a 2 cap x 8 projection chunk
-  return (size_t)(cap * (cap + 1) > 2 * cap * 8 ? cap * (cap + 1) : 2 * cap * 8);
-}
+// Doubles per CTA slot of the level kernels' partial sums: the packed Gram
+// entries of both sides, r (r + 1) <= cap (cap + 1), and projections of at least
+// eight ancestor columns.
+__host__ __device__ inline size_t level_part_stride(int cap) { return (size_t)cap * (cap + 1) + (size_t)2 * cap * 8; }
+// Nodes of at most this many rows are factored by a thread-block cluster, larger
+// ones by a group of CTAs (eight CTAs of a cluster hold 256 rows each, the
+// fewest a group's CTA gets).
+#define LEVEL_CLUSTER_ROWS 2048
+inline bool level_clustered(int side_max) { return 2 * side_max <= LEVEL_CLUSTER_ROWS; }
 cudaError_t launch_leaf_factor(const HmatDesc* Hd, const FactDesc* Fd, int prec, int nleaf, int Bm, int L, int cap,
                                cudaStream_t st, int nprob = 1);
 #define LEVEL_BUCKETS 3
 // Level kernels: rank buckets (.., 4], (4, 16], (16, cap] with groups of G[b]
-// CTAs; bucket b uses the barriers at bar + b * bar_stride.
+// CTAs (clusters for small nodes); bucket b uses the barriers at bar + b * bar_stride.
 // nprob problems in one launch (grid.y): descriptor arrays, scratch sstride bytes apart.
 cudaError_t launch_level(const FactDesc* Fd, int prec, int lvl, int nodes, const int* G, int cap, double* part,
                          unsigned int* bar, int bar_stride, int* abort_flag, int side_max, cudaStream_t st,
                          int nprob = 1, size_t sstride = 0);
+// k_node.cu: rank bucket rb (4: all ranks <= 4; 16: ranks in (rlo, 16]) with a
+// cluster or a co-resident group of G CTAs per node; ranks <= skip are left out.
+cudaError_t launch_node(const FactDesc* Fd, int rb, int rlo, bool cluster, int lvl, int nodes, int G, double* part,
+                        unsigned int* bar, int* abort_flag, int skip, cudaStream_t st, int nprob, size_t sstride);
+int node_ctas_per_sm(int rb);
 // Co-resident CTAs of the level kernel of rank bucket b (0: <= 4, 1: 5..16, 2: > 16).
 int level_bucket_coresident(int prec, int b, int cap);
 cudaError_t launch_logdet_reduce(const FactDesc* Fd, cudaStream_t st, int nprob = 1);

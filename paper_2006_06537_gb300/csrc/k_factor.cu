@@ -6,21 +6,23 @@
 //                  memory, log-det partial, and L_i^-1 applied to the rows of
 //                  every ancestor basis lying in the leaf (the first transform),
 //                  the first chunk of those columns inside the Cholesky steps.
-//  k_level       : per node of one level (bottom-up), the orthonormal bases
-//                  Q_U, Q_V of the transformed U~, V~ by CholeskyQR2 (two Gram
-//                  passes; stable here because the column-scaled bases are
-//                  well conditioned), R = R2 R1, L_S = chol(I + R X R^T),
-//                  Zf = L_S - I, Zi = L_S^-1 - I, and the inverse node factor
-//                  I + Q Zi Q^T applied to every ancestor basis on the node's rows.
-//                  Large nodes: G CTAs split the rows and exchange partial sums
-//                  through bounded-spin group barriers.
+//  k_level       : (k_node.cu) per node of one level (bottom-up), ranks <= 16: the
+//                  orthonormal bases Q_U, Q_V of the transformed U~, V~ by
+//                  CholeskyQR2 (two Gram passes; stable here because the
+//                  column-scaled bases are well conditioned), R = R2 R1,
+//                  L_S = chol(I + R X R^T), Zf = L_S - I, Zi = L_S^-1 - I, and
+//                  the inverse node factor I + Q Zi Q^T applied to every
+//                  ancestor basis on the node's rows.
+//  k_level_wide  : the same for ranks above 16.  Large nodes: G CTAs split the
+//                  rows and exchange partial sums through bounded-spin group
+//                  barriers.
 //  k_level_multi : the same for the deepest levels (sides of <= 128 rows,
-//                  rank <= 4), several nodes per CTA staged in shared memory;
-//  k_level_small : rank 5..8 nodes of those levels, one CTA each.
+//                  rank <= 4), several nodes per CTA staged in shared memory.
 #include <algorithm>
 #include <atomic>
 #include "fifa_common.cuh"
 #include "fifa_launch.h"
+#include "fifa_level.cuh"
 
 // Ancestor columns per right-hand-side chunk of the leaf TRSM: the first chunk
 // is eliminated together with the Cholesky steps, later chunks (more ancestor
@@ -192,14 +194,12 @@ __global__ void __launch_bounds__(256, 7) k_leaf_factor(const HmatDesc* __restri
 }
 
 // ---------------------------------------------------------------------------
-// General level kernel (large nodes, ranks above the small-node buckets).  Row
-// transforms and updates are row-parallel with coalesced column accesses;
-// reductions over rows use the tiled output-major helpers below; small dense
-// algebra (r <= cap) runs in shared memory.
+// Level kernel for ranks above 16.  Row transforms and updates are
+// row-parallel with coalesced column accesses; reductions over rows use the
+// tiled output-major helpers; small dense algebra (r <= cap) runs in shared
+// memory.
 // ---------------------------------------------------------------------------
-// Ancestor columns per update chunk (the same for every rank bucket: 16 for the
-// rank <= 4 kernel measured slower, its accumulators spill).
-#define LEVEL_W(RB) 8
+#define LEVEL_W 8  // ancestor columns per update chunk
 #define LV_RED 64
 
 // Serial upper Cholesky of A (r x r, ld) in place by one thread, pivots from
@@ -238,37 +238,15 @@ __device__ inline void thr_triinv_upper(const double* R, int ldr, const double* 
     }
 }
 
-template <typename T, int RB>
-__device__ __forceinline__ void rowmul_row(T* __restrict__ Xb, int64_t n, int r, int p, const double* Ri, int ldr) {
-  double x[RB];
-#pragma unroll
-  for (int c = 0; c < RB; ++c) x[c] = c < r ? to_d(Xb[(size_t)c * n + p]) : 0.0;
-#pragma unroll
-  for (int c = 0; c < RB; ++c) {
-    if (c < r) {
-      double v = 0.0;
-#pragma unroll
-      for (int a = 0; a <= c; ++a) v += x[a] * Ri[a * ldr + c];
-      Xb[(size_t)c * n + p] = (T)v;
-    }
-  }
-}
-
 // Rows [a0, a1): X[:, p] <- X[:, p] Ri (r x r upper triangular, shared, ld ldr).
 template <typename T>
 __device__ void rowmul_pass(T* __restrict__ Xb, int64_t n, int r, int a0, int a1, const double* Ri, int ldr) {
-  for (int p = a0 + threadIdx.x; p < a1; p += blockDim.x) {
-    if (r <= 4) rowmul_row<T, 4>(Xb, n, r, p, Ri, ldr);
-    else if (r <= 8) rowmul_row<T, 8>(Xb, n, r, p, Ri, ldr);
-    else if (r <= 16) rowmul_row<T, 16>(Xb, n, r, p, Ri, ldr);
-    else {
-      for (int c = r - 1; c >= 0; --c) {  // right to left: column c reads only columns <= c
-        double v = 0.0;
-        for (int a = 0; a <= c; ++a) v += to_d(Xb[(size_t)a * n + p]) * Ri[a * ldr + c];
-        Xb[(size_t)c * n + p] = (T)v;
-      }
+  for (int p = a0 + threadIdx.x; p < a1; p += blockDim.x)
+    for (int c = r - 1; c >= 0; --c) {  // right to left: column c reads only columns <= c
+      double v = 0.0;
+      for (int a = 0; a <= c; ++a) v += to_d(Xb[(size_t)a * n + p]) * Ri[a * ldr + c];
+      Xb[(size_t)c * n + p] = (T)v;
     }
-  }
   __syncthreads();
 }
 
@@ -312,114 +290,6 @@ __device__ void update_pass(const T* __restrict__ Qb, T* const* Bp, int w, int64
 // precondition an FP64 iteration (0: plain Cholesky, failures are reported).
 template <typename T> __device__ __forceinline__ double clamp_gram() { return sizeof(T) == 4 ? 1e-12 : 0.0; }
 template <typename T> __device__ __forceinline__ double clamp_cap() { return sizeof(T) == 4 ? 1e-6 : 0.0; }
-
-// Reduce `count` doubles of the G partials of this group (slot order fixed)
-// into dst; if G == 1 the partial already sits in dst.  The G partials of each
-// output are split over the CTA's threads in chunks and the chunk sums
-// combined by a pairwise tree in `red` (>= blockDim.x doubles of shared
-// memory), so a large group costs a few loads per thread, not G serial ones.
-__device__ inline bool group_reduce(double* dst, const double* src_local, int count, int G, int g, int base,
-                                    double* part, size_t pstride, unsigned int* bar, unsigned int& phase,
-                                    int* status, int* abort_flag, double* red, unsigned int spin) {
-  if (G == 1) return true;
-  // two slot sets alternate with the barrier count: a slot is rewritten only
-  // after a later barrier that every reader of its previous contents has passed
-  const size_t set = (size_t)(phase & 1u) * gridDim.x;
-  double* mine = part + (set + base + g) * pstride;
-  for (int t = threadIdx.x; t < count; t += blockDim.x) mine[t] = src_local[t];
-  ++phase;
-  if (!group_barrier(bar + base, (unsigned)G * phase, status, abort_flag, spin)) return false;
-  const double* slots = part + (set + base) * pstride;
-  if (count >= (int)blockDim.x) {
-    for (int t = threadIdx.x; t < count; t += blockDim.x) {
-      double v = 0.0;
-      for (int q = 0; q < G; ++q) v += __ldcg(slots + (size_t)q * pstride + t);
-      dst[t] = v;
-    }
-    __syncthreads();
-    return true;
-  }
-  const int nch = min(G, (int)blockDim.x / count);
-  const int t = threadIdx.x;
-  if (t < nch * count) {
-    const int o = t % count, ch = t / count;
-    double v = 0.0;
-    for (int q = ch; q < G; q += nch) v += __ldcg(slots + (size_t)q * pstride + o);
-    red[ch * count + o] = v;
-  }
-  __syncthreads();
-  for (int w = nch; w > 1;) {
-    const int hw = (w + 1) / 2;
-    for (int i = t; i < (w - hw) * count; i += blockDim.x) red[i] += red[i + hw * count];
-    w = hw;
-    __syncthreads();
-  }
-  for (int o = t; o < count; o += blockDim.x) dst[o] = red[o];
-  __syncthreads();
-  return true;
-}
-
-
-// ---------------------------------------------------------------------------
-// Tiled, output-major reductions for the general level kernel: tiles of rows
-// are staged in shared memory (coalesced loads, two buffers: the next tile's
-// asynchronous copies are in flight while the current one is reduced), each
-// output entry is owned by a group of threads that walk disjoint rows of the
-// tile, and the groups' partial sums are combined by a short pairwise tree.
-// FP64 instructions go to products of nonzero entries only.
-// ---------------------------------------------------------------------------
-#define LV_TR 128  // rows per staged tile
-#define LV_TRP (LV_TR + 1)
-
-__device__ __forceinline__ void pair_decode(int o, int r, int& a, int& b) {
-  int rem = o;
-  a = 0;
-  while (rem >= r - a) {
-    rem -= r - a;
-    ++a;
-  }
-  b = a + rem;
-}
-
-// 8-byte asynchronous global -> shared copy (cp.async), its group commit and wait.
-__device__ __forceinline__ void cp_async8(double* sdst, const void* gsrc) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(sdst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gsrc) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_prev() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-
-// Stage rows [p0, p0 + tr) of ncol columns (column c at col(c)) into a tile
-// (column c at c * LV_TRP): asynchronous copies for FP64 storage, converting
-// loads for FP32 storage.
-template <typename T, typename ColF>
-__device__ __forceinline__ void stage_tile(double* tile, int ncol, int p0, int tr, ColF col) {
-  for (int i = threadIdx.x; i < ncol * tr; i += blockDim.x) {
-    const int c = i / tr, p = i - c * tr;
-    const T* src = col(c) + p0 + p;
-    if constexpr (sizeof(T) == sizeof(double)) cp_async8(tile + c * LV_TRP + p, src);
-    else tile[c * LV_TRP + p] = to_d(*src);
-  }
-}
-
-// Walk the tiles of rows [a0, a1) with double buffering: body(tile, tr) runs on
-// each staged tile by every thread (tbuf: doubles per buffer).
-template <typename T, typename ColF, typename BodyF>
-__device__ __forceinline__ void tile_walk(double* tile, int tbuf, int ncol, int a0, int a1, ColF col, BodyF body) {
-  const int nt = a1 > a0 ? (a1 - a0 + LV_TR - 1) / LV_TR : 0;
-  if (nt > 0) stage_tile<T>(tile, ncol, a0, min(LV_TR, a1 - a0), col);
-  cp_async_commit();
-  for (int k = 0; k < nt; ++k) {
-    const int pn = a0 + (k + 1) * LV_TR;
-    if (k + 1 < nt) stage_tile<T>(tile + ((k + 1) & 1) * tbuf, ncol, pn, min(LV_TR, a1 - pn), col);
-    cp_async_commit();
-    cp_async_wait_prev();  // this thread's copies of tile k have landed
-    __syncthreads();       // ... and every thread's
-    body(tile + (k & 1) * tbuf, min(LV_TR, a1 - (a0 + k * LV_TR)));
-    __syncthreads();       // the buffer is free for tile k + 2
-  }
-}
 
 // Packed Gram matrix: Gp[q] = sum over rows [a0, a1) of X[a][p] X[b][p] for the
 // pair (a, b), a <= b < r, q = pair index (row-major upper triangle).  More
@@ -502,13 +372,12 @@ __device__ void proj_tiled(const T* __restrict__ Qb, T* const* Bp, int w, int64_
   __syncthreads();
 }
 
-// RB > 0: a rank bucket, nodes with RLO < r <= RB, small matrices with leading
-// dimension RB (less shared memory and registers, more CTAs per SM); RB == 0:
-// nodes with r > RLO, leading dimension cap.
-template <typename T, int RB, int RLO>
-__global__ void __launch_bounds__(256, RB == 4 ? 4 : (RB == 16 ? 3 : 2))
-    k_level(const FactDesc* __restrict__ Fd, int lvl, int G, double* __restrict__ gpart,
-            unsigned int* __restrict__ bar, int* __restrict__ abort_flag, int skip_le, size_t sstride) {
+// Nodes of rank above LW_RLO; small matrices with leading dimension cap.
+#define LW_RLO 16
+template <typename T>
+__global__ void __launch_bounds__(256, 2)
+    k_level_wide(const FactDesc* __restrict__ Fd, int lvl, int G, double* __restrict__ gpart,
+                 unsigned int* __restrict__ bar, int* __restrict__ abort_flag, size_t sstride) {
   extern __shared__ double sm[];
   // problem of a batched launch: its descriptor, and its scratch sstride bytes on
   Fd += blockIdx.y;
@@ -524,18 +393,14 @@ __global__ void __launch_bounds__(256, RB == 4 ? 4 : (RB == 16 ? 3 : 2))
   int s, h, e;
   node_range(bnd, lvl, bi, s, h, e);
   const int r = Fd->rank[nid];
-  if (r <= skip_le || r <= RLO || (RB > 0 && r > RB)) return;  // another launch takes this node
-  if (r == 0) {
-    if (g == 0 && threadIdx.x == 0) Fd->ld_parts[nleaf + nid] = 0.0;
-    return;
-  }
+  if (r <= LW_RLO) return;  // another launch takes this node
   int* status = Fd->status;
   T* Qall = (T*)Fd->Q;
   T* Qb = Qall + (size_t)lvl * cap * n;
   const int len = e - s, rc = (len + G - 1) / G;
   const int r0 = s + min(len, g * rc), r1 = s + min(len, g * rc + rc);
-  const int ldm = RB > 0 ? RB : cap;  // leading dimension of the small matrices
-  constexpr int W = LEVEL_W(RB);      // ancestor columns per update chunk
+  const int ldm = cap;      // leading dimension of the small matrices
+  constexpr int W = LEVEL_W;  // ancestor columns per update chunk
   const int cc2 = ldm * ldm;
   double* Gm = sm;                        // Gram / factor of the left side
   double* Gm2 = Gm + cc2;                 // ... of the right side
@@ -571,46 +436,23 @@ __global__ void __launch_bounds__(256, RB == 4 ? 4 : (RB == 16 ? 3 : 2))
       return;
     gram_unpack(Ri, r, Gm, ldm);
     gram_unpack(Ri + npk, r, Gm2, ldm);
-    if (r <= 8) {
-      // small ranks: each side's factorization by one thread (two warps side by side)
-      if (threadIdx.x == 0 || threadIdx.x == 32) {
-        const int sd = threadIdx.x >> 5;
-        double* Gs = sd ? Gm2 : Gm;
-        double* Rs = sd ? RV : RU;
-        double* rv = rvs + 8 * sd;
-        if (!thr_chol_upper(Gs, ldm, r, rv, clamp_gram<T>())) iflag[2] = 1;
-        thr_triinv_upper(Gs, ldm, rv, sd ? Ri2 : Ri, ldm, r);
-        for (int i = 0; i < r; ++i)
-          for (int j = 0; j < r; ++j) {
-            if (pass == 0) {
-              Rs[i * ldm + j] = Gs[i * ldm + j];
-            } else if (i <= j) {  // R = R2 R1 in place, rows top-down: row i reads rows >= i of R1
-              double v = 0.0;
-              for (int k = i; k <= j; ++k) v += Gs[i * ldm + k] * Rs[k * ldm + j];
-              Rs[i * ldm + j] = v;
-            }
+    for (int sd = 0; sd < 2; ++sd) {
+      double* Gs = sd ? Gm2 : Gm;
+      double* Rs = sd ? RV : RU;
+      ok = blk_chol_upper(Gs, ldm, r, iflag, clamp_gram<T>()) && ok;
+      blk_triinv_upper(Gs, ldm, sd ? Ri2 : Ri, ldm, r);
+      if (pass == 0) {
+        for (int t = threadIdx.x; t < cc2; t += blockDim.x) Rs[t] = Gs[t];
+      } else {
+        // R = R2 R1 in place, one thread per column, rows top-down
+        for (int j = threadIdx.x; j < r; j += blockDim.x)
+          for (int i = 0; i <= j; ++i) {
+            double v = 0.0;
+            for (int k = i; k <= j; ++k) v += Gs[i * ldm + k] * Rs[k * ldm + j];
+            Rs[i * ldm + j] = v;
           }
       }
       __syncthreads();
-    } else {
-      for (int sd = 0; sd < 2; ++sd) {
-        double* Gs = sd ? Gm2 : Gm;
-        double* Rs = sd ? RV : RU;
-        ok = blk_chol_upper(Gs, ldm, r, iflag, clamp_gram<T>()) && ok;
-        blk_triinv_upper(Gs, ldm, sd ? Ri2 : Ri, ldm, r);
-        if (pass == 0) {
-          for (int t = threadIdx.x; t < cc2; t += blockDim.x) Rs[t] = Gs[t];
-        } else {
-          // R = R2 R1 in place, one thread per column, rows top-down
-          for (int j = threadIdx.x; j < r; j += blockDim.x)
-            for (int i = 0; i <= j; ++i) {
-              double v = 0.0;
-              for (int k = i; k <= j; ++k) v += Gs[i * ldm + k] * Rs[k * ldm + j];
-              Rs[i * ldm + j] = v;
-            }
-        }
-        __syncthreads();
-      }
     }
     rowmul_pass<T>(Qb, n, r, sa0, sa1, Ri, ldm);
     rowmul_pass<T>(Qb, n, r, sb0, sb1, Ri2, ldm);
@@ -742,196 +584,8 @@ __global__ void __launch_bounds__(256, RB == 4 ? 4 : (RB == 16 ? 3 : 2))
 }
 
 // ---------------------------------------------------------------------------
-// Small-node level kernel.  One CTA per node with sides of at most MS rows and
-// rank in (RLO, R].  The node's basis rows and each chunk of ancestor columns
-// are staged in shared memory, and every reduction is computed by one thread
-// per output entry (a dot product over the node's rows): no cross-thread FP64
-// reductions, so FP64 instructions are spent on the products alone.
-// ---------------------------------------------------------------------------
-template <typename T, int R, int RLO, int MS, int W>
-__global__ void __launch_bounds__(128) k_level_small(const FactDesc* __restrict__ Fd, int lvl) {
-  Fd += blockIdx.y;  // problem of a batched launch
-  if (Fd->skip && *Fd->skip) return;
-  constexpr int R2 = 2 * R;
-  __shared__ double Xs[2][R][MS];   // side-major basis rows (FP64 during the QR)
-  __shared__ T Bs[W][2 * MS];       // ancestor-column chunk on the node's rows
-  __shared__ double Gm[R * R], Ri[R * R], R1[R * R], RU[R * R], RV[R * R];
-  __shared__ double S[R2 * R2], Si[R2 * R2];
-  __shared__ double Pm[R2 * W];
-  __shared__ T Tm[R2 * W];
-  __shared__ double red[40];
-  __shared__ int iflag[4];
-  __shared__ int rpre[FIFA_LEVELS_MAX + 1];  // prefix sums of the ancestor ranks
-  __shared__ int ccode[W];                    // (level << 8) | column of the chunk's columns
-  const int bi = blockIdx.x;
-  const int nid = node_id(lvl, bi);
-  const int r = Fd->rank[nid];
-  if (r > R || r <= RLO) return;  // another bucket's launch takes this node
-  const int cap = Fd->cap, nleaf = Fd->nleaf;
-  const int64_t n = Fd->n;
-  const int* bnd = Fd->bnd;
-  int s, h, e;
-  node_range(bnd, lvl, bi, s, h, e);
-  if (r == 0) {
-    if (threadIdx.x == 0) Fd->ld_parts[nleaf + nid] = 0.0;
-    return;
-  }
-  T* Qall = (T*)Fd->Q;
-  T* Qb = Qall + (size_t)lvl * cap * n;
-  int* status = Fd->status;
-  const int mu = h - s, mv = e - h;  // rows per side
-  for (int t = threadIdx.x; t < r * MS; t += blockDim.x) {
-    const int c = t / MS, p = t % MS;
-    Xs[0][c][p] = p < mu ? (double)Qb[(size_t)c * n + s + p] : 0.0;
-    Xs[1][c][p] = p < mv ? (double)Qb[(size_t)c * n + h + p] : 0.0;
-  }
-  __syncthreads();
-  bool ok = true;
-  const double cg = clamp_gram<T>();
-  for (int side = 0; side < 2; ++side) {
-    const int m = side ? mv : mu;
-    double(*X)[MS] = Xs[side];
-    for (int pass = 0; pass < 2; ++pass) {
-      // Gram matrix, one thread per entry a <= b
-      for (int t = threadIdx.x; t < r * r; t += blockDim.x) {
-        const int a = t / r, b = t % r;
-        if (a <= b) {
-          double acc = 0.0;
-          for (int p = 0; p < m; ++p) acc += X[a][p] * X[b][p];
-          Gm[a * R + b] = acc;
-          Gm[b * R + a] = acc;
-        }
-      }
-      __syncthreads();
-      ok = blk_chol_upper(Gm, R, r, iflag, cg) && ok;
-      if (pass == 0) {
-        for (int t = threadIdx.x; t < R * R; t += blockDim.x) R1[t] = Gm[t];
-      } else {
-        double* Rs = side ? RV : RU;
-        for (int t = threadIdx.x; t < R * R; t += blockDim.x) {
-          const int i = t / R, j = t % R;
-          double v = 0.0;
-          if (i < r && j < r && i <= j)
-            for (int k = i; k <= j; ++k) v += Gm[i * R + k] * R1[k * R + j];
-          Rs[t] = v;
-        }
-      }
-      __syncthreads();
-      blk_triinv_upper(Gm, R, Ri, R, r);
-      // X <- X Ri, one thread per row (the row is read before it is overwritten)
-      for (int p = threadIdx.x; p < m; p += blockDim.x) {
-        double xr[R];
-#pragma unroll
-        for (int c = 0; c < R; ++c) xr[c] = c < r ? X[c][p] : 0.0;
-#pragma unroll
-        for (int c = 0; c < R; ++c) {
-          if (c < r) {
-            double v = 0.0;
-#pragma unroll
-            for (int a = 0; a <= c; ++a) v += xr[a] * Ri[a * R + c];
-            X[c][p] = (double)(T)v;  // the stored basis is rounded to T
-          }
-        }
-      }
-      __syncthreads();
-    }
-  }
-  for (int t = threadIdx.x; t < r * MS; t += blockDim.x) {
-    const int c = t / MS, p = t % MS;
-    if (p < mu) Qb[(size_t)c * n + s + p] = (T)Xs[0][c][p];
-    if (p < mv) Qb[(size_t)c * n + h + p] = (T)Xs[1][c][p];
-  }
-  // capacitance: S = I + R X R^T, L_S = chol(S) = R_S^T
-  const int r2 = 2 * r;
-  for (int t = threadIdx.x; t < r2 * r2; t += blockDim.x) {
-    const int a = t / r2, b = t % r2;
-    double v = (a == b) ? 1.0 : 0.0;
-    if (a < r && b >= r) {
-      for (int k = 0; k < r; ++k) v += RU[a * R + k] * RV[(b - r) * R + k];
-    } else if (a >= r && b < r) {
-      for (int k = 0; k < r; ++k) v += RV[(a - r) * R + k] * RU[b * R + k];
-    }
-    S[a * R2 + b] = v;
-  }
-  __syncthreads();
-  ok = blk_chol_upper(S, R2, r2, iflag, clamp_cap<T>()) && ok;
-  double ls = 0.0;
-  for (int k = threadIdx.x; k < r2; k += blockDim.x) ls += log(S[k * R2 + k]);
-  ls = block_sum(ls, red);
-  blk_triinv_upper(S, R2, Si, R2, r2);
-  const int ld2 = 2 * cap;
-  double* Zf = Fd->Zf + (size_t)nid * ld2 * ld2;
-  double* Zi = Fd->Zi + (size_t)nid * ld2 * ld2;
-  for (int t = threadIdx.x; t < r2 * r2; t += blockDim.x) {
-    const int a = t / r2, b = t % r2;
-    const double d = (a == b) ? 1.0 : 0.0;
-    Zf[a * ld2 + b] = (a >= b ? S[b * R2 + a] : 0.0) - d;
-    Zi[a * ld2 + b] = (a >= b ? Si[b * R2 + a] : 0.0) - d;
-  }
-  if (threadIdx.x == 0) {
-    Fd->ld_parts[nleaf + nid] = ls;
-    if (!ok) atomicOr(status, FIFA_DEV_NOT_SPD);
-  }
-  if (lvl == 0) return;
-  // ancestor bases on the node's rows: B <- B + Q (L_S^-1 - I) Q^T B
-  if (threadIdx.x == 0) {
-    int c = 0;
-    for (int j = 0; j < lvl; ++j) {
-      rpre[j] = c;
-      c += Fd->rank[node_id(j, bi >> (lvl - j))];
-    }
-    rpre[lvl] = c;
-  }
-  __syncthreads();
-  const int na = rpre[lvl], mn = e - s;
-  for (int c0 = 0; c0 < na; c0 += W) {
-    const int w = min(W, na - c0);
-    if (threadIdx.x < w) {  // ancestor column c0 + t: level j with rpre[j] <= c < rpre[j + 1]
-      const int c = c0 + threadIdx.x;
-      int j = 0;
-      while (rpre[j + 1] <= c) ++j;
-      ccode[threadIdx.x] = (j << 8) | (c - rpre[j]);
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < w * mn; t += blockDim.x) {
-      const int j = t / mn, p = t % mn;
-      const int code = ccode[j];
-      Bs[j][p] = Qall[((size_t)(code >> 8) * cap + (code & 255)) * n + s + p];
-    }
-    __syncthreads();
-    // P[a][j] = Q^T B: rows a < r from the left child, r <= a < 2r from the right
-    for (int t = threadIdx.x; t < r2 * w; t += blockDim.x) {
-      const int a = t / w, j = t % w;
-      const int side = a >= r, c = side ? a - r : a, m = side ? mv : mu, off = side ? mu : 0;
-      T acc = (T)0;
-      for (int p = 0; p < m; ++p) acc += (T)Xs[side][c][p] * Bs[j][off + p];
-      Pm[a * W + j] = (double)acc;
-    }
-    __syncthreads();
-    // T = (L_S^-1 - I) P
-    for (int t = threadIdx.x; t < r2 * w; t += blockDim.x) {
-      const int a = t / w, j = t % w;
-      double v = -Pm[a * W + j];
-      for (int b = 0; b <= a; ++b) v += Si[b * R2 + a] * Pm[b * W + j];
-      Tm[a * W + j] = (T)v;
-    }
-    __syncthreads();
-    // B += Q T, one thread per (row, column)
-    for (int t = threadIdx.x; t < w * mn; t += blockDim.x) {
-      const int j = t / mn, p = t % mn;
-      const int side = p >= mu, pp = side ? p - mu : p, toff = side ? r : 0;
-      T acc = Bs[j][p];
-      for (int a = 0; a < r; ++a) acc += (T)Xs[side][a][pp] * Tm[(toff + a) * W + j];
-      const int code = ccode[j];
-      Qall[((size_t)(code >> 8) * cap + (code & 255)) * n + s + p] = acc;
-    }
-    __syncthreads();
-  }
-}
-
-// ---------------------------------------------------------------------------
 // Multi-node small-level kernel: NPC nodes of one level per CTA (sides of at
-// most MS rows, rank <= R), the same arithmetic as k_level_small.  Every step
+// most MS rows, rank <= R), the algebra of k_level.  Every step
 // is spread over the nodes: the per-node dense algebra (Cholesky, triangular
 // inverse, capacitance) runs one thread per node and side, and the row and
 // column work runs over all the CTA's nodes at once, so few lanes idle while
@@ -949,11 +603,11 @@ struct LmLayout {
   static constexpr size_t xs = (size_t)NPC * 2 * R * MS;  // doubles
   static constexpr size_t mats = (size_t)NPC * 2 * R * R;  // Gm / Ri / R1 / rinv (doubles each)
   static constexpr size_t ruv = (size_t)NPC * R * R;       // RU / RV
-  static constexpr size_t sm = (size_t)NPC * R2 * R2;      // S / Si
-  static constexpr size_t pm = (size_t)NPC * R2 * LM_W;    // Pm / Tm
-  static constexpr size_t doubles = xs + 3 * mats + (size_t)NPC * 2 * R + 2 * ruv + 2 * sm + pm;
+  static constexpr size_t pm = (size_t)NPC * R2 * LM_W;    // Pm (Tm half of it)
+  // R_U, R_V, M, I - M^T M, L2^-T, K
+  static constexpr size_t doubles = xs + 3 * mats + (size_t)NPC * 2 * R + 6 * ruv + pm;
   static size_t bytes(int elt) {
-    return doubles * sizeof(double) + (size_t)LmDB<NPC>::nbuf * NPC * LM_W * 2 * MS * elt + pm * elt +
+    return doubles * sizeof(double) + (size_t)LmDB<NPC>::nbuf * NPC * LM_W * 2 * MS * elt + pm / 2 * elt +
            (size_t)NPC * (FIFA_LEVELS_MAX + 1 + LmDB<NPC>::nbuf * LM_W + 8) * sizeof(int) + 64;
   }
 };
@@ -972,13 +626,15 @@ __global__ void __launch_bounds__(256) k_level_multi(const FactDesc* __restrict_
   double* rv = R1 + LY::mats;             // [j][side][R] reciprocal pivots
   double* RU = rv + NPC * 2 * R;          // [j][R*R]
   double* RV = RU + LY::ruv;
-  double* S = RV + LY::ruv;               // [j][R2*R2]
-  double* Si = S + LY::sm;
-  double* Pm = Si + LY::sm;               // [j][R2][LM_W]
+  double* Mm = RV + LY::ruv;              // [j][R*R]
+  double* S = Mm + LY::ruv;
+  double* Si = S + LY::ruv;
+  double* Kk = Si + LY::ruv;
+  double* Pm = Kk + LY::ruv;              // [j][R2][LM_W]
   constexpr int NB = LmDB<NPC>::nbuf;
   T* Bs2 = (T*)(Pm + LY::pm);             // NB buffers of [j][LM_W][2 MS]
-  T* Tm = Bs2 + NB * (size_t)NPC * LM_W * 2 * MS;  // [j][R2][LM_W]
-  int* ib = (int*)(Tm + LY::pm);
+  T* Tm = Bs2 + NB * (size_t)NPC * LM_W * 2 * MS;  // [j][R][LM_W]
+  int* ib = (int*)(Tm + LY::pm / 2);
   int* rpre = ib;                          // [j][LEVELS_MAX + 1]
   int* ccode2 = rpre + NPC * (FIFA_LEVELS_MAX + 1);  // NB buffers of [j][LM_W]
   int* info = ccode2 + NB * NPC * LM_W;    // [j][8]: r, s, h, e, active, ok
@@ -1101,7 +757,9 @@ __global__ void __launch_bounds__(256) k_level_multi(const FactDesc* __restrict_
     const int a0 = side ? in[2] : in[1], m = side ? in[3] - in[2] : in[2] - in[1];
     if (p < m) Qb[(size_t)c * n + a0 + p] = (T)Xs[t];
   }
-  // capacitance S = I + R X R^T, L_S = chol(S) = R_S^T, one thread per node
+  // capacitance S = I + R X R^T = [I M; M^T I], M = R_U R_V^T: L_S = [I 0; M^T L2]
+  // with L2 = chol(I - M^T M), L_S^-1 = [I 0; K L2^-1], K = -L2^-1 M^T; one thread
+  // per node
   if (tid < NPC) {
     const int j = tid;
     int* in = info + j * 8;
@@ -1109,39 +767,59 @@ __global__ void __launch_bounds__(256) k_level_multi(const FactDesc* __restrict_
       const int r = in[0], r2 = 2 * r;
       const double* ru = RU + j * R * R;
       const double* rvv = RV + j * R * R;
-      double* Sj = S + j * R2 * R2;
-      for (int a = 0; a < r2; ++a)
-        for (int b = 0; b < r2; ++b) {
-          double v = (a == b) ? 1.0 : 0.0;
-          if (a < r && b >= r) {
-            for (int k = 0; k < r; ++k) v += ru[a * R + k] * rvv[(b - r) * R + k];
-          } else if (a >= r && b < r) {
-            for (int k = 0; k < r; ++k) v += rvv[(a - r) * R + k] * ru[b * R + k];
-          }
-          Sj[a * R2 + b] = v;
+      double* Mj = Mm + j * R * R;
+      double* Nj = S + j * R * R;
+      double* Lij = Si + j * R * R;
+      double* Kj = Kk + j * R * R;
+      for (int a = 0; a < r; ++a)
+        for (int b = 0; b < r; ++b) {
+          double v = 0.0;
+          for (int k = max(a, b); k < r; ++k) v += ru[a * R + k] * rvv[b * R + k];
+          Mj[a * R + b] = v;
         }
-      double srv[R2];
-      if (!thr_chol_upper(Sj, R2, r2, srv, clamp_cap<T>())) in[5] = 0;
+      for (int a = 0; a < r; ++a)
+        for (int b = a; b < r; ++b) {
+          double v = (a == b) ? 1.0 : 0.0;
+          for (int k = 0; k < r; ++k) v -= Mj[k * R + a] * Mj[k * R + b];
+          Nj[a * R + b] = v;
+        }
+      double srv[R];
+      if (!thr_chol_upper(Nj, R, r, srv, clamp_cap<T>())) in[5] = 0;
       // log det L_S from one logarithm of the pivots' product (a serial chain
-      // of r2 logarithms here costs more than the rest of the node's algebra);
+      // of logarithms here costs more than the rest of the node's algebra);
       // a product out of range falls back to the sum of logarithms
       double prod = 1.0;
-      for (int k = 0; k < r2; ++k) prod *= Sj[k * R2 + k];
+      for (int k = 0; k < r; ++k) prod *= Nj[k * R + k];
       double ls = 0.0;
       if (prod > 0.0 && prod < INFINITY && prod > 1e-300) {
         ls = log(prod);
       } else {
-        for (int k = 0; k < r2; ++k) ls += log(Sj[k * R2 + k]);
+        for (int k = 0; k < r; ++k) ls += log(Nj[k * R + k]);
       }
-      thr_triinv_upper(Sj, R2, srv, Si + j * R2 * R2, R2, r2);
+      thr_triinv_upper(Nj, R, srv, Lij, R, r);  // (L2^-1)^T
+      for (int a = 0; a < r; ++a)
+        for (int c = 0; c < r; ++c) {
+          double v = 0.0;
+          for (int b = 0; b <= a; ++b) v -= Lij[b * R + a] * Mj[c * R + b];
+          Kj[a * R + c] = v;
+        }
       const int nid = node_id(lvl, b0 + j), ld2 = 2 * cap;
       double* Zf = Fd->Zf + (size_t)nid * ld2 * ld2;
       double* Zi = Fd->Zi + (size_t)nid * ld2 * ld2;
       for (int a = 0; a < r2; ++a)
         for (int b = 0; b < r2; ++b) {
-          const double d = (a == b) ? 1.0 : 0.0;
-          Zf[a * ld2 + b] = (a >= b ? Sj[b * R2 + a] : 0.0) - d;
-          Zi[a * ld2 + b] = (a >= b ? Si[j * R2 * R2 + b * R2 + a] : 0.0) - d;
+          const int ra = a - r, rb = b - r;
+          double zf = 0.0, zi = 0.0;
+          if (ra >= 0 && rb < 0) {
+            zf = Mj[b * R + ra];
+            zi = Kj[ra * R + b];
+          } else if (ra >= 0 && rb <= ra) {
+            const double d = (ra == rb) ? 1.0 : 0.0;
+            zf = Nj[rb * R + ra] - d;
+            zi = Lij[rb * R + ra] - d;
+          }
+          Zf[a * ld2 + b] = zf;
+          Zi[a * ld2 + b] = zi;
         }
       Fd->ld_parts[nleaf + nid] = ls;
       if (!in[5]) atomicOr(Fd->status, FIFA_DEV_NOT_SPD);
@@ -1234,35 +912,38 @@ __global__ void __launch_bounds__(256) k_level_multi(const FactDesc* __restrict_
       Pm[t] = (double)acc;
     }
     __syncthreads();
-    // T = (L_S^-1 - I) P, in the node's compact 2r layout
-    for (int t = tid; t < NPC * R2 * LM_W; t += nt) {
-      const int j = t / (R2 * LM_W), a = (t / LM_W) % R2, w = t % LM_W;
+    // T = (L_S^-1 - I) P: zero on the left side, K P_left + (L2^-1 - I) P_right
+    // on the right
+    for (int t = tid; t < NPC * R * LM_W; t += nt) {
+      const int j = t / (R * LM_W), a = (t / LM_W) % R, w = t % LM_W;
       const int* in = info + j * 8;
       const int r = in[0];
       double v = 0.0;
-      if (in[4] && a < 2 * r) {
-        // a is the compact index of the 2r x 2r factor (a < r: left child, else right)
-        const double* Sij = Si + j * R2 * R2;
+      if (in[4] && a < r) {
+        const double* Lij = Si + j * R * R;
+        const double* Kj = Kk + j * R * R;
         const double* P = Pm + (size_t)j * R2 * LM_W;
-        v = -P[a * LM_W + w];
-        for (int b = 0; b <= a; ++b) v += Sij[b * R2 + a] * P[b * LM_W + w];
+        v = -P[(r + a) * LM_W + w];
+        for (int b = 0; b < r; ++b) v += Kj[a * R + b] * P[b * LM_W + w];
+        for (int b = 0; b <= a; ++b) v += Lij[b * R + a] * P[(r + b) * LM_W + w];
       }
       Tm[t] = (T)v;
     }
     __syncthreads();
-    // B += Q T, one thread per (node, column, row), written back
-    for (int t = tid; t < NPC * LM_W * 2 * MS; t += nt) {
-      const int j = t / (LM_W * 2 * MS), w = (t / (2 * MS)) % LM_W, p = t % (2 * MS);
+    // B += Q T on the right side's rows (the left side's keep their values),
+    // one thread per (node, column, row), written back
+    for (int t = tid; t < NPC * LM_W * MS; t += nt) {
+      const int j = t / (LM_W * MS), w = (t / MS) % LM_W, pp = t % MS;
       const int code = ccode[j * LM_W + w];
       const int* in = info + j * 8;
-      const int mu = in[2] - in[1], mn = in[3] - in[1];
-      if (code < 0 || p >= mn) continue;
-      const int r = in[0], side = p >= mu, pp = side ? p - mu : p, toff = side ? r : 0;
-      const double* X = Xs + (size_t)(j * 2 + side) * R * MS;
-      const T* Tj = Tm + (size_t)j * R2 * LM_W;
-      T acc = Bs[t];
-      for (int a = 0; a < r; ++a) acc += (T)X[a * MS + pp] * Tj[(toff + a) * LM_W + w];
-      Qall[((size_t)(code >> 8) * cap + (code & 255)) * n + in[1] + p] = acc;
+      const int mu = in[2] - in[1], mv = in[3] - in[2];
+      if (code < 0 || pp >= mv) continue;
+      const int r = in[0];
+      const double* X = Xs + (size_t)(j * 2 + 1) * R * MS;
+      const T* Tj = Tm + (size_t)j * R * LM_W;
+      T acc = Bs[((size_t)j * LM_W + w) * 2 * MS + mu + pp];
+      for (int a = 0; a < r; ++a) acc += (T)X[a * MS + pp] * Tj[a * LM_W + w];
+      Qall[((size_t)(code >> 8) * cap + (code & 255)) * n + in[2] + pp] = acc;
     }
     __syncthreads();
   }
@@ -1301,8 +982,8 @@ size_t leaf_factor_smem(int Bm, int L, int cap, int prec) {
   b += 16 + 40 * sizeof(double) + (4 + (size_t)L * cap) * sizeof(int);
   return b;
 }
-size_t level_smem(int ldm, int cap) {
-  const size_t W = LEVEL_W(ldm);
+static size_t level_wide_smem(int cap) {
+  const size_t W = LEVEL_W, ldm = cap;
   return ((size_t)6 * ldm * ldm + 16 + 2 * (size_t)(ldm + W) * LV_TRP + 256 + LV_RED + 4 * (size_t)ldm * W) * sizeof(double) +
          W * sizeof(void*) + (4 + (size_t)FIFA_LEVELS_MAX * cap) * sizeof(int);
 }
@@ -1340,84 +1021,89 @@ cudaError_t launch_leaf_factor(const HmatDesc* Hd, const FactDesc* Fd, int prec,
   return launch_leaf_factor_t<double>(Hd, Fd, nleaf, smem, st, nprob);
 }
 
-template <typename T, int RB, int RLO>
-static cudaError_t launch_level_bucket(const FactDesc* Fd, int lvl, int nodes, int G, int cap, double* part,
-                                       unsigned int* bar, int* abort_flag, int skip, cudaStream_t st, int nprob,
-                                       size_t sstride) {
-  const size_t smem = level_smem(RB > 0 ? RB : cap, cap);
+static cudaError_t launch_level_wide(const FactDesc* Fd, int lvl, int nodes, int G, int cap, double* part,
+                                     unsigned int* bar, int* abort_flag, bool cluster, cudaStream_t st, int nprob,
+                                     size_t sstride) {
+  if (cluster)  // a cluster of a power of two CTAs: scheduled together, so the group may wait
+    for (int c = 8; c >= 1; c /= 2)
+      if (c <= G) {
+        G = c;
+        break;
+      }
+  const size_t smem = level_wide_smem(cap);
   if (smem > (size_t)smem_optin()) return cudaErrorInvalidConfiguration;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_level<T, RB, RLO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  cudaError_t e = cudaFuncSetAttribute(k_level_wide<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(nodes * G, nprob);
   cfg.blockDim = dim3(256);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = G > 1 ? 1 : 0;
+  if (cluster) {
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = G;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+  } else {
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = G > 1 ? 1 : 0;
+  }
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_level<T, RB, RLO>, Fd, lvl, G, part, bar, abort_flag, skip, sstride);
+  return cudaLaunchKernelEx(&cfg, k_level_wide<double>, Fd, lvl, G, part, bar, abort_flag, sstride);
 }
 
-template <typename T>
-static cudaError_t launch_level_t(const FactDesc* Fd, int lvl, int nodes, const int* G, int cap, double* part,
-                                  unsigned int* bar, int bar_stride, int* abort_flag, int side_max, cudaStream_t st,
-                                  int nprob, size_t sstride) {
-  int skip = -1;
-  if (G[0] == 1 && side_max <= 128) {  // (nodes this small are never split over CTAs)
-    // small nodes: rank <= 4 several nodes per CTA, rank 5..8 one node per CTA
-    // (static shared memory); larger nodes take the tiled bucket kernels below,
-    // whose output-major Gram and projection passes use the lanes better
-    cudaError_t e0 = side_max <= 32   ? launch_level_multi<T, 4, 32, 4>(Fd, lvl, nodes, st, nprob)
-                     : side_max <= 64 ? launch_level_multi<T, 4, 64, 2>(Fd, lvl, nodes, st, nprob)
-                                      : launch_level_multi<T, 4, 128, 1>(Fd, lvl, nodes, st, nprob);
-    if (e0 != cudaSuccess) return e0;
-    k_level_small<T, 8, 4, 128, 8><<<dim3(nodes, nprob), 128, 0, st>>>(Fd, lvl);
-    skip = 8;
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  // rank buckets: (.., 4] and (4, 16] with small-matrix storage sized by the
-  // bucket, then (16, cap]; a node's CTAs skip the launches of other buckets
-  // (buckets entirely below the small kernels' ranks are not launched)
-  cudaError_t e = cudaSuccess;
-  if ((G[0] > 1 || G[1] > 1) && nodes <= 64) {
-    // a top level with CTA groups has few nodes, often of both rank buckets:
-    // one launch for every rank <= 16 instead of two launches that would each
-    // leave the other bucket's groups idle (measured: the split is faster only
-    // at levels of >= 128 nodes, which are mostly of one bucket)
-    e = launch_level_bucket<T, 16, -1>(Fd, lvl, nodes, G[1], cap, part, bar + bar_stride, abort_flag, skip, st, nprob, sstride);
-    if (e == cudaSuccess && cap > 16)
-      e = launch_level_bucket<T, 0, 16>(Fd, lvl, nodes, G[2], cap, part, bar + 2 * bar_stride, abort_flag, skip, st, nprob, sstride);
-    return e;
-  }
-  if (skip < 4) e = launch_level_bucket<T, 4, -1>(Fd, lvl, nodes, G[0], cap, part, bar, abort_flag, skip, st, nprob, sstride);
-  if (e == cudaSuccess && cap > 4 && skip < 16)
-    e = launch_level_bucket<T, 16, 4>(Fd, lvl, nodes, G[1], cap, part, bar + bar_stride, abort_flag, skip, st, nprob, sstride);
-  if (e == cudaSuccess && cap > 16)
-    e = launch_level_bucket<T, 0, 16>(Fd, lvl, nodes, G[2], cap, part, bar + 2 * bar_stride, abort_flag, skip, st, nprob, sstride);
-  return e;
+// CTAs of a cluster for a node of `rows` rows when a launch has `nodes` nodes:
+// up to eight while they fill at most two CTAs per SM of 152 and keep 12 rows
+// each.
+static int level_cluster(int64_t nodes, int64_t rows) {
+  int c = 1;
+  while (c < 8 && 2 * c * nodes <= 304 && rows / (2 * c) >= 12) c *= 2;
+  return c;
 }
 
+// Ranks <= 16: nodes of at most LEVEL_CLUSTER_ROWS rows by a cluster each (its
+// CTAs are scheduled together by the hardware, so no cooperative launch and no
+// waiting on other launches), larger ones by groups of G CTAs.  Ranks above 16:
+// groups of G[2] CTAs, a cluster of them for the small nodes.
 cudaError_t launch_level(const FactDesc* Fd, int prec, int lvl, int nodes, const int* G, int cap, double* part,
                          unsigned int* bar, int bar_stride, int* abort_flag, int side_max, cudaStream_t st, int nprob,
                          size_t sstride) {
   if (prec != 0) return cudaErrorInvalidValue;
-  return launch_level_t<double>(Fd, lvl, nodes, G, cap, part, bar, bar_stride, abort_flag, side_max, st, nprob,
-                                sstride);
+  cudaError_t e = cudaSuccess;
+  const bool cluster = level_clustered(side_max);
+  int skip = -1;
+  if (side_max <= 128) {
+    // small nodes of rank <= 4: several nodes per CTA
+    e = side_max <= 32   ? launch_level_multi<double, 4, 32, 4>(Fd, lvl, nodes, st, nprob)
+        : side_max <= 64 ? launch_level_multi<double, 4, 64, 2>(Fd, lvl, nodes, st, nprob)
+                         : launch_level_multi<double, 4, 128, 1>(Fd, lvl, nodes, st, nprob);
+    skip = 4;
+  }
+  const int cl = level_cluster((int64_t)nodes * nprob, 2 * (int64_t)side_max);
+  const int Gn[2] = {cluster ? cl : G[0], cluster ? cl : G[1]};
+  // a level of few nodes often has ranks of both buckets: one launch for every
+  // rank <= 16 instead of two that would each leave the other's CTAs idle
+  // (measured for groups: the split is faster only at levels of >= 128 nodes,
+  // which are mostly of one bucket)
+  const bool merged = (Gn[0] > 1 || Gn[1] > 1) && nodes <= 64 && skip < 0;
+  if (e == cudaSuccess && !merged && skip < 4)
+    e = launch_node(Fd, 4, -1, cluster, lvl, nodes, Gn[0], part, bar, abort_flag, skip, st, nprob, sstride);
+  if (e == cudaSuccess && (merged || cap > 4))
+    e = launch_node(Fd, 16, merged ? -1 : 4, cluster, lvl, nodes, Gn[1], part, bar + bar_stride, abort_flag, skip, st,
+                    nprob, sstride);
+  if (e == cudaSuccess && cap > LW_RLO)
+    e = launch_level_wide(Fd, lvl, nodes, G[2], cap, part, bar + 2 * bar_stride, abort_flag, cluster, st, nprob, sstride);
+  return e;
 }
 
-template <typename T, int RB, int RLO>
-static int level_bucket_per_sm(int cap) {
-  const size_t smem = level_smem(RB > 0 ? RB : cap, cap);
+static int level_wide_per_sm(int cap) {
+  const size_t smem = level_wide_smem(cap);
   if (smem > (size_t)smem_optin()) return 0;
-  if (smem > 48 * 1024) cudaFuncSetAttribute(k_level<T, RB, RLO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaFuncSetAttribute(k_level_wide<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_level<T, RB, RLO>, 256, smem) != cudaSuccess) per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_level_wide<double>, 256, smem) != cudaSuccess) per_sm = 0;
   cudaGetLastError();
   return per_sm;
 }
@@ -1427,12 +1113,7 @@ int level_bucket_coresident(int prec, int b, int cap) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   (void)prec;  // factorizations run in FP64 only
-  int per_sm = 0;
-  if (b == 0) per_sm = level_bucket_per_sm<double, 4, -1>(cap);
-  else if (b == 1)  // also launched as <16, -1> at levels with CTA groups
-    per_sm = std::min(level_bucket_per_sm<double, 16, 4>(cap), level_bucket_per_sm<double, 16, -1>(cap));
-  else per_sm = level_bucket_per_sm<double, 0, 16>(cap);
-  return sms * per_sm;
+  return sms * (b == 2 ? level_wide_per_sm(cap) : node_ctas_per_sm(b == 0 ? 4 : 16));
 }
 
 cudaError_t launch_logdet_reduce(const FactDesc* Fd, cudaStream_t st, int nprob) {
