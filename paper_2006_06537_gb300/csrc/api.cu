@@ -579,9 +579,16 @@ fifa_status hmat_assemble_grouped_enqueue(fifa_ctx* ctx, fifa_hmat* H) {
   if (P->aca_ncoop > 0) {
     CK(cudaMemsetAsync(S.aca_bar, 0, sizeof(unsigned int) * P->aca_ncoop, s));
     CK(cudaMemsetAsync(S.flags, 0, sizeof(int), s));
-    CK(launch_aca(H->dev, P->aca_work, P->aca_ncoop, true, S.aca_part, S.aca_bar, S.flags, s));
+    CK(launch_aca(H->dev, P->aca_work, P->aca_ncoop, S.aca_part, S.aca_bar, S.flags, s));
   }
   return FIFA_OK;
+}
+
+// Rows and columns of the largest block without a group of its own.
+static int aca_solo_span(const Plan* P) {
+  if (P->aca_nsolo == 0) return 0;
+  const int4 w = P->work_host[P->aca_ncoop];
+  return P->bnd_host[bnd_off(w.x) + w.y + 1] - P->bnd_host[bnd_off(w.x) + w.y];
 }
 
 // Second part (after the first in stream order): dense leaves, one-CTA and
@@ -593,7 +600,7 @@ fifa_status hmat_assemble_rest_enqueue(fifa_ctx* ctx, fifa_hmat* H) {
   Scratch S = carve(ctx, P);
   cudaStream_t s = ctx->stream;
   CK(launch_leaf_assemble(H->dev, P->nleaf, s));
-  if (P->aca_nsolo > 0) CK(launch_aca(H->dev, P->aca_work + P->aca_ncoop, P->aca_nsolo, false, S.aca_part, S.aca_bar, S.flags, s));
+  CK(launch_aca_solo(H->dev, P->aca_work + P->aca_ncoop, P->aca_nsolo, aca_solo_span(P), s));
   if (P->aca_nwarp > 0) CK(launch_aca_warp(H->dev, P->aca_work + P->aca_ncoop + P->aca_nsolo, P->aca_nwarp, s));
   return FIFA_OK;
 }
@@ -610,7 +617,7 @@ fifa_status hmat_assemble_batched(fifa_ctx* ctx, Plan* P, HmatDesc* H0, int npro
     if ((int64_t)P->aca_ncoop * nprob <= ctx->aca_coresident) {  // every problem's groups co-resident at once
       CK(cudaMemset2DAsync(S.aca_bar, sstride, 0, sizeof(unsigned int) * P->aca_ncoop, nprob, s));
       CK(cudaMemset2DAsync(S.flags, sstride, 0, sizeof(int), nprob, s));
-      CK(launch_aca(H0, P->aca_work, P->aca_ncoop, true, S.aca_part, S.aca_bar, S.flags, s, nprob, sstride));
+      CK(launch_aca(H0, P->aca_work, P->aca_ncoop, S.aca_part, S.aca_bar, S.flags, s, nprob, sstride));
     } else {
       for (int q = 0; q < nprob; ++q) {  // one grouped launch per problem, each filling the GPU
         const size_t off = (size_t)q * sstride;
@@ -618,13 +625,11 @@ fifa_status hmat_assemble_batched(fifa_ctx* ctx, Plan* P, HmatDesc* H0, int npro
         int* flags = (int*)((char*)S.flags + off);
         CK(cudaMemsetAsync(bar, 0, sizeof(unsigned int) * P->aca_ncoop, s));
         CK(cudaMemsetAsync(flags, 0, sizeof(int), s));
-        CK(launch_aca(H0 + q, P->aca_work, P->aca_ncoop, true, (ArgMax*)((char*)S.aca_part + off), bar, flags, s));
+        CK(launch_aca(H0 + q, P->aca_work, P->aca_ncoop, (ArgMax*)((char*)S.aca_part + off), bar, flags, s));
       }
     }
   }
-  if (P->aca_nsolo > 0)
-    CK(launch_aca(H0, P->aca_work + P->aca_ncoop, P->aca_nsolo, false, S.aca_part, S.aca_bar, S.flags, s, nprob,
-                  sstride));
+  CK(launch_aca_solo(H0, P->aca_work + P->aca_ncoop, P->aca_nsolo, aca_solo_span(P), s, nprob));
   if (P->aca_nwarp > 0) CK(launch_aca_warp(H0, P->aca_work + P->aca_ncoop + P->aca_nsolo, P->aca_nwarp, s, nprob));
   return FIFA_OK;
 }

@@ -189,50 +189,6 @@ __device__ __forceinline__ ArgMax am_better(ArgMax a, ArgMax b) { return am_wins
 __device__ __forceinline__ double nn_max(double a, double b) {
   return __double_as_longlong(b) > __double_as_longlong(a) ? b : a;
 }
-__device__ __forceinline__ ArgMax warp_argmax(ArgMax a) {
-  for (int o = 16; o > 0; o >>= 1) {
-    ArgMax b;
-    b.v = __shfl_down_sync(0xffffffffu, a.v, o);
-    b.i = __shfl_down_sync(0xffffffffu, a.i, o);
-    b.sv = __shfl_down_sync(0xffffffffu, a.sv, o);
-    a = am_better(a, b);
-  }
-  return a;
-}
-// Block argmax; result valid in every thread. `sh` >= 33 ArgMax slots.
-__device__ inline ArgMax block_argmax(ArgMax a, ArgMax* sh) {
-  int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  a = warp_argmax(a);
-  __syncthreads();
-  if (lane == 0) sh[w] = a;
-  __syncthreads();
-  if (w == 0) {
-    ArgMax t = lane < nw ? sh[lane] : ArgMax{-1.0, 0x7fffffff, 0.0};
-    t = warp_argmax(t);
-    if (lane == 0) sh[32] = t;
-  }
-  __syncthreads();
-  ArgMax r = sh[32];
-  __syncthreads();
-  return r;
-}
-// Block max of values >= 0 (or -1); result valid in every thread.
-__device__ __forceinline__ double block_max(double v, double* sh) {
-  int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int o = 16; o > 0; o >>= 1) v = nn_max(v, __shfl_down_sync(0xffffffffu, v, o));
-  __syncthreads();
-  if (lane == 0) sh[w] = v;
-  __syncthreads();
-  if (w == 0) {
-    double t = lane < nw ? sh[lane] : -1.0;
-    for (int o = 16; o > 0; o >>= 1) t = nn_max(t, __shfl_down_sync(0xffffffffu, t, o));
-    if (lane == 0) sh[32] = t;
-  }
-  __syncthreads();
-  double r = sh[32];
-  __syncthreads();
-  return r;
-}
 
 // ---------------------------------------------------------------------------
 // Small dense routines run by a whole block on row-major matrices with

@@ -10,8 +10,11 @@
 cudaError_t launch_leaf_assemble(const HmatDesc* Hd, int nleaf, cudaStream_t st, int nprob = 1);
 #define ACA_WARP_MAX 128  // largest side of a block that the warp-per-block ACA takes
 cudaError_t launch_aca_warp(const HmatDesc* Hd, const int4* work, int nwork, cudaStream_t st, int nprob = 1);
-cudaError_t launch_aca(const HmatDesc* Hd, const int4* work, int ncta, bool cooperative, ArgMax* part,
-                       unsigned int* bar, int* abort_flag, cudaStream_t st, int nprob = 1, size_t pstride = 0);
+// ncta CTAs of the grouped blocks' work list (a cooperative launch: they wait on each other)
+cudaError_t launch_aca(const HmatDesc* Hd, const int4* work, int ncta, ArgMax* part, unsigned int* bar, int* abort_flag,
+                       cudaStream_t st, int nprob = 1, size_t pstride = 0);
+// one CTA or cluster per block; span: rows and columns of the largest block
+cudaError_t launch_aca_solo(const HmatDesc* Hd, const int4* work, int nblocks, int span, cudaStream_t st, int nprob = 1);
 int aca_max_coresident_ctas();
 
 size_t leaf_factor_smem(int Bm, int L, int cap, int prec);

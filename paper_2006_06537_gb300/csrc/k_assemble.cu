@@ -69,14 +69,72 @@ __global__ void __launch_bounds__(256) k_leaf_assemble(const HmatDesc* __restric
 }
 
 // ---------------------------------------------------------------------------
-// ACA.  work[cta] = {level, node, g, G}: the G CTAs of one group split the
-// block's rows and columns; every CTA of the group takes identical pivot
-// decisions from the same reduced data, so only partial maxima are exchanged.
+// ACA.  The G CTAs of one block split its rows and columns; every CTA takes
+// identical pivot decisions from the same reduced data, so only maxima are
+// exchanged and the bases do not depend on G.  CL: the CTAs are a thread-block
+// cluster of C CTAs on work[blockIdx.x / C] = {level, node, ..} and exchange
+// through distributed shared memory; else work[blockIdx.x] = {level, node, g, G}
+// and a group of G > 1 meets at bounded-spin barriers.
 // The arithmetic (fused multiply-adds acc - U V with l ascending, the row
 // scaled by one IEEE reciprocal of the pivot) matches the CPU reference
 // operation for operation.
+//
+// What bounds it: large blocks the FP64 pipe (11-14 operations per kernel entry
+// and k multiply-adds); small ones the chain of 2 (r + 1) dependent phases, each
+// a load, one entry's operations (64 cycles apiece for a warp) and a reduction.
+// So a phase costs one barrier: a CTA keeps its slices of U and V in shared
+// memory as far as they fit (ACA_KEEP doubles), the pivot row's U entries come
+// in one load, and a reduction is one shuffle tree per warp, one exchange in
+// shared memory and a second tree in every warp.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256, 4) k_aca(const HmatDesc* __restrict__ Hd, const int4* __restrict__ work,
+#define ACA_KEEP 5632  // doubles of U and V kept per CTA (four CTAs per SM)
+
+// Candidate of a reduction: |value| as its IEEE bits (-1.0 for none), index and
+// sign packed; ties to the lower index.  u: the largest |value| of any entry.
+struct AcaBest {
+  long long v, u;
+  int p;  // 2 index + (value negative)
+};
+__device__ __forceinline__ AcaBest aca_none() { return {__double_as_longlong(-1.0), __double_as_longlong(-1.0), 0x7fffffff}; }
+__device__ __forceinline__ void aca_take(AcaBest& a, const AcaBest& b) {
+  if (b.v > a.v || (b.v == a.v && b.p < a.p)) {
+    a.v = b.v;
+    a.p = b.p;
+  }
+  if (b.u > a.u) a.u = b.u;
+}
+template <int FROM>
+__device__ __forceinline__ void aca_shuffle(AcaBest& a) {
+#pragma unroll
+  for (int o = FROM; o > 0; o >>= 1) {
+    AcaBest b;
+    b.v = __shfl_xor_sync(0xffffffffu, a.v, o);
+    b.u = __shfl_xor_sync(0xffffffffu, a.u, o);
+    b.p = __shfl_xor_sync(0xffffffffu, a.p, o);
+    aca_take(a, b);
+  }
+}
+// The entry's value from its bits and sign.
+__device__ __forceinline__ double aca_value(const AcaBest& a) {
+  return __longlong_as_double(a.v | ((long long)(a.p & 1) << 63));
+}
+
+__device__ __forceinline__ void aca_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+__device__ __forceinline__ AcaBest aca_remote(const AcaBest* p, int rank) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+  unsigned r;
+  AcaBest b;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  asm volatile("ld.shared::cluster.s64 %0, [%1];" : "=l"(b.v) : "r"(r) : "memory");
+  asm volatile("ld.shared::cluster.s64 %0, [%1 + 8];" : "=l"(b.u) : "r"(r) : "memory");
+  asm volatile("ld.shared::cluster.s32 %0, [%1 + 16];" : "=r"(b.p) : "r"(r) : "memory");
+  return b;
+}
+
+template <bool CL>
+__global__ void __launch_bounds__(256, 4) k_aca(const HmatDesc* __restrict__ Hd, const int4* __restrict__ work, int C,
                                               ArgMax* __restrict__ part, unsigned int* __restrict__ bar,
                                               int* __restrict__ abort_flag, size_t pstride) {
   // problem of a batched launch: its descriptor, its partials, barriers and
@@ -85,8 +143,8 @@ __global__ void __launch_bounds__(256, 4) k_aca(const HmatDesc* __restrict__ Hd,
   part = (ArgMax*)((char*)part + blockIdx.y * pstride);
   bar = (unsigned int*)((char*)bar + blockIdx.y * pstride);
   abort_flag = (int*)((char*)abort_flag + blockIdx.y * pstride);
-  const int4 w = work[blockIdx.x];
-  const int lvl = w.x, bi = w.y, g = w.z, G = w.w;
+  const int4 w = work[CL ? blockIdx.x / C : blockIdx.x];
+  const int lvl = w.x, bi = w.y, g = CL ? blockIdx.x % C : w.z, G = CL ? C : w.w;
   const int base = blockIdx.x - g;
   const int64_t n = Hd->n;
   const int cap = Hd->cap, kind = Hd->kind;
@@ -100,103 +158,133 @@ __global__ void __launch_bounds__(256, 4) k_aca(const HmatDesc* __restrict__ Hd,
   const int rc = (m + G - 1) / G, cc = (p + G - 1) / G;
   const int r0 = min(m, g * rc), r1 = min(m, g * rc + rc);
   const int c0 = min(p, g * cc), c1 = min(p, g * cc + cc);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
+  extern __shared__ double keep[];  // steps l < kl: V on [c0, c1), then U on [r0, r1)
   __shared__ int rowp[FIFA_CAP_MAX], colp[FIFA_CAP_MAX];
-  __shared__ ArgMax shA[33];
-  __shared__ double shD[33];
+  __shared__ double piv_row[FIFA_CAP_MAX];  // the pivot row's U entries, then the pivot column's V entries
+  __shared__ AcaBest wbest[2][8], cbest[2];
+  const int kl = min(cap, ACA_KEEP / (rc + cc)), kstep = rc + cc;
+  unsigned int phase = 0;
+
+  // reduce over the node's CTAs; two buffers in turn, each written again only
+  // after a barrier that follows every read of it
+  bool dead = false;
+  auto reduce = [&](AcaBest a) -> AcaBest {
+    aca_shuffle<16>(a);
+    AcaBest* wb = wbest[phase & 1u];
+    if (lane == 0) wb[warp] = a;
+    __syncthreads();
+    a = wb[lane & 7];
+    aca_shuffle<4>(a);
+    if (G > 1) {
+      if constexpr (CL) {
+        if (tid == 0) cbest[phase & 1u] = a;
+        aca_cluster_sync();
+        a = aca_remote(&cbest[phase & 1u], min(lane & 7, G - 1));
+        aca_shuffle<4>(a);
+      } else {
+        // slots 2 * cta + parity
+        ArgMax* mine = part + 2 * (base + g) + (phase & 1u);
+        if (tid == 0) *mine = ArgMax{__longlong_as_double(a.v), a.p, __longlong_as_double(a.u)};
+        if (!group_barrier(bar + base, G * (phase + 1), Hd->status, abort_flag, Hd->spin)) dead = true;
+        a = aca_none();
+        for (int q = lane; q < G && !dead; q += 32) {
+          const ArgMax* pq = part + 2 * (base + q) + (phase & 1u);
+          aca_take(a, AcaBest{__double_as_longlong(__ldcg(&pq->v)), __double_as_longlong(__ldcg(&pq->sv)), __ldcg(&pq->i)});
+        }
+        aca_shuffle<16>(a);
+      }
+    }
+    ++phase;
+    return a;
+  };
+  // acc - sum_{l < k} piv_row[l] (this CTA's entry q of V or U in step l)
+  auto residual = [&](double acc, int k, const double* kp, const double* gp) {
+    const int k1 = min(k, kl);
+    int l = 0;
+#pragma unroll 4
+    for (; l < k1; ++l) acc = __fma_rn(-piv_row[l], kp[l * kstep], acc);
+#pragma unroll 4
+    for (; l < k; ++l) acc = __fma_rn(-piv_row[l], gp[(size_t)l * n], acc);
+    return acc;
+  };
 
   int i = m - 1, k = 0;
   bool hit = false;
-  unsigned int phase = 0;
-  if (m <= 0 || p <= 0) k = 0;
-  else
+  if (m > 0 && p > 0)
     while (true) {
       if (k == cap) { hit = true; break; }
-      // residual of row i over this CTA's columns, stored unnormalised in V[:, k]
+      // residual of row i over this CTA's columns, unnormalised in V[:, k]
+      if (tid < k) piv_row[tid] = __ldcg(Bs + (size_t)tid * n + s + i);
       const double xi = x[s + i];
-      ArgMax best{-1.0, 0x7fffffff, 0.0};
-      for (int j = c0 + threadIdx.x; j < c1; j += blockDim.x) {
-        double acc = kern_entry(kind, kc, xi, x[h + j]);
-        for (int l = 0; l < k; ++l)
-          acc = __fma_rn(-__ldcg(Bs + (size_t)l * n + s + i), Bs[(size_t)l * n + h + j], acc);
-        Bs[(size_t)k * n + h + j] = acc;
+      double first = 0.0;  // (the thread's first entry while the row's U arrives)
+      if (c0 + tid < c1) first = kern_entry(kind, kc, xi, x[h + c0 + tid]);
+      __syncthreads();
+      AcaBest best = aca_none();
+      for (int j = c0 + tid; j < c1; j += blockDim.x) {
+        const double en = j == c0 + tid ? first : kern_entry(kind, kc, xi, x[h + j]);
+        const double acc = residual(en, k, keep + (j - c0), Bs + h + j);
+        if (k < kl) keep[k * kstep + (j - c0)] = acc;
+        else Bs[(size_t)k * n + h + j] = acc;
         // an entry that would win is checked against the used columns (the
         // check runs only then: same result as checking every entry)
-        const ArgMax cand{fabs(acc), j, acc};
-        if (am_wins(best, cand)) {
+        const AcaBest cand{__double_as_longlong(fabs(acc)), 0, 2 * j + (__double2hiint(acc) < 0)};
+        if (cand.v > best.v || (cand.v == best.v && cand.p < best.p)) {
           bool used = false;
           for (int l = 0; l < k; ++l) used |= (colp[l] == j);
-          if (!used) best = cand;
+          if (!used) {
+            best.v = cand.v;
+            best.p = cand.p;
+          }
         }
       }
-      best = block_argmax(best, shA);
-      if (G > 1) {
-        if (threadIdx.x == 0) part[3 * (base + g)] = best;
-        ++phase;
-        if (!group_barrier(bar + base, G * phase, Hd->status, abort_flag, Hd->spin)) return;
-        ArgMax t{-1.0, 0x7fffffff, 0.0};
-        for (int q = threadIdx.x; q < G; q += blockDim.x) {
-          const ArgMax* pq = part + 3 * (base + q);
-          t = am_better(t, ArgMax{__ldcg(&pq->v), __ldcg(&pq->i), __ldcg(&pq->sv)});
-        }
-        best = block_argmax(t, shA);
-      }
-      if (!(best.v > 0.0)) break;
-      const int js = best.i;
-      const double piv = best.sv;
-      const double rpiv = __ddiv_rn(1.0, piv);
-      for (int j = c0 + threadIdx.x; j < c1; j += blockDim.x) {
-        double* vp = Bs + (size_t)k * n + h + j;
-        *vp = __dmul_rn(*vp, rpiv);
-      }
-      // residual of column js over this CTA's rows, stored in U[:, k]
+      best = reduce(best);
+      if (dead) return;
+      if (best.v <= 0 || best.v > 0x7ff0000000000000LL) break;  // no unused column, a zero row, or not a number
+      const int js = best.p >> 1;
+      // the pivot column's V entries: V[js, l] (its own CTA's copy in global memory)
+      if (tid < k) piv_row[tid] = __ldcg(Bs + (size_t)tid * n + h + js);
+      const double rpiv = __ddiv_rn(1.0, aca_value(best));
       const double xj = x[h + js];
-      double umax = 0.0;
-      ArgMax nb{-1.0, 0x7fffffff, 0.0};
-      for (int ii = r0 + threadIdx.x; ii < r1; ii += blockDim.x) {
-        double acc = kern_entry(kind, kc, x[s + ii], xj);
-        for (int l = 0; l < k; ++l)
-          acc = __fma_rn(-Bs[(size_t)l * n + s + ii], __ldcg(Bs + (size_t)l * n + h + js), acc);
+      if (r0 + tid < r1) first = kern_entry(kind, kc, x[s + r0 + tid], xj);
+      for (int j = c0 + tid; j < c1; j += blockDim.x) {
+        double* vp = Bs + (size_t)k * n + h + j;
+        if (k < kl) *vp = keep[k * kstep + (j - c0)] = __dmul_rn(keep[k * kstep + (j - c0)], rpiv);
+        else *vp = __dmul_rn(*vp, rpiv);
+      }
+      __syncthreads();
+      // residual of column js over this CTA's rows, in U[:, k]
+      AcaBest nb = aca_none();
+      for (int ii = r0 + tid; ii < r1; ii += blockDim.x) {
+        const double en = ii == r0 + tid ? first : kern_entry(kind, kc, x[s + ii], xj);
+        const double acc = residual(en, k, keep + cc + (ii - r0), Bs + s + ii);
+        if (k < kl) keep[k * kstep + cc + (ii - r0)] = acc;
         Bs[(size_t)k * n + s + ii] = acc;
-        umax = nn_max(umax, fabs(acc));
-        const ArgMax cand{fabs(acc), ii, acc};
-        if (am_wins(nb, cand)) {
+        const AcaBest cand{__double_as_longlong(fabs(acc)), 0, 2 * ii + (__double2hiint(acc) < 0)};
+        if (cand.v > nb.u) nb.u = cand.v;
+        if (cand.v > nb.v || (cand.v == nb.v && cand.p < nb.p)) {
           bool used = (ii == i);
           for (int l = 0; l < k; ++l) used |= (rowp[l] == ii);
-          if (!used) nb = cand;
+          if (!used) {
+            nb.v = cand.v;
+            nb.p = cand.p;
+          }
         }
       }
-      umax = block_max(umax, shD);
-      nb = block_argmax(nb, shA);
-      if (G > 1) {
-        if (threadIdx.x == 0) {
-          part[3 * (base + g) + 1] = ArgMax{umax, 0, 0.0};
-          part[3 * (base + g) + 2] = nb;
-        }
-        ++phase;
-        if (!group_barrier(bar + base, G * phase, Hd->status, abort_flag, Hd->spin)) return;
-        double tm = 0.0;
-        ArgMax t{-1.0, 0x7fffffff, 0.0};
-        for (int q = threadIdx.x; q < G; q += blockDim.x) {
-          const ArgMax* pq = part + 3 * (base + q);
-          tm = nn_max(tm, __ldcg(&pq[1].v));
-          t = am_better(t, ArgMax{__ldcg(&pq[2].v), __ldcg(&pq[2].i), __ldcg(&pq[2].sv)});
-        }
-        umax = block_max(tm, shD);
-        nb = block_argmax(t, shA);
-        // Slots: 3*cta + {0: row phase, 1-2: column phase}.  A slot is rewritten
-        // one phase later, after a barrier every reader has already passed.
-      }
-      if (umax <= eps) break;
-      if (threadIdx.x == 0) {
+      nb = reduce(nb);
+      if (dead) return;
+      if (__longlong_as_double(nb.u) <= eps) break;
+      if (tid == 0) {
         rowp[k] = i;
         colp[k] = js;
       }
       __syncthreads();
       ++k;
-      if (nb.v < 0.0) break;
-      i = nb.i;
+      if (nb.v < 0) break;
+      i = nb.p >> 1;
     }
+  if (CL && G > 1) aca_cluster_sync();  // no CTA leaves while another may still read its maxima
   if (g == 0 && threadIdx.x == 0) {
     Hd->rank[nid] = k;
     for (int l = 0; l < cap; ++l) {
@@ -210,7 +298,7 @@ __global__ void __launch_bounds__(256, 4) k_aca(const HmatDesc* __restrict__ Hd,
 // ---------------------------------------------------------------------------
 // ACA of small blocks (both sides <= ACA_WARP_MAX rows): one warp per block,
 // eight independent blocks per CTA.  Same arithmetic and pivot rules as k_aca
-// with G = 1 (so the same bases, bit for bit); the reductions are warp
+// (so the same bases, bit for bit); the reductions are warp
 // shuffles, with no CTA barrier and no idle warps in them.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ ArgMax warp_argmax_all(ArgMax a) {
@@ -319,8 +407,40 @@ __global__ void __launch_bounds__(256, 3) k_aca_warp(const HmatDesc* __restrict_
 // ---------------------------------------------------------------------------
 // Host launchers.
 // ---------------------------------------------------------------------------
+// CTAs of a cluster for each of `blocks` ACA blocks of one launch: up to eight
+// while all of them fill the GPU at most four CTAs to an SM, and not more than
+// leave 16 rows of a side to a CTA (span: rows and columns of the largest).
+static int aca_cluster(int64_t blocks, int span) {
+  int c = 1;
+  while (c < 8 && 2 * c * blocks <= 608 && span / (4 * c) >= 16) c *= 2;
+  return c;
+}
+
+static cudaError_t launch_aca_cluster(const HmatDesc* Hd, const int4* work, int blocks, int C, cudaStream_t st,
+                                      int nprob) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks * C, nprob);
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = ACA_KEEP * sizeof(double);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = C;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_aca<true>, Hd, work, C, (ArgMax*)nullptr, (unsigned int*)nullptr, (int*)nullptr,
+                            (size_t)0);
+}
+
+// Small blocks: one warp each when there are enough to fill the GPU, else a CTA
+// or a cluster each (the same bases either way: 15 blocks of n = 500 took one
+// warp each 278 us).
 cudaError_t launch_aca_warp(const HmatDesc* Hd, const int4* work, int nwork, cudaStream_t st, int nprob) {
   if (nwork <= 0) return cudaSuccess;
+  if ((int64_t)nwork * nprob <= 608)
+    return launch_aca_cluster(Hd, work, nwork, aca_cluster((int64_t)nwork * nprob, 2 * ACA_WARP_MAX), st, nprob);
   k_aca_warp<<<dim3((nwork + 7) / 8, nprob), 256, 0, st>>>(Hd, work, nwork);
   return cudaGetLastError();
 }
@@ -330,26 +450,32 @@ cudaError_t launch_leaf_assemble(const HmatDesc* Hd, int nleaf, cudaStream_t st,
   return cudaGetLastError();
 }
 
-cudaError_t launch_aca(const HmatDesc* Hd, const int4* work, int ncta, bool cooperative, ArgMax* part,
-                       unsigned int* bar, int* abort_flag, cudaStream_t st, int nprob, size_t pstride) {
+cudaError_t launch_aca_solo(const HmatDesc* Hd, const int4* work, int nblocks, int span, cudaStream_t st, int nprob) {
+  if (nblocks <= 0) return cudaSuccess;
+  return launch_aca_cluster(Hd, work, nblocks, aca_cluster((int64_t)nblocks * nprob, span), st, nprob);
+}
+
+cudaError_t launch_aca(const HmatDesc* Hd, const int4* work, int ncta, ArgMax* part, unsigned int* bar, int* abort_flag,
+                       cudaStream_t st, int nprob, size_t pstride) {
   if (ncta <= 0) return cudaSuccess;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ncta, nprob);
   cfg.blockDim = dim3(256);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = ACA_KEEP * sizeof(double);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = cooperative ? 1 : 0;
+  attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_aca, Hd, work, part, bar, abort_flag, pstride);
+  return cudaLaunchKernelEx(&cfg, k_aca<false>, Hd, work, 1, part, bar, abort_flag, pstride);
 }
 
 int aca_max_coresident_ctas() {
   int dev = 0, sms = 0, per_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_aca, 256, 0) != cudaSuccess) per_sm = 1;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_aca<false>, 256, ACA_KEEP * sizeof(double)) != cudaSuccess)
+    per_sm = 1;
   return sms * per_sm;
 }
