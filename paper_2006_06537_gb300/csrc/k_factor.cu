@@ -30,12 +30,13 @@
 __host__ __device__ inline int lf_nch(int Bm) { return Bm <= 64 ? 64 : 32; }
 
 template <typename T>
-__global__ void __launch_bounds__(256, 7) k_leaf_factor(const HmatDesc* __restrict__ Hd, const FactDesc* __restrict__ Fd) {
+__global__ void __launch_bounds__(256, 7)
+    k_leaf_factor(const HmatDesc* __restrict__ Hd, const FactDesc* __restrict__ Fd, int nsplit) {
   extern __shared__ double sm[];
   Hd += blockIdx.y;  // problem of a batched launch (descriptor arrays)
   Fd += blockIdx.y;
   if (Fd->skip && *Fd->skip) return;  // this factor is kept as it is
-  const int leaf = blockIdx.x;
+  const int leaf = blockIdx.x / nsplit, split = blockIdx.x % nsplit;
   const int L = Fd->L, Bm = Fd->Bm, cap = Fd->cap;
   const int64_t n = Fd->n;
   const double sc = Hd->scale, shf = Hd->shift;
@@ -74,7 +75,9 @@ __global__ void __launch_bounds__(256, 7) k_leaf_factor(const HmatDesc* __restri
     ncols = c;
   }
   __syncthreads();
-  const int nc = ncols;
+  // the leaf's CTAs factor it alike and share the columns
+  const int cfirst = ncols * split / nsplit, nc = ncols * (split + 1) / nsplit - cfirst;
+  clist += cfirst;
   T* Q = (T*)Fd->Q;
   auto load_chunk = [&](int c0, int w) {
     for (int t = threadIdx.x; t < w * m; t += blockDim.x) {
@@ -151,21 +154,23 @@ __global__ void __launch_bounds__(256, 7) k_leaf_factor(const HmatDesc* __restri
     }
     __syncthreads();
   }
-  double lsum = 0.0;
-  for (int k = threadIdx.x; k < m; k += blockDim.x) lsum += log(A[k * ld + k]);
-  lsum = block_sum(lsum, red);
-  if (threadIdx.x == 0) {
-    Fd->ld_parts[leaf] = lsum;
-    if (flag[0]) atomicOr(Fd->status, FIFA_DEV_NOT_SPD);
-  }
-  for (int k = threadIdx.x; k < m; k += blockDim.x) ((double*)Fd->Ldinv)[(size_t)leaf * Bm + k] = rinv[k];
-  T* Lout = (T*)Fd->Lleaf + (size_t)leaf * Bm * Bm;
-  for (int t = threadIdx.x; t < Bm * Bm; t += blockDim.x) {
-    int i = t % Bm, j = t / Bm;
-    // L in the lower triangle, L^T mirrored into the upper one (transposed
-    // solves then read contiguous columns as well)
-    double v = (i < m && j < m) ? (i >= j ? A[j * ld + i] : A[i * ld + j]) : 0.0;
-    Lout[t] = (T)v;
+  if (split == 0) {
+    double lsum = 0.0;
+    for (int k = threadIdx.x; k < m; k += blockDim.x) lsum += log(A[k * ld + k]);
+    lsum = block_sum(lsum, red);
+    if (threadIdx.x == 0) {
+      Fd->ld_parts[leaf] = lsum;
+      if (flag[0]) atomicOr(Fd->status, FIFA_DEV_NOT_SPD);
+    }
+    for (int k = threadIdx.x; k < m; k += blockDim.x) ((double*)Fd->Ldinv)[(size_t)leaf * Bm + k] = rinv[k];
+    T* Lout = (T*)Fd->Lleaf + (size_t)leaf * Bm * Bm;
+    for (int t = threadIdx.x; t < Bm * Bm; t += blockDim.x) {
+      int i = t % Bm, j = t / Bm;
+      // L in the lower triangle, L^T mirrored into the upper one (transposed
+      // solves then read contiguous columns as well)
+      double v = (i < m && j < m) ? (i >= j ? A[j * ld + i] : A[i * ld + j]) : 0.0;
+      Lout[t] = (T)v;
+    }
   }
   store_chunk(0, w0);
   if (nc <= w0) return;
@@ -190,6 +195,271 @@ __global__ void __launch_bounds__(256, 7) k_leaf_factor(const HmatDesc* __restri
     }
     store_chunk(c0, w);
     __syncthreads();
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Leaves of more than 64 rows: the same factor in blocks of LB_NB columns.  Per
+// block: the diagonal block's factor by one warp (warp_chol_inv), the panel
+// below it and the block row of the right-hand sides by substitution (a thread
+// per row or column; not by the block's inverse, whose backward error grows
+// with the block's condition number), then one rank-LB_NB update of the
+// trailing triangle and of the right-hand sides: two barriers per eight columns
+// instead of one per column, and LB_NB multiply-adds per load and store of an
+// entry.  The next diagonal block is factored by warp 0 while the other warps
+// update.  The matrix is a packed lower triangle, column after column, so the
+// trailing triangle is one contiguous range and two CTAs of 128-row leaves fit
+// an SM.
+// 1024 leaves of 128 rows with 21 ancestor columns: 3.04 -> 1.66 ms (0.92 ms at
+// the FP64 peak; 1024 leaves are 3.4 waves of two CTAs per SM).  The line at 64
+// rows: 32 leaves of 64 rows take 84 us either way, 512 leaves of 40 rows 73 us
+// column by column and 81 us in blocks (the chain of diagonal blocks).
+// ---------------------------------------------------------------------------
+#define LB_NB 8
+#define LB_COLS 32  // ancestor columns per pass
+
+__host__ __device__ inline size_t leaf_block_doubles(int Bm) {
+  const size_t nblk = (Bm + LB_NB - 1) / LB_NB;
+  return (size_t)Bm * (Bm + 1) / 2 + (size_t)LB_COLS * (Bm | 1) + nblk * LB_NB * LB_NB + LB_NB * LB_NB + LB_NB + 40 + Bm;
+}
+
+__global__ void __launch_bounds__(256, 4)
+    k_leaf_factor_block(const HmatDesc* __restrict__ Hd, const FactDesc* __restrict__ Fd, int nsplit) {
+  extern __shared__ double sm[];
+  Hd += blockIdx.y;  // problem of a batched launch (descriptor arrays)
+  Fd += blockIdx.y;
+  if (Fd->skip && *Fd->skip) return;  // this factor is kept as it is
+  const int leaf = blockIdx.x / nsplit, split = blockIdx.x % nsplit;
+  const int L = Fd->L, Bm = Fd->Bm, cap = Fd->cap;
+  const int64_t n = Fd->n;
+  const double sc = Hd->scale, shf = Hd->shift;
+  const int* bnd = Fd->bnd;
+  const int s = bnd[bnd_off(L) + leaf], e = bnd[bnd_off(L) + leaf + 1], m = e - s;
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+  const int ld = Bm | 1;
+  double* A = sm;                                   // packed: entry (i, j), i >= j, at off(j) + i - j
+  double* X = A + (size_t)Bm * (Bm + 1) / 2;        // columns ld apart
+  double* Dg = X + (size_t)LB_COLS * ld;           // diagonal blocks of L, reciprocals on the diagonal
+  double* Mw = Dg + (size_t)((Bm + LB_NB - 1) / LB_NB) * LB_NB * LB_NB;
+  double* Rd = Mw + LB_NB * LB_NB;
+  double* red = Rd + LB_NB;                         // 40
+  double* dinv = red + 40;                          // reciprocal pivots
+  __shared__ int ncols, bad, chunk;
+  __shared__ int pre[FIFA_LEVELS_MAX + 1];
+  auto off = [&](int j) { return j * m - j * (j - 1) / 2; };
+  const double* D = Hd->leaves + (size_t)leaf * Bm * Bm;
+  for (int t = tid; t < m * m; t += nt) {
+    const int i = t % m, j = t / m;
+    if (i < j) continue;
+    double v = __dmul_rn(sc, D[(size_t)j * Bm + i]);
+    if (i == j) v = __dadd_rn(v, Hd->diag ? Hd->diag[s + i] : shf);
+    A[off(j) + i - j] = v;
+  }
+  if (tid < 32) {  // prefix sums of the ancestors' ranks
+    int c = lane < L ? Hd->rank[node_id(lane, leaf >> (L - lane))] : 0;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, c, o);
+      if (lane >= o) c += t;
+    }
+    if (lane < L) pre[lane + 1] = c;
+    if (lane == 0) {
+      pre[0] = 0;
+      bad = 0;
+    }
+    if (lane == L - 1 || (L == 0 && lane == 0)) ncols = L == 0 ? 0 : c;
+  }
+  __syncthreads();
+  // the leaf's CTAs factor it alike and share the columns
+  const int cfirst = ncols * split / nsplit, nc = ncols * (split + 1) / nsplit - cfirst;
+  double* Q = (double*)Fd->Q;
+  // column cfirst + c: its level, basis column and whether this leaf lies in the
+  // left child (U rows, scaled in a view)
+  auto column = [&](int c, double& scl) -> size_t {
+    int l = 0;
+    while (pre[l + 1] <= cfirst + c) ++l;
+    scl = ((leaf >> (L - l - 1)) & 1) ? 1.0 : sc;
+    return ((size_t)l * cap + (cfirst + c - pre[l])) * n + s;
+  };
+  auto load_cols = [&](int c0, int w) {
+    for (int cc = tid >> 5; cc < w; cc += nt >> 5) {
+      double scl;
+      const double* src = Hd->bases + column(c0 + cc, scl);
+      for (int i = lane; i < m; i += 32) X[cc * ld + i] = scl == 1.0 ? src[i] : __dmul_rn(scl, src[i]);
+    }
+  };
+  auto store_cols = [&](int c0, int w) {
+    for (int cc = tid >> 5; cc < w; cc += nt >> 5) {
+      double scl;
+      double* dst = Q + column(c0 + cc, scl);
+      for (int i = lane; i < m; i += 32) dst[i] = X[cc * ld + i];
+    }
+  };
+  // rows [k0, k0 + bw) of w right-hand sides solved with the diagonal block iv, by the threads t0, t0 + 1, ..
+  auto solve_block = [&](int k0, int bw, int w, const double* iv, int t0) {
+    for (int cc = tid - t0; cc < w; cc += nt - t0) {
+      if (cc < 0) continue;
+      double x[LB_NB];
+#pragma unroll
+      for (int q = 0; q < LB_NB; ++q) x[q] = q < bw ? X[cc * ld + k0 + q] : 0.0;
+#pragma unroll
+      for (int q = 0; q < LB_NB; ++q)
+        if (q < bw) {
+#pragma unroll
+          for (int u = 0; u < q; ++u) x[q] -= iv[q * LB_NB + u] * x[u];
+          x[q] *= iv[q * LB_NB + q];
+          X[cc * ld + k0 + q] = x[q];
+        }
+    }
+  };
+  const int w0 = min(LB_COLS, nc);
+  load_cols(0, w0);
+  // warp 0: the diagonal block at kd, less the products of the block of bq
+  // columns at kq before it (bq = 0: none), factored
+  auto factor_diag = [&](int kd, int kq, int bq) {
+    const int bw = min(LB_NB, m - kd);
+    double* iv = Dg + (size_t)(kd / LB_NB) * LB_NB * LB_NB;
+    for (int t = lane; t < bw * bw; t += 32) {
+      const int a = t / bw, b = t % bw;
+      if (a > b) continue;
+      double v = A[off(kd + a) + b - a];
+      for (int q = 0; q < bq; ++q) v -= A[off(kq + q) + kd + b - kq - q] * A[off(kq + q) + kd + a - kq - q];
+      Mw[a * LB_NB + b] = v;
+    }
+    __syncwarp();
+    if (!warp_chol_inv(Mw, LB_NB, bw, Rd, lane) && lane == 0) bad = 1;
+    for (int t = lane; t < bw * bw; t += 32) {
+      const int a = t / bw, b = t % bw;  // L = R^T
+      if (a > b) continue;
+      A[off(kd + a) + b - a] = a == b ? Rd[a] : Mw[a * LB_NB + b];
+      iv[b * LB_NB + a] = Mw[a * LB_NB + b];  // reciprocal pivots on the diagonal
+    }
+    if (lane < bw) dinv[kd + lane] = Mw[lane * LB_NB + lane];
+  };
+  __syncthreads();
+  if (tid < 32 && m > 0) factor_diag(0, 0, 0);
+  for (int k0 = 0; k0 < m; k0 += LB_NB) {
+    const int bw = min(LB_NB, m - k0), k1 = k0 + bw, w = m - k1;
+    const double* iv = Dg + (size_t)(k0 / LB_NB) * LB_NB * LB_NB;
+    if (tid == 0) chunk = 0;
+    __syncthreads();
+    // panel: row i of L21 = A21 L11^-T; block row of the right-hand sides
+    const int tp = (min(w, nt / 2) + 31) & ~31;  // threads on the panel's rows
+    if (tid < tp) {
+      for (int r = tid; r < w; r += tp) {
+        const int i = k1 + r;
+        double x[LB_NB];
+#pragma unroll
+        for (int q = 0; q < LB_NB; ++q) x[q] = q < bw ? A[off(k0 + q) + i - k0 - q] : 0.0;
+#pragma unroll
+        for (int q = 0; q < LB_NB; ++q)
+          if (q < bw) {
+#pragma unroll
+            for (int u = 0; u < q; ++u) x[q] -= x[u] * iv[q * LB_NB + u];
+            x[q] *= iv[q * LB_NB + q];
+            A[off(k0 + q) + i - k0 - q] = x[q];
+          }
+      }
+    } else {
+      solve_block(k0, bw, w0, iv, tp);
+    }
+    __syncthreads();
+    // trailing triangle (contiguous from off(k1)) and right-hand sides, 32
+    // entries at a time to whichever warp is free; warp 0 first factors the next
+    // diagonal block
+    const int tri = w * (w + 1) / 2, all = tri + w * w0;
+    if (tid < 32 && w > 0) factor_diag(k1, k0, bw);
+    while (true) {
+      int t = 0;
+      if (lane == 0) t = atomicAdd(&chunk, 32);
+      t = __shfl_sync(0xffffffffu, t, 0);
+      if (t >= all) break;
+      t += lane;
+      if (t >= all) continue;
+      int i;
+      const double* right;  // the second factor's LB_NB entries and their distance
+      int rstep;
+      double* dst;
+      if (t < tri) {
+        // column-major lower triangle read backwards is a row-major one: entry
+        // t is (w - 1 - b, w - 1 - a), tri - 1 - t = a (a + 1) / 2 + b
+        const int tr = tri - 1 - t;
+        int a = (int)((sqrtf(8.0f * (float)tr + 1.0f) - 1.0f) * 0.5f);
+        if ((a + 1) * (a + 2) / 2 <= tr) ++a;
+        if (a * (a + 1) / 2 > tr) --a;
+        const int b = tr - a * (a + 1) / 2, j = k1 + w - 1 - a;
+        i = k1 + w - 1 - b;
+        if (i < k1 + LB_NB) continue;  // in the next diagonal block
+        dst = A + off(k1) + t;
+        right = A + off(k0) + j - k0;
+        rstep = -1;
+      } else {
+        const int u = t - tri, cc = u / w;
+        i = k1 + u % w;
+        dst = X + cc * ld + i;
+        right = X + cc * ld + k0;
+        rstep = 1;
+      }
+      double v = *dst;
+      const double* left = A + off(k0) + i - k0;
+      // column q of the panel starts m - k0 - q entries after column q - 1, one row further
+      if (bw == LB_NB) {
+        int lo = 0, ro = 0;
+#pragma unroll
+        for (int q = 0; q < LB_NB; ++q) {
+          v -= left[lo] * right[ro];
+          const int st = m - k0 - q - 1;
+          lo += st;
+          ro += rstep > 0 ? 1 : st;
+        }
+      } else {
+        int lo = 0, ro = 0;
+        for (int q = 0; q < bw; ++q) {
+          v -= left[lo] * right[ro];
+          const int st = m - k0 - q - 1;
+          lo += st;
+          ro += rstep > 0 ? 1 : st;
+        }
+      }
+      *dst = v;
+    }
+    __syncthreads();
+  }
+  if (split == 0) {
+    double lsum = 0.0;
+    for (int k = tid; k < m; k += nt) lsum += log(A[off(k)]);
+    lsum = block_sum(lsum, red);
+    if (tid == 0) {
+      Fd->ld_parts[leaf] = lsum;
+      if (bad) atomicOr(Fd->status, FIFA_DEV_NOT_SPD);
+    }
+    for (int k = tid; k < m; k += nt) ((double*)Fd->Ldinv)[(size_t)leaf * Bm + k] = dinv[k];
+    // L in the lower triangle, L^T mirrored into the upper one
+    double* Lout = (double*)Fd->Lleaf + (size_t)leaf * Bm * Bm;
+    for (int t = tid; t < Bm * Bm; t += nt) {
+      const int i = t % Bm, j = t / Bm;
+      Lout[t] = (i < m && j < m) ? (i >= j ? A[off(j) + i - j] : A[off(i) + j - i]) : 0.0;
+    }
+  }
+  store_cols(0, w0);
+  // further columns: forward substitution by blocks with the finished factor
+  for (int c0 = w0; c0 < nc; c0 += LB_COLS) {
+    const int wc = min(LB_COLS, nc - c0);
+    __syncthreads();
+    load_cols(c0, wc);
+    __syncthreads();
+    for (int k0 = 0; k0 < m; k0 += LB_NB) {
+      const int bw = min(LB_NB, m - k0), k1 = k0 + bw, w = m - k1;
+      solve_block(k0, bw, wc, Dg + (size_t)(k0 / LB_NB) * LB_NB * LB_NB, 0);
+      __syncthreads();
+      for (int t = tid; t < w * wc; t += nt) {
+        const int cc = t / w, i = k1 + t % w;
+        double v = X[cc * ld + i];
+        for (int q = 0; q < bw; ++q) v -= A[off(k0 + q) + i - k0 - q] * X[cc * ld + k0 + q];
+        X[cc * ld + i] = v;
+      }
+      __syncthreads();
+    }
+    store_cols(c0, wc);
   }
 }
 
@@ -1000,25 +1270,28 @@ static int smem_optin() {
   return v;
 }
 
-template <typename T>
-static cudaError_t launch_leaf_factor_t(const HmatDesc* Hd, const FactDesc* Fd, int nleaf, size_t smem, cudaStream_t st,
-                                        int nprob) {
-  if (smem > (size_t)smem_optin()) return cudaErrorInvalidConfiguration;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_leaf_factor<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  k_leaf_factor<T><<<dim3(nleaf, nprob), 256, smem, st>>>(Hd, Fd);
-  return cudaGetLastError();
-}
-
 // Factorizations are computed in FP64 (prec 0); an FP32 factor is only ever a
-// rounded copy of an FP64 one (k_mixed.cu), never factored directly.
+// rounded copy of an FP64 one (k_mixed.cu), never factored directly.  When the
+// leaves are too few to fill the GPU, up to four CTAs share a leaf's ancestor
+// columns (each repeats its Cholesky factor; 32 leaves of 64 rows with 47
+// columns 122 -> 84 us).
 cudaError_t launch_leaf_factor(const HmatDesc* Hd, const FactDesc* Fd, int prec, int nleaf, int Bm, int L, int cap,
                                cudaStream_t st, int nprob) {
   if (prec != 0) return cudaErrorInvalidValue;
-  size_t smem = leaf_factor_smem(Bm, L, cap, 0);
-  return launch_leaf_factor_t<double>(Hd, Fd, nleaf, smem, st, nprob);
+  int nsplit = 1;
+  while (nsplit < 4 && 2 * (int64_t)nsplit * nleaf * nprob <= 304) nsplit *= 2;
+  const bool block = Bm > 64;
+  const size_t smem = block ? leaf_block_doubles(Bm) * sizeof(double) : leaf_factor_smem(Bm, L, cap, 0);
+  if (smem > (size_t)smem_optin()) return cudaErrorInvalidConfiguration;
+  if (smem > 48 * 1024) {
+    cudaError_t e = block ? cudaFuncSetAttribute(k_leaf_factor_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
+                          : cudaFuncSetAttribute(k_leaf_factor<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  const dim3 grid(nleaf * nsplit, nprob);
+  if (block) k_leaf_factor_block<<<grid, 256, smem, st>>>(Hd, Fd, nsplit);
+  else k_leaf_factor<double><<<grid, 256, smem, st>>>(Hd, Fd, nsplit);
+  return cudaGetLastError();
 }
 
 static cudaError_t launch_level_wide(const FactDesc* Fd, int lvl, int nodes, int G, int cap, double* part,

@@ -60,70 +60,6 @@ __device__ __forceinline__ double ld_cluster(const double* p, int rank) {
   return v;
 }
 
-// One warp, in place: M (r x r symmetric, r <= 16, rows ld apart, upper triangle
-// read) = R^T R.  Leaves R above the diagonal of M, its diagonal in Rd, and
-// R^-T below and on the diagonal of M (1 / R_kk there).  Left-looking, lane =
-// column: row k of R (lanes > k) and of R^-T (lanes < k) are one dot product
-// each.  A warp issues an FP64 instruction every 64 cycles (its quarter of the
-// SM's FP64 pipe), so what counts is their number, 7 + k for pivot k: the
-// reciprocal root is the hardware's approximation y refined by one step of
-// Householder's method of third order, y + y e (1/2 + 3/8 e) with e = 1 - d y^2
-// (what remains, about e^3, is far below the rounding), and the diagonal of R
-// is left to one product at the end.  A pivot that is not positive is taken as
-// 1 and reported.
-__device__ __noinline__ bool warp_chol_inv(double* M, int ld, int r, double* Rd, int lane) {
-  constexpr unsigned FULL = 0xffffffffu;
-  bool ok = true;
-  double acc = lane < r ? M[lane] : 0.0;  // row 0
-  for (int k = 0; k < r; ++k) {
-    double d = __shfl_sync(FULL, acc, k);
-    const long long bits = __double_as_longlong(d);
-    if (!(bits > 0 && bits <= 0x7ff0000000000000LL)) {  // d > 0, tested on the integer pipe
-      ok = false;
-      d = 1.0;
-    }
-    const int ex = (__double2hiint(d) >> 20) & 0x7ff;
-    double rs;
-    if (ex < 100 || ex > 1900) {  // the approximation flushes subnormals, d y must not overflow
-      rs = rsqrt(d);
-    } else {
-      double y;
-      asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-      const double e = fma(-(d * y), y, 1.0);
-      rs = fma(y * e, fma(0.375, e, 0.5), y);
-    }
-    const double own = lane == k ? rs : acc * rs;
-    if (lane == k) Rd[k] = d;
-    if (lane < r) M[k * ld + lane] = own;
-    if (k + 1 == r) break;
-    // row k + 1 over the rows i <= k: columns of R for lanes > k, of R^-T (from
-    // its diagonal on) else
-    const bool right = lane > k;
-    acc = right && lane < r ? M[(k + 1) * ld + lane] : 0.0;
-    acc -= __shfl_sync(FULL, own, k + 1) * own;
-    const int lo = right ? 0 : lane;
-    const double* col = M + min(lane, r - 1);
-    const double* piv = M + k + 1;
-    int i = 0;
-    for (; i + 4 <= k; i += 4) {
-      double a[4], b[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        a[u] = piv[(i + u) * ld];
-        b[u] = i + u >= lo ? col[(i + u) * ld] : 0.0;
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) acc -= a[u] * b[u];
-    }
-    for (; i < k; ++i) acc -= piv[i * ld] * (i >= lo ? col[i * ld] : 0.0);
-    __syncwarp();
-  }
-  __syncwarp();
-  if (lane < r) Rd[lane] *= M[lane * ld + lane];  // sqrt(d) = d / sqrt(d)
-  __syncwarp();
-  return ok;
-}
-
 // Pairs of columns in shared memory (column c at src + c ld): out[idx(o)] = sum
 // over local rows [a0, a1) of column ca times column cb, o -> (ca, cb) by pair().
 template <typename PairF, typename IdxF>
