@@ -86,12 +86,15 @@ static int levels_for(int64_t n, int B) {
   return L;
 }
 
-// Partials of the fused sweep: two buffers of one projection per CTA, for up to
-// min(nleaf, FS_CTAS_MAX) CTAs (none with independent CTAs: no grid barriers).
+// Partials of the fused sweep: one projection per CTA, level and sweep (a solve
+// has two), for up to min(nleaf, FS_CTAS_MAX) CTAs (none with independent CTAs:
+// no CTA hands anything over).
 static size_t fused_sweep_part_doubles(const Plan* P, const fifa_opts& o) {
   if (o.independent_ctas) return 1;
-  return (size_t)2 * std::min(P->nleaf, FS_CTAS_MAX) * FS_PART_STRIDE;
+  return (size_t)2 * std::max(1, std::min(P->L, 10)) * std::min(P->nleaf, FS_CTAS_MAX) * o.rank_cap * SWEEP_RHS_MAX;
 }
+// Bytes of its abort flag and counters.
+static size_t fused_sweep_bar_bytes(const Plan* P) { return sizeof(unsigned int) * fs_bar_uints(std::min(P->L, 10)); }
 
 // Partials of the fused H-matvec: one projection per CTA and level below the
 // CTA level, for up to min(nleaf, FS_CTAS_MAX) CTAs and 10 such levels.
@@ -236,7 +239,7 @@ static Plan* plan_build(int64_t n, const fifa_opts& o, int aca_cores, const int*
   add(sizeof(double) * 512);                                              // reduction partials
   add(256);                                                               // flags
   add(sizeof(double) * fused_sweep_part_doubles(P, o));                   // fused sweep partials
-  add(256);                                                               // fused sweep barrier
+  add(fused_sweep_bar_bytes(P));                                          // fused sweep abort flag and counters
   add(sizeof(double) * fused_mv_part_doubles(P, o));                      // fused matvec partials
   add(256);                                                               // fused matvec barrier
   add(sizeof(double) * PCG_SCRATCH_DOUBLES);                              // mixed-precision solve state
@@ -404,7 +407,7 @@ Scratch carve(fifa_ctx* ctx, Plan* P) {
   S.red = (double*)take(sizeof(double) * 512);
   S.flags = (int*)take(256);
   S.fs_part = (double*)take(sizeof(double) * fused_sweep_part_doubles(P, ctx->opts));
-  S.fs_bar = (unsigned int*)take(256);
+  S.fs_bar = (unsigned int*)take(fused_sweep_bar_bytes(P));
   S.mv_fpart = (double*)take(sizeof(double) * fused_mv_part_doubles(P, ctx->opts));
   S.mv_bar = (unsigned int*)take(256);
   S.pcg = (double*)take(sizeof(double) * PCG_SCRATCH_DOUBLES);
@@ -956,9 +959,8 @@ fifa_status sweep_enqueue_batched(fifa_ctx* ctx, Plan* P, const FactDesc* F0, do
   Scratch S = carve(ctx, P);
   ctx->active_scratch = saved;
   cudaStream_t s = ctx->stream;
-  CK(cudaMemset2DAsync(S.fs_bar, sstride, 0, sizeof(unsigned int), nprob, s));
-  CK(cudaMemset2DAsync(S.flags, sstride, 0, sizeof(int), nprob, s));
-  CK(launch_sweep_fused_batched(F0, ls, rows, vlist, nprob, mode, S.fs_part, S.fs_bar, S.flags, sstride, s));
+  CK(cudaMemset2DAsync(S.fs_bar, sstride, 0, sizeof(unsigned int) * fs_bar_uints(ls), nprob, s));
+  CK(launch_sweep_fused_batched(F0, ls, rows, vlist, nprob, mode, S.fs_part, S.fs_bar, (int*)S.fs_bar, sstride, s));
   return FIFA_OK;
 }
 
@@ -967,10 +969,9 @@ fifa_status sweep_enqueue_desc(fifa_ctx* ctx, Plan* P, const FactDesc* Fdev, int
   Scratch S = carve(ctx, P);
   cudaStream_t s = ctx->stream;
   if (P->fs_ls >= 0) {
-    CK(cudaMemsetAsync(S.fs_bar, 0, sizeof(unsigned int), s));
-    CK(cudaMemsetAsync(S.flags, 0, sizeof(int), s));
+    if (mode != 5) CK(cudaMemsetAsync(S.fs_bar, 0, sizeof(unsigned int) * fs_bar_uints(P->fs_ls), s));
     CK(launch_sweep_fused(Fdev, prec, P->fs_ls, P->fs_rows, ctx->opts.rank_cap, v, nrhs, mode, S.fs_part, S.fs_bar,
-                          S.flags, s, active));
+                          (int*)S.fs_bar, s, active));
     return FIFA_OK;
   }
   auto level = [&](int l, int zsel, int zt) -> cudaError_t {

@@ -47,7 +47,7 @@ struct Scratch {
   double* red;  // 512 doubles of reduction partials
   int* flags;
   double* fs_part;        // fused sweep partials
-  unsigned int* fs_bar;   // fused sweep grid barrier
+  unsigned int* fs_bar;   // fused sweep: abort flag, counters
   double* mv_fpart;       // fused H-matvec partials
   unsigned int* mv_bar;   // fused H-matvec grid barrier
   double* pcg;            // PCG_SCRATCH_DOUBLES: partial sums and state of a mixed-precision solve

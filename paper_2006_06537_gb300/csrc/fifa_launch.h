@@ -51,8 +51,11 @@ cudaError_t launch_logdet_reduce(const FactDesc* Fd, cudaStream_t st, int nprob 
 cudaError_t launch_sweep_level(const FactDesc* Fd, int prec, int lvl, int nodes, int G, double* v, int nrhs, double* part,
                                int zsel, int ztrans, cudaStream_t st, const int* active = nullptr);
 // Fused sweep (one cooperative launch of 2^ls CTAs; rows >= the longest
-// level-ls node).  part: 2 * 2^ls * FS_PART_STRIDE doubles; bar zeroed before.
-#define FS_PART_STRIDE (2 * FIFA_CAP_MAX * SWEEP_RHS_MAX)
+// level-ls node).  part: 2 ls slots of 2^ls x cap x SWEEP_RHS_MAX doubles; bar,
+// zeroed before: the abort flag, then a counter per node of the levels < ls for
+// each of two sweeps.
+#define FS_BAR_COUNTERS 16
+inline size_t fs_bar_uints(int ls) { return FS_BAR_COUNTERS + ((size_t)2 << ls); }
 #define FS_CTAS_MAX 1024
 int sweep_fused_coresident(int prec, int rows, int cap);
 // mode 0: W v, 1: W^-1 v, 2: W^T v, 3: W^-T v, 4: W^-T W^-1 v (both inverse sweeps

@@ -110,75 +110,98 @@ __device__ __forceinline__ T reg_sel(const T (&a)[N], int q) {
 // upper triangle (L[k][j] at k*Bm + j, j < k): every step reads one contiguous
 // column, L's for modes 0 / 1 and L^T's for modes 2 / 3.
 // ---------------------------------------------------------------------------
-template <typename T, typename V, int RPL>  // RPL: rows per lane, 32 RPL >= m; dinv: reciprocal pivots
-__device__ __forceinline__ void leaf_warp_apply_r(const T* __restrict__ Lm, const T* __restrict__ dinv, int Bm,
-                                                  int m, V* vj, int mode, int lane) {
-  T x[RPL], o[RPL];
+// RPL: rows per lane, 32 RPL >= m; dinv: reciprocal pivots; NR right-hand sides
+// (v1 for the second) share the loads of L.  The CH columns after the current
+// ones are in flight while those are used: a warp spends 64 cycles on every FP64
+// instruction, so a chunk covers the load's latency (64-row leaves: a dependent
+// load per column took most of a 30 us substitution).
+template <typename T, typename V, int RPL, int CH, int MODE, int NR>
+__device__ __forceinline__ void leaf_warp_chunks(const T* __restrict__ Lm, const T* __restrict__ dinv, int Bm, int m,
+                                                 V* v0, V* v1, int lane) {
+  constexpr unsigned FULL = 0xffffffffu;
+  constexpr bool subst = MODE == 1 || MODE == 3;
+  T x[NR][RPL], o[NR][RPL];
 #pragma unroll
   for (int q = 0; q < RPL; ++q) {
-    int i = lane + 32 * q;
-    x[q] = i < m ? (T)vj[i] : (T)0;
-    o[q] = (T)0;
+    const int i = lane + 32 * q;
+    x[0][q] = i < m ? (T)v0[i] : (T)0;
+    if (NR > 1) x[NR - 1][q] = i < m ? (T)v1[i] : (T)0;
+#pragma unroll
+    for (int j = 0; j < NR; ++j) o[j][q] = subst ? x[j][q] : (T)0;
   }
-  if (mode == 0) {  // o_i = sum_{k<=i} L[i][k] x_k
-    for (int k = 0; k < m; ++k) {
-      T xk = __shfl_sync(0xffffffffu, reg_sel<T, RPL>(x, k >> 5), k & 31);
+  auto fetch = [&](int t0, T (&c)[CH][RPL], T (&d)[CH]) {
+#pragma unroll
+    for (int u = 0; u < CH; ++u) {
+      const int k = MODE == 3 ? m - 1 - (t0 + u) : t0 + u;
+      const bool in = t0 + u < m;
+      d[u] = subst && in ? dinv[k] : (T)1;
 #pragma unroll
       for (int q = 0; q < RPL; ++q) {
-        int i = lane + 32 * q;
-        if (i >= k && i < m) o[q] += Lm[(size_t)k * Bm + i] * xk;
+        const int i = lane + 32 * q;
+        c[u][q] = in && i < m ? Lm[(size_t)k * Bm + i] : (T)0;
       }
     }
-  } else if (mode == 1) {  // forward substitution
+  };
+  T cur[CH][RPL], dcur[CH];
+  fetch(0, cur, dcur);
+  for (int t0 = 0; t0 < m; t0 += CH) {
+    T nxt[CH][RPL], dnxt[CH];
+    fetch(t0 + CH, nxt, dnxt);
 #pragma unroll
-    for (int q = 0; q < RPL; ++q) o[q] = x[q];
-    for (int k = 0; k < m; ++k) {
-      const int qk = k >> 5;
-      T ok = (T)0;
+    for (int u = 0; u < CH; ++u) {
+      if (t0 + u < m) {
+        const int k = MODE == 3 ? m - 1 - (t0 + u) : t0 + u;
+        T xk[NR];
 #pragma unroll
-      for (int q = 0; q < RPL; ++q)
-        if (q == qk) ok = o[q];
-      T xk = __shfl_sync(0xffffffffu, ok, k & 31) * dinv[k];
+        for (int j = 0; j < NR; ++j) {
+          xk[j] = __shfl_sync(FULL, reg_sel<T, RPL>(subst ? o[j] : x[j], k >> 5), k & 31);
+          if (subst) xk[j] *= dcur[u];
+        }
 #pragma unroll
-      for (int q = 0; q < RPL; ++q) {
-        int i = lane + 32 * q;
-        if (i == k) o[q] = xk;
-        else if (i > k && i < m) o[q] -= Lm[(size_t)k * Bm + i] * xk;
+        for (int q = 0; q < RPL; ++q) {
+          // whole row groups on the finished side of column k: no arithmetic
+          if (MODE == 0 || MODE == 1 ? 32 * q + 31 < k : 32 * q > k) continue;
+          const int i = lane + 32 * q;
+          const T a = cur[u][q];
+#pragma unroll
+          for (int j = 0; j < NR; ++j) {
+            if (MODE == 0) {
+              if (i >= k) o[j][q] += a * xk[j];
+            } else if (MODE == 2) {
+              if (i <= k) o[j][q] += a * xk[j];
+            } else {
+              if (i == k) o[j][q] = xk[j];
+              else if (MODE == 1 ? i > k : i < k) o[j][q] -= a * xk[j];
+            }
+          }
+        }
       }
     }
-  } else if (mode == 2) {  // o_j = sum_{k>=j} L[k][j] x_k, right-looking over k
-    // row k of L is column k of the stored upper triangle (L^T mirrored there):
-    // coalesced, and no cross-lane sums
-    for (int k = 0; k < m; ++k) {
-      const T xk = __shfl_sync(0xffffffffu, reg_sel<T, RPL>(x, k >> 5), k & 31);
 #pragma unroll
-      for (int q = 0; q < RPL; ++q) {
-        const int j = lane + 32 * q;
-        if (j <= k) o[q] += Lm[(size_t)k * Bm + j] * xk;
-      }
-    }
-  } else {  // backward substitution L^T x = v, column-oriented (x_k, then o_j -= L[k][j] x_k for j < k)
+    for (int u = 0; u < CH; ++u) {
+      dcur[u] = dnxt[u];
 #pragma unroll
-    for (int q = 0; q < RPL; ++q) o[q] = x[q];
-    for (int k = m - 1; k >= 0; --k) {
-      const int qk = k >> 5;
-      T ok = (T)0;
-#pragma unroll
-      for (int q = 0; q < RPL; ++q)
-        if (q == qk) ok = o[q];
-      const T xk = __shfl_sync(0xffffffffu, ok, k & 31) * dinv[k];
-#pragma unroll
-      for (int q = 0; q < RPL; ++q) {
-        const int j = lane + 32 * q;
-        if (j == k) o[q] = xk;
-        else if (j < k) o[q] -= Lm[(size_t)k * Bm + j] * xk;
-      }
+      for (int q = 0; q < RPL; ++q) cur[u][q] = nxt[u][q];
     }
   }
 #pragma unroll
   for (int q = 0; q < RPL; ++q) {
-    int i = lane + 32 * q;
-    if (i < m) vj[i] = (V)o[q];
+    const int i = lane + 32 * q;
+    if (i < m) {
+      v0[i] = (V)o[0][q];
+      if (NR > 1) v1[i] = (V)o[NR - 1][q];
+    }
+  }
+}
+
+template <typename T, typename V, int RPL, int CH, int NR>
+__device__ __forceinline__ void leaf_warp_modes(const T* __restrict__ Lm, const T* __restrict__ dinv, int Bm, int m,
+                                                V* v0, V* v1, int mode, int lane) {
+  switch (mode) {
+    case 0: leaf_warp_chunks<T, V, RPL, CH, 0, NR>(Lm, dinv, Bm, m, v0, v1, lane); break;
+    case 1: leaf_warp_chunks<T, V, RPL, CH, 1, NR>(Lm, dinv, Bm, m, v0, v1, lane); break;
+    case 2: leaf_warp_chunks<T, V, RPL, CH, 2, NR>(Lm, dinv, Bm, m, v0, v1, lane); break;
+    default: leaf_warp_chunks<T, V, RPL, CH, 3, NR>(Lm, dinv, Bm, m, v0, v1, lane); break;
   }
 }
 
@@ -250,12 +273,15 @@ __device__ __forceinline__ void leaf_warp_apply32(const T* __restrict__ Lm, cons
   }
 }
 
-template <typename T, typename V>
+// Leaves of any size, NR right-hand sides.
+template <typename T, typename V, int NR>
 __device__ __forceinline__ void leaf_warp_apply(const T* __restrict__ Lm, const T* __restrict__ dinv, int Bm, int m,
-                                                V* vj, int mode, int lane) {
-  if (Bm <= 32) leaf_warp_apply_r<T, V, 1>(Lm, dinv, Bm, m, vj, mode, lane);
-  else if (Bm <= 64) leaf_warp_apply_r<T, V, 2>(Lm, dinv, Bm, m, vj, mode, lane);
-  else leaf_warp_apply_r<T, V, FIFA_LEAF_MAX / 32>(Lm, dinv, Bm, m, vj, mode, lane);
+                                                V* v0, V* v1, int mode, int lane) {
+  if (Bm <= 32) leaf_warp_apply32<T, V>(Lm, dinv, Bm, m, v0, NR > 1 ? v1 : nullptr, mode, lane);
+  else if (Bm <= 64) leaf_warp_modes<T, V, 2, 2, NR>(Lm, dinv, Bm, m, v0, v1, mode, lane);
+  else  // one at a time: registers
+    for (int j = 0; j < NR; ++j)
+      leaf_warp_modes<T, V, FIFA_LEAF_MAX / 32, 1, 1>(Lm, dinv, Bm, m, j ? v1 : v0, nullptr, mode, lane);
 }
 
 // Leaf step over all leaves: one warp per leaf.
@@ -271,12 +297,8 @@ __global__ void __launch_bounds__(256) k_sweep_leaf(const FactDesc* __restrict__
   const int s = Fd->bnd[bnd_off(L) + warp], e = Fd->bnd[bnd_off(L) + warp + 1];
   const T* Lm = (const T*)Fd->Lleaf + (size_t)warp * Bm * Bm;
   const T* dinv = (const T*)Fd->Ldinv + (size_t)warp * Bm;
-  if (Bm <= 32) {
-    leaf_warp_apply32<T, double>(Lm, dinv, Bm, e - s, v + s, nrhs > 1 ? v + n + s : nullptr,
-                                                           mode, lane);
-    return;
-  }
-  for (int j = 0; j < nrhs; ++j) leaf_warp_apply<T, double>(Lm, dinv, Bm, e - s, v + (size_t)j * n + s, mode, lane);
+  if (nrhs > 1) leaf_warp_apply<T, double, 2>(Lm, dinv, Bm, e - s, v + s, v + n + s, mode, lane);
+  else leaf_warp_apply<T, double, 1>(Lm, dinv, Bm, e - s, v + s, nullptr, mode, lane);
 }
 
 // ---------------------------------------------------------------------------
@@ -285,12 +307,25 @@ __global__ void __launch_bounds__(256) k_sweep_leaf(const FactDesc* __restrict__
 // keeps v on them in shared memory for the whole sweep, so v crosses HBM once
 // each way.  The leaves and every level >= ls act inside one CTA (a node there
 // lies in one CTA's rows); each level < ls exchanges one partial projection
-// per CTA through `part` (two buffers alternating by level) around one grid
-// barrier.  Same arithmetic as the per-level kernels above:
-//   p = [Q_left^T v_left ; Q_right^T v_right],  t = op(Z) p,  v += Q t.
+// per CTA through `part` (its own slots for every level).  Same arithmetic as
+// the per-level kernels above:
+//   p = [Q_left^T v_left ; Q_right^T v_right],  t = op(Z) p,  v += Q t,
+// without its zeros: Z = [0 0; K Y] (the capacitance's factor is [I 0; M^T L2]),
+// so t is zero on the left side for Z, and Z^T takes p from the right side
+// alone.  A CTA left of the split hands over its partial and goes on; the right
+// ones wait for the CTAs of their own node only (a counter per node).
+//
+// What bounds it: up to n ~ 2^17 the chain of levels < ls (a barrier of the
+// whole grid and loads behind it cost ~17 us per level; now ~4), beyond that
+// the FP64 pipe.  So a level's basis rows and its block of Z are copied to
+// shared memory while the level before runs (as far as FS_QBUF holds them), and
+// sums go over lanes that share an output, not over one thread's chain: a lone
+// warp takes 64 cycles per FP64 instruction.
 // ---------------------------------------------------------------------------
 #define FS_WARPS 8
-#define FS_K (2 * FIFA_CAP_MAX * SW_RHS_MAX)  // stride of one CTA's partial in `part`
+#define FS_QBUF 1536        // entries of a level's basis rows staged ahead
+#define FS_QROWS 512        // CTAs of more rows stage nothing (their levels are long)
+#define FS_ZBUF 512         // doubles of a level's Z block staged ahead: 2 r^2, r <= 16
 
 // Ask L2 to fetch the 128-byte line holding p (no data is returned; p must
 // point into an allocation).
@@ -366,6 +401,8 @@ struct FsShared {
   T* pj;                  // FS_BUF: projections p of a batch of nodes
   T* tv;                  // FS_BUF: t = op(Z) p of the batch
   T* red;                 // 256 reduction partials
+  double* zb;             // 2 x FS_ZBUF: staged blocks of Z
+  T* qb;                  // 2 x FS_QBUF: staged basis rows (null: none)
   unsigned short* lmap;   // rows: local leaf of each row
 };
 
@@ -410,13 +447,14 @@ __device__ void fs_local_level(const FactDesc* __restrict__ Fd, int l, int ls, i
   int rmax = 0;
   for (int q = 0; q < nsub; ++q) rmax = max(rmax, Fd->rank[node_id(l, i0 + q)]);
   if (rmax == 0) return;
-  const int per = 2 * rmax * nrhs;  // entries per node: (side, a, j)
-  const int nb = max(1, FS_BUF / per);
+  // Z: p of both sides, t of the right one; Z^T: p of the right side, t of both
+  const int half = rmax * nrhs, np = zt ? half : 2 * half, ntt = zt ? 2 * half : half;  // entries per node
+  const int nb = max(1, FS_BUF / (2 * half));
   for (int b0 = 0; b0 < nsub; b0 += nb) {
     const int bn = min(nb, nsub - b0);
-    tile_dots<T, T>(bn * per, Qb, n, vs, rows, S,
+    tile_dots<T, T>(bn * np, Qb, n, vs, rows, S,
                     [&](int o, int& a0, int& a1, int& col, int& j) {
-                      const int node = o / per, rem = o % per, side = rem / (rmax * nrhs), aj = rem % (rmax * nrhs);
+                      const int node = o / np, rem = o % np, side = zt ? 1 : rem / half, aj = rem % half;
                       const int a = aj / nrhs;
                       j = aj % nrhs;
                       int s0, h0, e0;
@@ -426,19 +464,20 @@ __device__ void fs_local_level(const FactDesc* __restrict__ Fd, int l, int ls, i
                       col = a < Fd->rank[node_id(l, i0 + b0 + node)] ? a : -1;
                     },
                     sh.red, sh.pj);
-    for (int k = threadIdx.x; k < bn * per; k += blockDim.x) {
-      const int node = k / per, rem = k % per, sa = rem / nrhs, j = rem % nrhs;
-      const int side = sa / rmax, a = sa % rmax;
+    for (int k = threadIdx.x; k < bn * ntt; k += blockDim.x) {
+      const int node = k / ntt, rem = k % ntt, j = rem % nrhs;
+      const int side = zt ? rem / half : 1, a = (rem % half) / nrhs;
       const int nid = node_id(l, i0 + b0 + node);
       const int r = Fd->rank[nid];
       T acc = (T)0;
       if (a < r) {
         const double* Z = (zsel ? Fd->Zi : Fd->Zf) + (size_t)nid * ld2 * ld2;
-        const int row = side * r + a;
-        const T* pn = sh.pj + node * per;
-        for (int bb = 0; bb < 2 * r; ++bb) {
-          const int bs = bb >= r ? 1 : 0, ba = bb - bs * r;
-          acc += (T)(zt ? Z[bb * ld2 + row] : Z[row * ld2 + bb]) * pn[(bs * rmax + ba) * nrhs + j];
+        const T* pn = sh.pj + node * np;
+        if (zt) {
+          for (int b = 0; b < r; ++b) acc += (T)Z[(r + b) * ld2 + side * r + a] * pn[b * nrhs + j];
+        } else {
+          for (int b = 0; b < r; ++b) acc += (T)Z[(r + a) * ld2 + b] * pn[b * nrhs + j];
+          for (int b = 0; b < r; ++b) acc += (T)Z[(r + a) * ld2 + r + b] * pn[half + b * nrhs + j];
         }
       }
       sh.tv[k] = acc;
@@ -451,7 +490,8 @@ __device__ void fs_local_level(const FactDesc* __restrict__ Fd, int l, int ls, i
       const int r = Fd->rank[node_id(l, gi)];
       int s0, h0, e0;
       node_range(bnd, l, gi, s0, h0, e0);
-      const T* tn = sh.tv + node * per + (p < h0 ? 0 : rmax) * nrhs;
+      if (!zt && p < h0) continue;
+      const T* tn = sh.tv + node * ntt + (zt && p >= h0 ? half : 0);
       // the products accumulate onto v itself (no separate add per row)
       T acc0 = vs[p - S], acc1 = nrhs > 1 ? vs[rows + p - S] : (T)0;
       fs_row_update<T, NR>(Qb, n, p, r, tn, acc0, acc1);
@@ -462,120 +502,177 @@ __device__ void fs_local_level(const FactDesc* __restrict__ Fd, int l, int ls, i
   }
 }
 
+// Asynchronous copies into shared memory.
+__device__ __forceinline__ void fs_copy(double* dst, const double* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void fs_copy(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+
+// Start copying what level l < ls needs besides v into buffer b: the CTA's rows
+// of its r basis columns and rows r .. 2r of the node's Z (one group of copies,
+// empty if they do not fit).
+template <typename T>
+__device__ void fs_stage(const FactDesc* __restrict__ Fd, int l, int ls, int c, int r, int S, int R, int zsel, int b,
+                         FsShared<T>& sh) {
+  if (sh.qb && r * R <= FS_QBUF && 2 * r * r <= FS_ZBUF) {
+    const int cap = Fd->cap, ld2 = 2 * cap;
+    const int64_t n = Fd->n;
+    const T* Qb = (const T*)Fd->Q + (size_t)l * cap * n + S;
+    const double* Z = (zsel ? Fd->Zi : Fd->Zf) + (size_t)node_id(l, c >> (ls - l)) * ld2 * ld2;
+    for (int t = threadIdx.x; t < r * R; t += blockDim.x) {
+      const int a = t / R, p = t - a * R;
+      fs_copy(sh.qb + b * FS_QBUF + t, Qb + (size_t)a * n + p);
+    }
+    for (int t = threadIdx.x; t < 2 * r * r; t += blockDim.x) {
+      const int a = t / (2 * r), q = t - a * 2 * r;
+      fs_copy(sh.zb + b * FS_ZBUF + t, Z + (size_t)(r + a) * ld2 + q);
+    }
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// Sum over a power of two of neighbouring lanes; every one of them gets it.
+template <typename T>
+__device__ __forceinline__ T lanes_sum(T v, int width) {
+  for (int o = width >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+// Lanes per output when K outputs share 256 threads: a power of two, 1 .. 32.
+__device__ __forceinline__ int lanes_for(int K) {
+  int w = 32;
+  while (w > 1 && w * K > 256) w >>= 1;
+  return w;
+}
+
 // One level < ls: node i = c >> (ls - l) spans 2^(ls - l) CTAs; c's rows lie in
-// one child (side).  The CTAs exchange their partial projections in FP64
-// (`part`).  Returns false if the grid barrier gave up.
+// one child (side).  The CTAs hand over their partial projections in FP64
+// (`part`, this level's slots) and count themselves in at their node's counter.
+// What the level needs is in buffer `buf` (fs_stage, the oldest group of
+// copies) or still in global memory.  Returns false if the wait gave up.
 template <typename T, int NR>
-__device__ bool fs_global_level(const FactDesc* __restrict__ Fd, int l, int ls, int c, T* vs, int rows, int S,
-                                int E, int zsel, int zt, double* __restrict__ part, int buf,
-                                unsigned int* bar, unsigned int& phase, int* abort_flag, FsShared<T>& sh,
-                                int lnext) {
+__device__ bool fs_global_level(const FactDesc* __restrict__ Fd, int l, int ls, int c, int r, T* vs, int rows, int S,
+                                int E, int zsel, int zt, double* __restrict__ part, int buf, unsigned int* counter,
+                                int* abort_flag, FsShared<T>& sh) {
   constexpr int nrhs = NR;
-  constexpr int RG = FS_RG_OF(T);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int C = gridDim.x;
-  const int cap = Fd->cap, ld2 = 2 * cap;
+  const int tid = threadIdx.x, R = E - S;
+  const int cap = Fd->cap, ld2 = 2 * cap, pstr = cap * SW_RHS_MAX;
   const int64_t n = Fd->n;
-  const int span = ls - l, i = c >> span, side = (c >> (span - 1)) & 1;
+  const int span = ls - l, i = c >> span, side = (c >> (span - 1)) & 1, half = 1 << (span - 1), c0 = i << span;
   const int nid = node_id(l, i);
-  const int r = Fd->rank[nid];
+  const bool staged = sh.qb && r * R <= FS_QBUF && 2 * r * r <= FS_ZBUF;
+  asm volatile("cp.async.wait_group 1;" ::: "memory");  // this level's copies; the next level's may be in flight
+  __syncthreads();                                       // ... every thread's, and v is up to date
+  if (r == 0) return true;                               // (for every CTA of the node: none waits)
   const T* Qb = (const T*)Fd->Q + (size_t)l * cap * n;
-  double* mine = part + ((size_t)buf * C + c) * FS_K;
-  // partial projection of this CTA's rows onto its side's r columns: every
-  // thread takes rows p = S + tid + 256 i and RG columns at a time (their
-  // loads issued together), then a fixed-order block reduction
-  for (int a0 = 0; a0 < r; a0 += RG) {
-    T acc0[RG], acc1[RG];
-#pragma unroll
-    for (int u = 0; u < RG; ++u) acc0[u] = acc1[u] = (T)0;
-#pragma unroll 2
-    for (int p = S + (int)threadIdx.x; p < E; p += blockDim.x) {
-      const T v0 = vs[p - S], v1 = nrhs > 1 ? vs[rows + p - S] : (T)0;
-      T q[RG];
-#pragma unroll
-      for (int u = 0; u < RG; ++u) q[u] = a0 + u < r ? Qb[(size_t)(a0 + u) * n + p] : (T)0;
-#pragma unroll
-      for (int u = 0; u < RG; ++u) {
-        if (a0 + u < r) {  // uniform over the CTA: no arithmetic on the columns past the rank
-          acc0[u] += q[u] * v0;
-          if (nrhs > 1) acc1[u] += q[u] * v1;
-        }
+  const T* q = staged ? sh.qb + buf * FS_QBUF : Qb + S;  // column a at q + a * qs, from row S
+  const size_t qs = staged ? (size_t)R : (size_t)n;
+  const double* Z = staged ? sh.zb + buf * FS_ZBUF
+                           : (zsel ? Fd->Zi : Fd->Zf) + (size_t)nid * ld2 * ld2 + (size_t)r * ld2;
+  const int zs = staged ? 2 * r : ld2;  // row a of Z's lower half at Z + a * zs
+  const int K = r * nrhs;
+  if (!zt || side) {
+    // this CTA's partial p: neighbouring lanes share an output, rows striding
+    const int w = lanes_for(K), ch = tid & (w - 1);
+    for (int o0 = 0; o0 < K; o0 += 256 / w) {
+      const int o = o0 + tid / w, a = o / nrhs, j = o % nrhs;
+      T acc = (T)0;
+      if (o < K) {
+        const T* qa = q + (size_t)a * qs;
+        const T* vj = vs + (size_t)j * rows;
+#pragma unroll 4
+        for (int p = ch; p < R; p += w) acc += qa[p] * vj[p];
       }
-    }
-#pragma unroll
-    for (int u = 0; u < RG; ++u) {
-      if (a0 + u < r) {  // uniform: no reduction for the columns past the rank
-        acc0[u] = warp_sum_t(acc0[u]);
-        if (nrhs > 1) acc1[u] = warp_sum_t(acc1[u]);
-      }
-    }
-    if (lane == 0)
-#pragma unroll
-      for (int u = 0; u < RG; ++u) {
-        sh.red[(warp * RG + u) * 2] = acc0[u];
-        sh.red[(warp * RG + u) * 2 + 1] = acc1[u];
-      }
-    __syncthreads();
-    if ((int)threadIdx.x < RG * nrhs) {
-      const int u = threadIdx.x / nrhs, j = threadIdx.x % nrhs;
-      if (a0 + u < r) {
-        T t = (T)0;
-        for (int w = 0; w < FS_WARPS; ++w) t += sh.red[(w * RG + u) * 2 + j];
-        __stcg(mine + (a0 + u) * nrhs + j, (double)t);
-      }
+      acc = lanes_sum(acc, w);
+      if (ch == 0 && o < K) __stcg(part + (size_t)c * pstr + o, (double)acc);
     }
     __syncthreads();
+    if (tid == 0) {
+      __threadfence();
+      atomicAdd(counter, 1u);
+    }
   }
-  (void)lane;
-  if (sizeof(T) == 4 && lnext >= 0)  // FP32: the next level's basis rows, fetched into L2 while the grid waits
-    prefetch_cols_l2<T>((const T*)Fd->Q + (size_t)lnext * cap * n, n, Fd->rank[node_id(lnext, c >> (ls - lnext))], S,
-                        E);
-  ++phase;
-  if (!group_barrier(bar, (unsigned)C * phase, Fd->status, abort_flag, Fd->spin)) return false;
-  if (r == 0) return true;
-  // p over the node: the left half of its CTAs for rows of the left child, the
-  // right half for the right child, summed in a fixed order
-  const int K = 2 * r * nrhs, half = 1 << (span - 1), c0 = i << span;
-  const int nch = blockDim.x / K;
-  T* red = sh.red;
-  if ((int)threadIdx.x < nch * K) {
-    const int k = threadIdx.x % K, ch = threadIdx.x / K;
-    const int sd = (k / nrhs) >= r ? 1 : 0, kk = k - sd * r * nrhs;
-    const double* src = part + ((size_t)buf * C + c0 + sd * half) * FS_K + kk;
-    double acc = 0.0;
-    for (int q = ch; q < half; q += nch) acc += __ldcg(src + (size_t)q * FS_K);
-    red[ch * K + k] = (T)acc;
-  }
-  __syncthreads();
-  if ((int)threadIdx.x < K) {
-    T acc = (T)0;
-    for (int ch = 0; ch < nch; ++ch) acc += red[ch * K + threadIdx.x];
-    sh.pj[threadIdx.x] = acc;
-  }
-  __syncthreads();
-  if ((int)threadIdx.x < K) {
-    const int a = threadIdx.x / nrhs, j = threadIdx.x % nrhs;
-    const double* Z = (zsel ? Fd->Zi : Fd->Zf) + (size_t)nid * ld2 * ld2;
-    T acc = (T)0;
-    for (int b = 0; b < 2 * r; ++b) acc += (T)(zt ? Z[b * ld2 + a] : Z[a * ld2 + b]) * sh.pj[b * nrhs + j];
-    sh.tv[threadIdx.x] = acc;
+  if (!zt && !side) return true;  // the left rows keep their values
+  // wait for the CTAs that hand over: both halves, or the right one
+  __shared__ int arrived;
+  if (tid == 0) {
+    const unsigned int target = zt ? half : 2 * half;
+    const unsigned int limit = Fd->spin ? Fd->spin : FIFA_SPIN_LIMIT;
+    unsigned int spins = 0;
+    int ok = 1;
+    while (*((volatile unsigned int*)counter) < target) {
+      if (*((volatile int*)abort_flag)) {
+        ok = 0;
+        break;
+      }
+      if (++spins > limit) {
+        atomicOr(Fd->status, FIFA_DEV_TIMEOUT);
+        *((volatile int*)abort_flag) = 1;
+        ok = 0;
+        break;
+      }
+      if (spins > 256) __nanosleep(64);
+    }
+    __threadfence();
+    arrived = ok;
   }
   __syncthreads();
-  const int off = side * r;
+  if (!arrived) return false;
+  // p (left entries, then right ones; right ones alone for Z^T)
+  {
+    const int K2 = zt ? K : 2 * K, w = lanes_for(K2), ch = tid & (w - 1);
+    for (int o0 = 0; o0 < K2; o0 += 256 / w) {
+      const int o = o0 + tid / w;
+      double acc = 0.0;
+      if (o < K2) {
+        const int sd = zt ? 1 : o / K, k = o - (zt ? 0 : sd * K);
+        const double* src = part + (size_t)(c0 + sd * half) * pstr + k;
+#pragma unroll 4
+        for (int g = ch; g < half; g += w) acc += __ldcg(src + (size_t)g * pstr);
+      }
+      acc = lanes_sum(acc, w);
+      if (ch == 0 && o < K2) sh.pj[o] = (T)acc;
+    }
+  }
+  __syncthreads();
+  // t on this CTA's side
+  {
+    const int w = lanes_for(K), ch = tid & (w - 1), terms = zt ? r : 2 * r;
+    for (int o0 = 0; o0 < K; o0 += 256 / w) {
+      const int o = o0 + tid / w, a = o / nrhs, j = o % nrhs;
+      T acc = (T)0;
+      if (o < K)
+        for (int b = ch; b < terms; b += w)
+          acc += (T)(zt ? Z[b * zs + side * r + a] : Z[a * zs + b]) * sh.pj[b * nrhs + j];
+      acc = lanes_sum(acc, w);
+      if (ch == 0 && o < K) sh.tv[o] = acc;
+    }
+  }
+  __syncthreads();
+  if (staged) {
+    for (int t = tid; t < R * nrhs; t += blockDim.x) {
+      const int j = t >= R ? 1 : 0, p = t - j * R;
+      T acc = vs[(size_t)j * rows + p];
+      for (int a = 0; a < r; ++a) acc += q[a * R + p] * sh.tv[a * nrhs + j];
+      vs[(size_t)j * rows + p] = acc;
+    }
+  } else {
 #pragma unroll 2
-  for (int p = S + (int)threadIdx.x; p < E; p += blockDim.x) {
-    T acc0 = vs[p - S], acc1 = nrhs > 1 ? vs[rows + p - S] : (T)0;
-    fs_row_update<T, NR>(Qb, n, p, r, sh.tv + off * nrhs, acc0, acc1);
-    vs[p - S] = acc0;
-    if (nrhs > 1) vs[rows + p - S] = acc1;
+    for (int p = S + tid; p < E; p += blockDim.x) {
+      T acc0 = vs[p - S], acc1 = nrhs > 1 ? vs[rows + p - S] : (T)0;
+      fs_row_update<T, NR>(Qb, n, p, r, sh.tv, acc0, acc1);
+      vs[p - S] = acc0;
+      if (nrhs > 1) vs[rows + p - S] = acc1;
+    }
   }
-  __syncthreads();
   return true;
 }
 
 template <typename T, int NR>
 __device__ void fs_leaves(const FactDesc* __restrict__ Fd, int ls, int c, T* vs, int rows, int S, int mode) {
-  constexpr int nrhs = NR;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int L = Fd->L, Bm = Fd->Bm;
   const int nl = 1 << (L - ls), first = c << (L - ls);
@@ -584,13 +681,7 @@ __device__ void fs_leaves(const FactDesc* __restrict__ Fd, int ls, int c, T* vs,
     const int s = Fd->bnd[bnd_off(L) + leaf], e = Fd->bnd[bnd_off(L) + leaf + 1];
     const T* Lm = (const T*)Fd->Lleaf + (size_t)leaf * Bm * Bm;
     const T* dinv = (const T*)Fd->Ldinv + (size_t)leaf * Bm;
-    if (Bm <= 32) {
-      leaf_warp_apply32<T, T>(Lm, dinv, Bm, e - s, vs + (s - S),
-                                                        nrhs > 1 ? vs + rows + (s - S) : nullptr, mode, lane);
-      continue;
-    }
-    for (int j = 0; j < nrhs; ++j)
-      leaf_warp_apply<T, T>(Lm, dinv, Bm, e - s, vs + (size_t)j * rows + (s - S), mode, lane);
+    leaf_warp_apply<T, T, NR>(Lm, dinv, Bm, e - s, vs + (s - S), vs + rows + (s - S), mode, lane);
   }
   __syncthreads();
 }
@@ -622,15 +713,16 @@ __device__ __forceinline__ T warp_allsum(T v) {
 }
 
 // t = op(Z) p for a node of rank r: lane k < 2 r nrhs computes t[k]
-// (k = (row, j)); p and t interleaved by right-hand side.
+// (k = (row, j)); p and t interleaved by right-hand side.  Z's upper half is
+// zero: t of the right side alone for Z, p of the right side alone for Z^T.
 template <typename T, int NR>
 __device__ __forceinline__ void fw_apply_z(const double* __restrict__ Z, int ld2, int r, int zt, const T* pw, T* tw,
                                            int lane) {
   constexpr int nrhs = NR;
-  if (lane < 2 * r * nrhs) {
+  if (lane < 2 * r * nrhs && (zt || lane >= r * nrhs)) {
     const int row = lane / nrhs, j = lane % nrhs;
     T acc = (T)0;
-    for (int b = 0; b < 2 * r; ++b) acc += (T)(zt ? Z[b * ld2 + row] : Z[row * ld2 + b]) * pw[b * nrhs + j];
+    for (int b = zt ? r : 0; b < 2 * r; ++b) acc += (T)(zt ? Z[b * ld2 + row] : Z[row * ld2 + b]) * pw[b * nrhs + j];
     tw[lane] = acc;
   }
   __syncwarp();
@@ -700,11 +792,11 @@ __device__ void fw_node(const FactDesc* __restrict__ Fd, int l, int i, T* vs, in
   int s0, h0, e0;
   node_range(Fd->bnd, l, i, s0, h0, e0);
   const T* Qb = (const T*)Fd->Q + (size_t)l * cap * n;
-  fw_project<T, NR>(Qb, n, r, vs, rows, S, s0, h0, pw, lane);
+  if (!zt) fw_project<T, NR>(Qb, n, r, vs, rows, S, s0, h0, pw, lane);
   fw_project<T, NR>(Qb, n, r, vs, rows, S, h0, e0, pw + r * NR, lane);
   __syncwarp();
   fw_apply_z<T, NR>((zsel ? Fd->Zi : Fd->Zf) + (size_t)nid * ld2 * ld2, ld2, r, zt, pw, tw, lane);
-  fw_update<T, NR>(Qb, n, r, vs, rows, S, s0, h0, tw, 0);
+  if (zt) fw_update<T, NR>(Qb, n, r, vs, rows, S, s0, h0, tw, 0);
   fw_update<T, NR>(Qb, n, r, vs, rows, S, h0, e0, tw, r);
   __syncwarp();
 }
@@ -723,11 +815,7 @@ __device__ void fw_subtree(const FactDesc* __restrict__ Fd, int lw, int wi, T* v
       const int s = Fd->bnd[bnd_off(L) + leaf], e = Fd->bnd[bnd_off(L) + leaf + 1];
       const T* Lm = (const T*)Fd->Lleaf + (size_t)leaf * Bm * Bm;
       const T* dinv = (const T*)Fd->Ldinv + (size_t)leaf * Bm;
-      if (Bm <= 32)
-        leaf_warp_apply32<T, T>(Lm, dinv, Bm, e - s, vs + (s - S), NR > 1 ? vs + rows + (s - S) : nullptr, mode,
-                                lane);
-      else
-        for (int j = 0; j < NR; ++j) leaf_warp_apply<T, T>(Lm, dinv, Bm, e - s, vs + (size_t)j * rows + (s - S), mode, lane);
+      leaf_warp_apply<T, T, NR>(Lm, dinv, Bm, e - s, vs + (s - S), vs + rows + (s - S), mode, lane);
       __syncwarp();
     }
   };
@@ -758,16 +846,16 @@ __device__ void fw_block_level(const FactDesc* __restrict__ Fd, int l, int lw, i
   const int nid = node_id(l, i);
   const int r = Fd->rank[nid];
   const T* Qb = (const T*)Fd->Q + (size_t)l * cap * n;
-  if (own && r > 0) {
+  const int side = (wi >> (span - 1)) & 1;
+  if (own && r > 0 && (!zt || side)) {
     const int a0 = Fd->bnd[bnd_off(lw) + wi], a1 = Fd->bnd[bnd_off(lw) + wi + 1];
     fw_project<T, NR>(Qb, n, r, vs, rows, S, a0, a1, part + warp * FS_WSL, lane);
   }
   __syncthreads();
-  if (!own || r == 0) return;
+  if (!own || r == 0 || (!zt && !side)) return;
   // warps of node i: [i << span, (i + 1) << span) - c nsub, left half first
   const int w0 = (i << span) - c * nsub, half = 1 << (span - 1);
-  const int side = (wi >> (span - 1)) & 1;
-  if (lane < 2 * r * nrhs) {
+  if (lane < 2 * r * nrhs && (!zt || lane >= r * nrhs)) {
     const int sd = lane / (r * nrhs), k = lane % (r * nrhs);
     T acc = (T)0;
     for (int q = 0; q < half; ++q) acc += part[(w0 + sd * half + q) * FS_WSL + k];
@@ -813,7 +901,9 @@ __global__ void __launch_bounds__(256, 4) k_sweep_fused(const FactDesc* __restri
   sh.pj = vs + (size_t)rows * nrhs;
   sh.tv = sh.pj + FS_BUF;
   sh.red = sh.tv + FS_BUF;
-  sh.lmap = (unsigned short*)(sh.red + 256);
+  sh.zb = (double*)(((uintptr_t)(sh.red + 256) + 7) & ~(uintptr_t)7);
+  sh.qb = rows <= FS_QROWS ? (T*)(sh.zb + 2 * FS_ZBUF) : nullptr;
+  sh.lmap = (unsigned short*)(sh.qb ? sh.qb + 2 * FS_QBUF : (T*)sh.zb);
   const int c = blockIdx.x;
   const int L = Fd->L;
   const int64_t n = Fd->n;
@@ -822,7 +912,9 @@ __global__ void __launch_bounds__(256, 4) k_sweep_fused(const FactDesc* __restri
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int lw = min(L, ls + FS_WL), nsub = 1 << (lw - ls);
   __shared__ int rk_big;
+  __shared__ int rkg[FIFA_LEVELS_MAX];  // this CTA's node's rank at each level < ls
   if (threadIdx.x == 0) rk_big = 0;
+  if ((int)threadIdx.x < ls) rkg[threadIdx.x] = Fd->rank[node_id(threadIdx.x, c >> (ls - threadIdx.x))];
   for (int j = 0; j < nrhs; ++j)
     for (int p = threadIdx.x; p < E - S; p += blockDim.x) vs[(size_t)j * rows + p] = (T)v[(size_t)j * n + S + p];
   __syncthreads();
@@ -852,7 +944,6 @@ __global__ void __launch_bounds__(256, 4) k_sweep_fused(const FactDesc* __restri
     }
     __syncthreads();
   }
-  unsigned int phase = 0;
   bool ok = true;
   T* pw = sh.pj + warp * 2 * FS_WSL;  // p of the warp's node
   T* tw = pw + FS_WSL;                // t of the warp's node
@@ -886,42 +977,64 @@ __global__ void __launch_bounds__(256, 4) k_sweep_fused(const FactDesc* __restri
       __syncthreads();
     }
   };
+  // the levels < ls of one sweep (pass 0, or 1 for the second of mode 4) upward
+  // or downward; the first one's basis rows are on their way before
+  const int pstr = Fd->cap * SW_RHS_MAX;
+  int buf = 0;
+  auto first_level = [&](bool upward, int zsel) {
+    const int l = upward ? ls - 1 : 0;
+    if (ls > 0) fs_stage(Fd, l, ls, c, rkg[l], S, E - S, zsel, buf, sh);
+  };
+  auto global_levels = [&](bool upward, int zsel, int zt, int pass) {
+    for (int q = 0; q < ls && ok; ++q) {
+      const int l = upward ? ls - 1 - q : q, ln = upward ? l - 1 : l + 1;
+      // the next level's copies go where the level before this one was read
+      // (every thread has passed a barrier since)
+      __syncthreads();
+      if (q + 1 < ls) fs_stage(Fd, ln, ls, c, rkg[ln], S, E - S, zsel, buf ^ 1, sh);
+      else asm volatile("cp.async.commit_group;" ::: "memory");
+      ok = fs_global_level<T, NR>(Fd, l, ls, c, rkg[l], vs, rows, S, E, zsel, zt,
+                                  part + (size_t)(pass * ls + l) * gridDim.x * pstr, buf,
+                                  bar + FS_BAR_COUNTERS + (pass << ls) + node_id(l, c >> (ls - l)), abort_flag, sh);
+      buf ^= 1;
+    }
+    __syncthreads();
+  };
   auto up = [&](int md) {  // leaves first, then the levels upward (W^-1, W^T)
     const int zsel = md == 1 ? 1 : 0, zt = md == 2 ? 1 : 0;
+    first_level(true, zsel);
     local_up(md, zsel, zt);
-    for (int l = ls - 1; l >= 0 && ok; --l)
-      ok = fs_global_level<T, NR>(Fd, l, ls, c, vs, rows, S, E, zsel, zt, part, phase & 1, bar, phase, abort_flag,
-                              sh, l - 1);
+    global_levels(true, zsel, zt, 0);
   };
-  auto down = [&](int md) {  // the levels downward, then the leaves (W, W^-T)
+  auto down = [&](int md, int pass) {  // the levels downward, then the leaves (W, W^-T)
     const int zsel = md == 3 ? 1 : 0, zt = md == 3 ? 1 : 0;
-    for (int l = 0; l < ls && ok; ++l)
-      ok = fs_global_level<T, NR>(Fd, l, ls, c, vs, rows, S, E, zsel, zt, part, phase & 1, bar, phase, abort_flag,
-                              sh, l + 1 < ls ? l + 1 : -1);
+    first_level(false, zsel);
+    global_levels(false, zsel, zt, pass);
     if (ok) local_down(md, zsel, zt);
   };
   if (mode == 1 || mode == 2) {
     up(mode);
-  } else if (mode == 5) {  // W^-1's leaves and levels >= ls only (no grid barrier)
+  } else if (mode == 5) {  // W^-1's leaves and levels >= ls only (no CTA waits)
     local_up(1, 1, 0);
   } else if (mode == 6) {  // W^-1's levels < ls only, on v that mode 5 left
-    for (int l = ls - 1; l >= 0 && ok; --l)
-      ok = fs_global_level<T, NR>(Fd, l, ls, c, vs, rows, S, E, 1, 0, part, phase & 1, bar, phase, abort_flag, sh,
-                                  l - 1);
+    first_level(true, 1);
+    global_levels(true, 1, 0, 0);
   } else if (mode == 4) {
     up(1);
-    if (ok) down(3);
+    if (ok) down(3, 1);
   } else {
-    down(mode);
+    down(mode, 0);
   }
-  if (!ok) return;  // the status word carries TIMEOUT; v is left as it was
+  if (!ok) return;  // the status word carries TIMEOUT; v is incomplete
   for (int j = 0; j < nrhs; ++j)
     for (int p = threadIdx.x; p < E - S; p += blockDim.x) v[(size_t)j * n + S + p] = (double)vs[(size_t)j * rows + p];
 }
 
 size_t sweep_fused_smem(int rows, int nrhs, int prec) {
   const size_t esz = prec ? sizeof(float) : sizeof(double);
-  return esz * ((size_t)rows * nrhs + 2 * FS_BUF + 256) + sizeof(unsigned short) * (size_t)rows;
+  return esz * ((size_t)rows * nrhs + 2 * FS_BUF + 256) + 8 +
+         (rows <= FS_QROWS ? 2 * FS_ZBUF * sizeof(double) + 2 * FS_QBUF * esz : 0) +
+         sizeof(unsigned short) * (size_t)rows;
 }
 
 template <typename T, int NR, bool BATCH = false>

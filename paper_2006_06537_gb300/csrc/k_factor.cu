@@ -758,8 +758,9 @@ __global__ void __launch_bounds__(256, 2)
     for (int t = threadIdx.x; t < r2 * r2; t += blockDim.x) {
       const int a = t / r2, b = t % r2;
       const double dd = (a == b) ? 1.0 : 0.0;
-      Zf[a * ld2 + b] = (a >= b ? Sm[b * r2 + a] : 0.0) - dd;
-      Zi[a * ld2 + b] = (a >= b ? Sim[b * r2 + a] : 0.0) - dd;
+      // (the upper half of L_S and its inverse is [I 0])
+      Zf[a * ld2 + b] = a < r ? 0.0 : (a >= b ? Sm[b * r2 + a] : 0.0) - dd;
+      Zi[a * ld2 + b] = a < r ? 0.0 : (a >= b ? Sim[b * r2 + a] : 0.0) - dd;
     }
     if (threadIdx.x == 0) {
       Fd->ld_parts[nleaf + nid] = ls;
@@ -799,8 +800,8 @@ __global__ void __launch_bounds__(256, 2)
     }
     __syncthreads();
     for (int a = threadIdx.x; a < r2; a += blockDim.x) {
-      Zf[a * ld2 + a] -= 1.0;
-      Zi[a * ld2 + a] -= 1.0;
+      Zf[a * ld2 + a] = a < r ? 0.0 : Zf[a * ld2 + a] - 1.0;  // (the upper half is [I 0])
+      Zi[a * ld2 + a] = a < r ? 0.0 : Zi[a * ld2 + a] - 1.0;
     }
     if (threadIdx.x == 0) {
       Fd->ld_parts[nleaf + nid] = ls;
