@@ -83,6 +83,11 @@ cudaError_t launch_mv_fused(const HmatDesc* Hd, int ls, int rows, const double* 
 cudaError_t launch_mv_fused_batched(const HmatDesc* Hd, int ls, int rows, const double* const* xlist,
                                     double* const* ylist, int nprob, double* part, unsigned int* bar, int* abort_flag,
                                     size_t pstride, cudaStream_t st);
+// Posterior mean (mu, alpha nullable together) and variance at nstar new inputs,
+// one CTA each; only where predict_many(n, nstar).
+bool predict_many(int64_t n, int64_t nstar);
+cudaError_t launch_predict(const HmatDesc* Hd, const FactDesc* Fd, int64_t n, const double* x, const double* xstar,
+                           int64_t nstar, const double* alpha, double tau2, double* mu, double* var, cudaStream_t st);
 cudaError_t launch_sweep_leaf(const FactDesc* Fd, int prec, int nleaf, double* v, int nrhs, int mode, cudaStream_t st,
                               const int* active = nullptr);
 cudaError_t launch_matvec(const HmatDesc* Hd, int nleaf, int L, const double* x, int nrhs, double* part, double* proj,

@@ -1115,6 +1115,84 @@ cudaError_t launch_sweep_fused(const FactDesc* Fd, int prec, int ls, int rows, i
 }
 
 // ---------------------------------------------------------------------------
+// Posterior at many new inputs: one CTA per new input x*_j takes its whole
+// cross-kernel column c through the sweep W^-1 alone (the fused sweep with the
+// root's rows in one CTA's shared memory, so no CTA waits on another), and the
+// column never leaves the SM:  mu_j = c . alpha (both nullable),
+// var_j = tau2 (1 - |W^-1 c|^2).
+// Bound by the FP64 pipe: per row one kernel entry, half a leaf's products and
+// three per basis column; two CTAs per SM fill it.  n = 10000 (leaves of 39
+// rows), 301 inputs: one two-column sweep of the whole GPU per two inputs, with
+// five launches, took 14.5 ms.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(256, 2)
+    k_predict(const HmatDesc* __restrict__ Hd, const FactDesc* __restrict__ Fd, const double* __restrict__ x,
+              const double* __restrict__ xstar, int64_t nstar, const double* __restrict__ alpha, double tau2,
+              double* __restrict__ mu, double* __restrict__ var) {
+  extern __shared__ __align__(16) unsigned char fs_smem[];
+  __shared__ double red[40];
+  const int n = (int)Fd->n, L = Fd->L, nleaf = Fd->nleaf;
+  double* vs = (double*)fs_smem;
+  FsShared<double> sh;
+  sh.pj = vs + n;
+  sh.tv = sh.pj + FS_BUF;
+  sh.red = sh.tv + FS_BUF;
+  sh.zb = nullptr;
+  sh.qb = nullptr;
+  sh.lmap = (unsigned short*)(sh.red + 256);
+  for (int q = threadIdx.x; q < nleaf; q += blockDim.x) {
+    const int s0 = Fd->bnd[bnd_off(L) + q], e0 = Fd->bnd[bnd_off(L) + q + 1];
+    for (int p = s0; p < e0; ++p) sh.lmap[p] = (unsigned short)q;
+  }
+  const double kc = Hd->kc;
+  const int kind = Hd->kind;
+  for (int64_t j = blockIdx.x; j < nstar; j += gridDim.x) {
+    const double xj = xstar[j];
+    double acc = 0.0;
+    for (int p = threadIdx.x; p < n; p += blockDim.x) {
+      const double c = kern_entry(kind, kc, xj, x[p]);
+      vs[p] = c;
+      if (mu) acc += c * alpha[p];
+    }
+    if (mu) {
+      acc = block_sum(acc, red);
+      if (threadIdx.x == 0) mu[j] = acc;
+    }
+    __syncthreads();
+    fs_leaves<double, 1>(Fd, 0, 0, vs, n, 0, 1);
+    for (int l = L - 1; l >= 0; --l) fs_local_level<double, 1>(Fd, l, 0, 0, vs, n, 0, n, 1, 0, sh);
+    double q = 0.0;
+    for (int p = threadIdx.x; p < n; p += blockDim.x) q += vs[p] * vs[p];
+    q = block_sum(q, red);
+    if (threadIdx.x == 0) var[j] = tau2 * (1.0 - q);
+  }
+}
+
+static size_t predict_smem(int64_t n) {
+  return sizeof(double) * ((size_t)n + 2 * FS_BUF + 256) + sizeof(unsigned short) * (size_t)n;
+}
+
+// Whether k_predict takes n training and nstar new inputs: the column fits one
+// SM's shared memory, and there are enough new inputs to make up for one CTA's
+// sweep being slower than the whole GPU's (one sweep of n = 10000 by one CTA
+// costs about as much as 40 inputs by two-column launches).
+bool predict_many(int64_t n, int64_t nstar) {
+  int dev = 0, optin = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  return predict_smem(n) + 1024 <= (size_t)optin && nstar >= std::max<int64_t>(8, n / 256);
+}
+
+cudaError_t launch_predict(const HmatDesc* Hd, const FactDesc* Fd, int64_t n, const double* x, const double* xstar,
+                           int64_t nstar, const double* alpha, double tau2, double* mu, double* var, cudaStream_t st) {
+  const size_t smem = predict_smem(n);
+  cudaError_t e = cudaFuncSetAttribute(k_predict, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k_predict<<<(unsigned)std::min<int64_t>(nstar, 1 << 20), 256, smem, st>>>(Hd, Fd, x, xstar, nstar, alpha, tau2, mu, var);
+  return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------
 // Fused H-matrix product y = scale (C~ x) + shift x in one cooperative launch
 // of 2^ls CTAs (the fused sweep's decomposition).  CTA c owns the rows [S, E)
 // of level-ls node c: x on them sits in shared memory and each thread keeps

@@ -8,7 +8,10 @@
 //   k_pred_mean : one CTA per new input, a fixed-order block sum over the n
 //                 training inputs of c(x*_j, x_i) alpha_i (alpha = C~^-1 f).
 //   k_pred_cols : the cross-kernel columns of two new inputs at a time, then
-//                 one W_C^-1 sweep for both and their squared norms.
+//                 one W_C^-1 sweep for both and their squared norms (few new
+//                 inputs, or n beyond one SM's shared memory);
+//   k_predict   : (k_apply.cu) otherwise one CTA per new input takes its column
+//                 through the whole sweep.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -74,6 +77,14 @@ extern "C" fifa_status fifa_predict(fifa_ctx* ctx, const fifa_hmat* C, const fif
   cudaStream_t s = ctx->stream;
   double* alpha = S.vec;     // n: C~^-1 f
   double* cols = S.vec + n;  // 2n: cross-kernel columns, then W_C^-1 of them
+  if (var_dev && predict_many(n, nstar)) {  // both from one pass over each new input's column
+    if (mu_dev) {
+      CK(cudaMemcpyAsync(alpha, f_dev, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
+      if ((st = sweep_enqueue_desc(ctx, P, WC->dev, 0, 4, alpha, 1)) != FIFA_OK) return st;  // W^-T W^-1 f
+    }
+    CK(launch_predict(C->dev, WC->dev, n, x_dev, xstar_dev, nstar, mu_dev ? alpha : nullptr, tau2, mu_dev, var_dev, s));
+    return FIFA_OK;
+  }
   if (mu_dev) {
     CK(cudaMemcpyAsync(alpha, f_dev, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
     if ((st = sweep_enqueue_desc(ctx, P, WC->dev, 0, 4, alpha, 1)) != FIFA_OK) return st;  // W^-T W^-1 f
