@@ -1087,6 +1087,7 @@ fifa_status solve_enqueue(fifa_ctx* ctx, const fifa_fact* F, const double* b, do
   int* act = ints;        // act[2]
   int* iters = ints + 2;  // iterations taken
   int* act_sw = ints + 3; // this step's preconditioner needed
+  int* count = ints + 4;  // blocks that have finished an update
   double* r = work;
   double* z = work + nn;
   double* p = work + 2 * nn;
@@ -1098,13 +1099,13 @@ fifa_status solve_enqueue(fifa_ctx* ctx, const fifa_fact* F, const double* b, do
   if ((e = matvec_enqueue(ctx, op, x, r, nrhs)) != FIFA_OK) return e;
   CK(launch_pcg_residual0(b, r, z, n, nrhs, part, s));  // r = b - A x0, z = r
   if ((e = sweep_enqueue_desc(ctx, P, F->dev32, 1, 4, z, nrhs)) != FIFA_OK) return e;
-  CK(launch_pcg_start(r, z, p, n, nrhs, part, st, act, iters, tol2, s));
+  CK(launch_pcg_start(r, z, p, n, nrhs, part, st, act, iters, count, tol2, s));
   const int slot = PCG_RHS_MAX * PCG_SLOT;
   for (int it = 0; it < ctx->opts.refine_max; ++it) {
     const int cur = it & 1, nxt = cur ^ 1;
     if ((e = matvec_enqueue(ctx, op, p, q, nrhs, act + cur)) != FIFA_OK) return e;
     CK(launch_pcg_pq(p, q, n, nrhs, part, act + cur, s));
-    CK(launch_pcg_update(x, r, z, p, q, n, nrhs, st + cur * slot, part, act + cur, act_sw, tol2, s));
+    CK(launch_pcg_update(x, r, z, p, q, n, nrhs, st + cur * slot, part, act + cur, act_sw, count, tol2, s));
     if ((e = sweep_enqueue_desc(ctx, P, F->dev32, 1, 4, z, nrhs, act_sw)) != FIFA_OK) return e;
     CK(launch_pcg_direction(r, p, z, n, nrhs, st + cur * slot, st + nxt * slot, act + cur, act + nxt, iters, part,
                             tol2, s));

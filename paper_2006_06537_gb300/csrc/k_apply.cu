@@ -531,6 +531,8 @@ __device__ void fs_stage(const FactDesc* __restrict__ Fd, int l, int ls, int c, 
       const int a = t / (2 * r), q = t - a * 2 * r;
       fs_copy(sh.zb + b * FS_ZBUF + t, Z + (size_t)(r + a) * ld2 + q);
     }
+  } else if (sizeof(T) == 4) {  // FP32 levels are memory-bound: into L2 at least
+    prefetch_cols_l2<T>((const T*)Fd->Q + (size_t)l * Fd->cap * Fd->n, Fd->n, r, S, S + R);
   }
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
@@ -575,19 +577,26 @@ __device__ bool fs_global_level(const FactDesc* __restrict__ Fd, int l, int ls, 
   const int zs = staged ? 2 * r : ld2;  // row a of Z's lower half at Z + a * zs
   const int K = r * nrhs;
   if (!zt || side) {
-    // this CTA's partial p: neighbouring lanes share an output, rows striding
-    const int w = lanes_for(K), ch = tid & (w - 1);
-    for (int o0 = 0; o0 < K; o0 += 256 / w) {
-      const int o = o0 + tid / w, a = o / nrhs, j = o % nrhs;
-      T acc = (T)0;
-      if (o < K) {
+    // this CTA's partial p: neighbouring lanes share a column, rows striding
+    const int w = lanes_for(r), ch = tid & (w - 1);
+    for (int o0 = 0; o0 < r; o0 += 256 / w) {
+      const int a = o0 + tid / w;
+      T acc0 = (T)0, acc1 = (T)0;
+      if (a < r) {
         const T* qa = q + (size_t)a * qs;
-        const T* vj = vs + (size_t)j * rows;
 #pragma unroll 4
-        for (int p = ch; p < R; p += w) acc += qa[p] * vj[p];
+        for (int p = ch; p < R; p += w) {
+          const T qv = qa[p];
+          acc0 += qv * vs[p];
+          if (nrhs > 1) acc1 += qv * vs[rows + p];
+        }
       }
-      acc = lanes_sum(acc, w);
-      if (ch == 0 && o < K) __stcg(part + (size_t)c * pstr + o, (double)acc);
+      acc0 = lanes_sum(acc0, w);
+      if (nrhs > 1) acc1 = lanes_sum(acc1, w);
+      if (ch == 0 && a < r) {
+        __stcg(part + (size_t)c * pstr + a * nrhs, (double)acc0);
+        if (nrhs > 1) __stcg(part + (size_t)c * pstr + a * nrhs + 1, (double)acc1);
+      }
     }
     __syncthreads();
     if (tid == 0) {

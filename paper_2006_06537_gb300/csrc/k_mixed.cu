@@ -72,11 +72,38 @@ cudaError_t launch_demote(const FactDesc* F64, const FactDesc* F32, int64_t n, c
 // ---------------------------------------------------------------------------
 #define PCG_PART(w, j) (((w) * 2 + (j)) * PCG_NB)
 
+// Sum of one set of partials, by a whole warp (every lane gets it; the same
+// order in every warp): 4 + 5 additions per lane instead of a chain of PCG_NB,
+// at 64 cycles each for a warp (a direction step of n = 65537 spent 34 us on
+// such chains).
 __device__ __forceinline__ double pcg_sum(const double* __restrict__ part, int w, int j) {
-  // every block adds the same partials in the same order
-  double v = 0.0;
-  for (int b = 0; b < PCG_NB; ++b) v += __ldcg(part + PCG_PART(w, j) + b);
+  const double* src = part + PCG_PART(w, j);
+  const int lane = threadIdx.x & 31;
+  double a[(PCG_NB + 31) / 32];
+#pragma unroll
+  for (int u = 0; u < (PCG_NB + 31) / 32; ++u) a[u] = lane + 32 * u < PCG_NB ? __ldcg(src + lane + 32 * u) : 0.0;
+  double v = a[0];
+#pragma unroll
+  for (int u = 1; u < (PCG_NB + 31) / 32; ++u) v += a[u];
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
+}
+
+// Whether this block is the last of `blocks` to get here; what the others wrote
+// before is then visible to it.  The counter is left at zero for the next use.
+__device__ __forceinline__ bool pcg_last_block(int* counter, int blocks) {
+  __shared__ int last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(counter, 1) == blocks - 1;
+    if (last) {
+      *counter = 0;
+      __threadfence();
+    }
+  }
+  __syncthreads();
+  return last != 0;
 }
 
 // r = b - r (r holds M~ x on entry), z = r; partials of r^T r and b^T b.
@@ -120,25 +147,30 @@ __global__ void __launch_bounds__(256) k_pcg_start(const double* __restrict__ r,
 
 // Slot 0 from the first residual (one block).
 __global__ void k_pcg_init(double* __restrict__ st, int* __restrict__ act, int* __restrict__ iters,
-                           const double* __restrict__ part, int nrhs, double tol2) {
-  if (threadIdx.x != 0) return;
+                           int* __restrict__ counter, const double* __restrict__ part, int nrhs, double tol2) {
+  const bool one = threadIdx.x == 0;  // (a warp: pcg_sum takes all of it)
+  if (one) *counter = 0;
   int any = 0;
   for (int j = 0; j < PCG_RHS_MAX; ++j) {
     double* s = st + j * PCG_SLOT;
     if (j >= nrhs) {
-      s[0] = 0.0; s[1] = 0.0; s[2] = 1.0; s[3] = 0.0;
+      if (one) { s[0] = 0.0; s[1] = 0.0; s[2] = 1.0; s[3] = 0.0; }
       continue;
     }
     const double rr = pcg_sum(part, 0, j), bb = pcg_sum(part, 1, j), rz = pcg_sum(part, 2, j);
     const bool done = !(rr > tol2 * bb) || !(rz > 0.0) || !isfinite(rz);
-    s[0] = rz;
-    s[1] = bb;
-    s[2] = done ? 1.0 : 0.0;
-    s[3] = rr;
+    if (one) {
+      s[0] = rz;
+      s[1] = bb;
+      s[2] = done ? 1.0 : 0.0;
+      s[3] = rr;
+    }
     any |= done ? 0 : 1;
   }
-  act[0] = any;
-  *iters = 0;
+  if (one) {
+    act[0] = any;
+    *iters = 0;
+  }
 }
 
 // Partials of p^T q (after q = M~ p).
@@ -162,11 +194,19 @@ __device__ __forceinline__ double pcg_alpha(const double* __restrict__ s, const 
 }
 
 // alpha = rho / p^T q; x += alpha p; r -= alpha q; z = r; partials of r^T r.
+// The last block then decides whether the preconditioner must run this step:
+// some system still iterating whose updated residual is above the tolerance.  A
+// system that has just met it is marked done by k_pcg_dir from the same r^T r,
+// so its z is never used and the sweep is skipped when no other system needs it.
 __global__ void __launch_bounds__(256) k_pcg_xr(double* __restrict__ x, double* __restrict__ r, double* __restrict__ z,
                                                const double* __restrict__ p, const double* __restrict__ q, int64_t n,
                                                const double* __restrict__ st, double* __restrict__ part,
-                                               const int* __restrict__ active) {
-  if (*active == 0) return;
+                                               const int* __restrict__ active, int* __restrict__ act_sweep,
+                                               int* __restrict__ counter, int nrhs, double tol2) {
+  if (*active == 0) {
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *act_sweep = 0;
+    return;
+  }
   const int j = blockIdx.y;
   const double a = pcg_alpha(st + j * PCG_SLOT, part, j);
   double rr = 0.0;
@@ -184,24 +224,15 @@ __global__ void __launch_bounds__(256) k_pcg_xr(double* __restrict__ x, double* 
   __shared__ double red[40];
   rr = block_sum(rr, red);
   if (threadIdx.x == 0) __stcg(part + PCG_PART(0, j) + blockIdx.x, rr);
-}
-
-// Whether the preconditioner must run this step: some system still iterating
-// whose updated residual is above the tolerance.  A system that has just met it
-// is marked done by k_pcg_dir from the same r^T r, so its z is never used and
-// the sweep is skipped when no other system needs it (one block).
-__global__ void k_pcg_gate(const double* __restrict__ st, const double* __restrict__ part,
-                           const int* __restrict__ active, int* __restrict__ act_sweep, int nrhs, double tol2) {
-  if (threadIdx.x != 0) return;
+  if (!pcg_last_block(counter, gridDim.x * gridDim.y) || threadIdx.x >= 32) return;
   int any = 0;
-  if (*active != 0)
-    for (int j = 0; j < nrhs; ++j) {
-      const double* s = st + j * PCG_SLOT;
-      if (s[2] != 0.0) continue;
-      const double rr = pcg_sum(part, 0, j);
-      if (pcg_alpha(s, part, j) != 0.0 && rr > tol2 * s[1]) any = 1;
-    }
-  *act_sweep = any;
+  for (int k = 0; k < nrhs; ++k) {
+    const double* s = st + k * PCG_SLOT;
+    if (s[2] != 0.0) continue;
+    const double r2 = pcg_sum(part, 0, k);
+    if (pcg_alpha(s, part, k) != 0.0 && r2 > tol2 * s[1]) any = 1;
+  }
+  if (threadIdx.x == 0) *act_sweep = any;
 }
 
 // Partials of r^T z (after z = P^-1 r).
@@ -227,23 +258,28 @@ __global__ void __launch_bounds__(256) k_pcg_dir(double* __restrict__ p, const d
                                                 double tol2) {
   const int j = blockIdx.y;
   const bool on = *act_cur != 0;
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 32) {
+    const bool one = threadIdx.x == 0;
     int any = 0;
     for (int k = 0; k < PCG_RHS_MAX; ++k) {
       const double* s = st_cur + k * PCG_SLOT;
       double* t = st_nxt + k * PCG_SLOT;
-      t[0] = s[0]; t[1] = s[1]; t[2] = s[2]; t[3] = s[3];
+      if (one) { t[0] = s[0]; t[1] = s[1]; t[2] = s[2]; t[3] = s[3]; }
       if (!on || k >= nrhs || s[2] != 0.0) continue;
       const double a = pcg_alpha(s, part, k);
       const double rr = pcg_sum(part, 0, k), rz = pcg_sum(part, 2, k);
       const bool done = a == 0.0 || !(rr > tol2 * s[1]) || !(rz > 0.0) || !isfinite(rz);
-      t[0] = rz;
-      t[2] = done ? 1.0 : 0.0;
-      t[3] = rr;
+      if (one) {
+        t[0] = rz;
+        t[2] = done ? 1.0 : 0.0;
+        t[3] = rr;
+      }
       any |= done ? 0 : 1;
     }
-    *act_nxt = any;
-    if (on) *iters += 1;
+    if (one) {
+      *act_nxt = any;
+      if (on) *iters += 1;
+    }
   }
   if (!on || j >= nrhs) return;
   const double* s = st_cur + j * PCG_SLOT;
@@ -278,13 +314,13 @@ __global__ void __launch_bounds__(256) k_pcg_true(const double* __restrict__ b, 
 
 __global__ void k_pcg_res(const double* __restrict__ part, int nrhs, double* __restrict__ res,
                           const int* __restrict__ iters, int* __restrict__ iters_out) {
-  if (threadIdx.x != 0) return;
   double m = 0.0;
   for (int j = 0; j < nrhs; ++j) {
     const double d = pcg_sum(part, 0, j), bb = pcg_sum(part, 1, j);
     const double v = bb > 0.0 ? sqrt(d / bb) : sqrt(d);
     m = fmax(m, v);
   }
+  if (threadIdx.x != 0) return;
   if (res) *res = m;
   if (iters_out) *iters_out = *iters;
 }
@@ -310,9 +346,9 @@ cudaError_t launch_pcg_residual0(const double* b, double* r, double* z, int64_t 
   return cudaGetLastError();
 }
 cudaError_t launch_pcg_start(const double* r, const double* z, double* p, int64_t n, int nrhs, double* part,
-                             double* stt, int* act, int* iters, double tol2, cudaStream_t st) {
+                             double* stt, int* act, int* iters, int* counter, double tol2, cudaStream_t st) {
   k_pcg_start<<<dim3(PCG_NB, nrhs), 256, 0, st>>>(r, z, p, n, part);
-  k_pcg_init<<<1, 32, 0, st>>>(stt, act, iters, part, nrhs, tol2);
+  k_pcg_init<<<1, 32, 0, st>>>(stt, act, iters, counter, part, nrhs, tol2);
   return cudaGetLastError();
 }
 cudaError_t launch_pcg_pq(const double* p, const double* q, int64_t n, int nrhs, double* part, const int* active,
@@ -321,10 +357,9 @@ cudaError_t launch_pcg_pq(const double* p, const double* q, int64_t n, int nrhs,
   return cudaGetLastError();
 }
 cudaError_t launch_pcg_update(double* x, double* r, double* z, const double* p, const double* q, int64_t n, int nrhs,
-                              const double* stt, double* part, const int* active, int* act_sweep, double tol2,
-                              cudaStream_t st) {
-  k_pcg_xr<<<dim3(PCG_NB, nrhs), 256, 0, st>>>(x, r, z, p, q, n, stt, part, active);
-  k_pcg_gate<<<1, 32, 0, st>>>(stt, part, active, act_sweep, nrhs, tol2);
+                              const double* stt, double* part, const int* active, int* act_sweep, int* counter,
+                              double tol2, cudaStream_t st) {
+  k_pcg_xr<<<dim3(PCG_NB, nrhs), 256, 0, st>>>(x, r, z, p, q, n, stt, part, active, act_sweep, counter, nrhs, tol2);
   return cudaGetLastError();
 }
 cudaError_t launch_pcg_direction(const double* r, double* p, const double* z, int64_t n, int nrhs,
