@@ -281,18 +281,32 @@ extern "C" fifa_status fifa_plan_describe(const fifa_opts* opts, int64_t n, int 
   return FIFA_OK;
 }
 
+// Most CTAs of a fused sweep or product: below n = 2^18 their time is the chain
+// of levels that cross CTAs, each a hand-over between them whose partial sums
+// grow with their number, so fewer CTAs with more rows are faster as long as
+// they fill the GPU; from 2^18 on the FP64 pipe wants them all.  W^-1 v / W^-T W^-1
+// v (two vectors) / C~ v at 2^7, 2^8, 2^9 CTAs: n = 20011 64/72/89, 134/154/202,
+// 43/37/40 us; n = 65537 114/111/127, 250/250/299, 70/65/78 us; n = 131072 (Matern)
+// 203/160/167, 500/460/486, 153/111/111 us; n = 300007 388/299/275, 861/644/630,
+// 262/176/145 us; n = 8192 at 2^6, 2^7, 2^8: 59/58/66, 114/111/137, 35/29/31 us.
+static int fused_ctas(int64_t n, int small) {
+  if (n >= (int64_t)1 << 18) return FS_CTAS_MAX;
+  const int64_t most = n < 32768 ? small : 256;
+  return (int)std::max<int64_t>(1, std::min<int64_t>(most, n < 64 * 32 ? 32 : n / 64));
+}
+
 Plan* get_plan(fifa_ctx* ctx, int64_t n, fifa_status* st) {
   auto key = std::make_pair(n, ctx->opts.leaf_size);
   auto it = ctx->plans.find(key);
   if (it != ctx->plans.end()) return it->second;
   Plan* P = plan_build(n, ctx->opts, ctx->aca_coresident, ctx->level_coresident, st);
   if (!P) return nullptr;
-  // fused sweep: the largest power-of-two grid (<= nleaf, FS_CTAS_MAX) whose
+  // fused sweep: the largest power-of-two grid (<= nleaf, fused_ctas) whose
   // CTAs, each holding the longest level-k node in shared memory, are all
   // co-resident (for both factor precisions)
   if (!ctx->opts.independent_ctas) {
     for (int k = std::min(P->L, 10); k >= 0; --k) {
-      if ((1 << k) > FS_CTAS_MAX) continue;
+      if ((1 << k) > fused_ctas(n, 128)) continue;
       int rows = 0;
       for (int i = 0; i < (1 << k); ++i)
         rows = std::max(rows, P->bnd_host[bnd_off(k) + i + 1] - P->bnd_host[bnd_off(k) + i]);
@@ -307,6 +321,7 @@ Plan* get_plan(fifa_ctx* ctx, int64_t n, fifa_status* st) {
     }
     // fused H-matvec: the same kind of grid, rows per CTA <= MV_FUSED_ROWS_MAX
     for (int k = std::min(P->L, 10); k >= 0; --k) {
+      if ((1 << k) > fused_ctas(n, 256)) continue;
       int rows = 0;
       for (int i = 0; i < (1 << k); ++i)
         rows = std::max(rows, P->bnd_host[bnd_off(k) + i + 1] - P->bnd_host[bnd_off(k) + i]);
@@ -1045,10 +1060,8 @@ fifa_status matvec_enqueue(fifa_ctx* ctx, const fifa_hmat* A, const double* in, 
   Plan* P = A->plan;
   Scratch S = carve(ctx, P);
   if (P->mv_ls >= 0) {
-    CK(cudaMemsetAsync(S.mv_bar, 0, sizeof(unsigned int), ctx->stream));
-    CK(cudaMemsetAsync(S.flags, 0, sizeof(int), ctx->stream));
-    CK(launch_mv_fused(A->dev, P->mv_ls, P->mv_rows, in, nrhs, out, S.mv_fpart, S.mv_bar, S.flags, ctx->stream,
-                       active));
+    CK(cudaMemsetAsync(S.mv_bar, 0, sizeof(unsigned int) * MV_BAR_UINTS, ctx->stream));
+    CK(launch_mv_fused(A->dev, P->mv_ls, P->mv_rows, in, nrhs, out, S.mv_fpart, S.mv_bar, ctx->stream, active));
     return FIFA_OK;
   }
   CK(launch_matvec(A->dev, P->nleaf, P->L, in, nrhs, S.mv_part, S.mv_proj, out, ctx->stream, active));
@@ -1225,9 +1238,8 @@ fifa_status sample_prior_batched(fifa_ctx* ctx, Plan* P, const HmatDesc* C0, con
   ctx->active_scratch = saved;
   fifa_status st = FIFA_OK;
   if (mv_ls >= 0) {  // C~ a for every block in one launch
-    CK(cudaMemset2DAsync(S.mv_bar, sstride, 0, sizeof(unsigned int), nprob, s));
-    CK(cudaMemset2DAsync(S.flags, sstride, 0, sizeof(int), nprob, s));
-    CK(launch_mv_fused_batched(C0, mv_ls, mv_rows, a_list, Ca_list, nprob, S.mv_fpart, S.mv_bar, S.flags, sstride, s));
+    CK(cudaMemset2DAsync(S.mv_bar, sstride, 0, sizeof(unsigned int) * MV_BAR_UINTS, nprob, s));
+    CK(launch_mv_fused_batched(C0, mv_ls, mv_rows, a_list, Ca_list, nprob, S.mv_fpart, S.mv_bar, sstride, s));
   }
   if (sweep_ls >= 0)  // W_C b for every block in one launch
     st = sweep_enqueue_batched(ctx, P, WC0, b_list, nprob, 0, sweep_ls, sweep_rows, scratch0, sstride);

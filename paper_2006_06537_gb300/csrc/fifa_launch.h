@@ -72,17 +72,18 @@ cudaError_t launch_sweep_fused_batched(const FactDesc* Fd, int ls, int rows, dou
                                        int mode, double* part, unsigned int* bar, int* abort_flag, size_t pstride,
                                        cudaStream_t st);
 // Fused H-matrix product (one cooperative launch of 2^ls CTAs, rows <= 4096).
-// part: 2^ls * ls * MV_PART_STRIDE doubles; bar zeroed before.
+// part: 2^ls * ls * MV_PART_STRIDE doubles; bar, zeroed before: abort flag and counter.
 #define MV_FUSED_ROWS_MAX 4096
+#define MV_BAR_UINTS 2
 int mv_fused_coresident(int rows);
 cudaError_t launch_mv_fused(const HmatDesc* Hd, int ls, int rows, const double* x, int nrhs, double* y, double* part,
-                            unsigned int* bar, int* abort_flag, cudaStream_t st, const int* active = nullptr);
+                            unsigned int* bar, cudaStream_t st, const int* active = nullptr);
 // nprob H-matrices of one plan in one launch (one right-hand side each:
-// xlist[q] -> ylist[q]; per-problem partials / barrier / abort flag pstride
+// xlist[q] -> ylist[q]; per-problem partials and abort flag / counter pstride
 // bytes apart)
 cudaError_t launch_mv_fused_batched(const HmatDesc* Hd, int ls, int rows, const double* const* xlist,
-                                    double* const* ylist, int nprob, double* part, unsigned int* bar, int* abort_flag,
-                                    size_t pstride, cudaStream_t st);
+                                    double* const* ylist, int nprob, double* part, unsigned int* bar, size_t pstride,
+                                    cudaStream_t st);
 // Posterior mean (mu, alpha nullable together) and variance at nstar new inputs,
 // one CTA each; only where predict_many(n, nstar).
 bool predict_many(int64_t n, int64_t nstar);

@@ -318,13 +318,15 @@ __global__ void __launch_bounds__(256) k_sweep_leaf(const FactDesc* __restrict__
 // What bounds it: up to n ~ 2^17 the chain of levels < ls (a barrier of the
 // whole grid and loads behind it cost ~17 us per level; now ~4), beyond that
 // the FP64 pipe.  So a level's basis rows and its block of Z are copied to
-// shared memory while the level before runs (as far as FS_QBUF holds them), and
+// shared memory while the level before runs (as far as they fit, fs_qcap), and
 // sums go over lanes that share an output, not over one thread's chain: a lone
 // warp takes 64 cycles per FP64 instruction.
 // ---------------------------------------------------------------------------
 #define FS_WARPS 8
-#define FS_QBUF 1536        // entries of a level's basis rows staged ahead
-#define FS_QROWS 512        // CTAs of more rows stage nothing (their levels are long)
+// Entries of a level's basis rows staged ahead, by the CTA's rows: as many as
+// leave four CTAs to an SM up to 160 rows, two up to 512; CTAs of more rows
+// stage nothing (their levels are long).
+__host__ __device__ inline int fs_qcap(int rows) { return rows <= 160 ? 1536 : (rows <= 512 ? 4608 : 0); }
 #define FS_ZBUF 512         // doubles of a level's Z block staged ahead: 2 r^2, r <= 16
 
 // Ask L2 to fetch the 128-byte line holding p (no data is returned; p must
@@ -402,7 +404,8 @@ struct FsShared {
   T* tv;                  // FS_BUF: t = op(Z) p of the batch
   T* red;                 // 256 reduction partials
   double* zb;             // 2 x FS_ZBUF: staged blocks of Z
-  T* qb;                  // 2 x FS_QBUF: staged basis rows (null: none)
+  T* qb;                  // 2 x qcap: staged basis rows
+  int qcap;               // (0: none)
   unsigned short* lmap;   // rows: local leaf of each row
 };
 
@@ -518,14 +521,14 @@ __device__ __forceinline__ void fs_copy(float* dst, const float* src) {
 template <typename T>
 __device__ void fs_stage(const FactDesc* __restrict__ Fd, int l, int ls, int c, int r, int S, int R, int zsel, int b,
                          FsShared<T>& sh) {
-  if (sh.qb && r * R <= FS_QBUF && 2 * r * r <= FS_ZBUF) {
+  if (r * R <= sh.qcap && 2 * r * r <= FS_ZBUF) {
     const int cap = Fd->cap, ld2 = 2 * cap;
     const int64_t n = Fd->n;
     const T* Qb = (const T*)Fd->Q + (size_t)l * cap * n + S;
     const double* Z = (zsel ? Fd->Zi : Fd->Zf) + (size_t)node_id(l, c >> (ls - l)) * ld2 * ld2;
     for (int t = threadIdx.x; t < r * R; t += blockDim.x) {
       const int a = t / R, p = t - a * R;
-      fs_copy(sh.qb + b * FS_QBUF + t, Qb + (size_t)a * n + p);
+      fs_copy(sh.qb + b * sh.qcap + t, Qb + (size_t)a * n + p);
     }
     for (int t = threadIdx.x; t < 2 * r * r; t += blockDim.x) {
       const int a = t / (2 * r), q = t - a * 2 * r;
@@ -565,12 +568,12 @@ __device__ bool fs_global_level(const FactDesc* __restrict__ Fd, int l, int ls, 
   const int64_t n = Fd->n;
   const int span = ls - l, i = c >> span, side = (c >> (span - 1)) & 1, half = 1 << (span - 1), c0 = i << span;
   const int nid = node_id(l, i);
-  const bool staged = sh.qb && r * R <= FS_QBUF && 2 * r * r <= FS_ZBUF;
+  const bool staged = r * R <= sh.qcap && 2 * r * r <= FS_ZBUF;
   asm volatile("cp.async.wait_group 1;" ::: "memory");  // this level's copies; the next level's may be in flight
   __syncthreads();                                       // ... every thread's, and v is up to date
   if (r == 0) return true;                               // (for every CTA of the node: none waits)
   const T* Qb = (const T*)Fd->Q + (size_t)l * cap * n;
-  const T* q = staged ? sh.qb + buf * FS_QBUF : Qb + S;  // column a at q + a * qs, from row S
+  const T* q = staged ? sh.qb + buf * sh.qcap : Qb + S;  // column a at q + a * qs, from row S
   const size_t qs = staged ? (size_t)R : (size_t)n;
   const double* Z = staged ? sh.zb + buf * FS_ZBUF
                            : (zsel ? Fd->Zi : Fd->Zf) + (size_t)nid * ld2 * ld2 + (size_t)r * ld2;
@@ -584,7 +587,8 @@ __device__ bool fs_global_level(const FactDesc* __restrict__ Fd, int l, int ls, 
       T acc0 = (T)0, acc1 = (T)0;
       if (a < r) {
         const T* qa = q + (size_t)a * qs;
-#pragma unroll 4
+        constexpr int IN_FLIGHT = sizeof(T) == 4 ? 16 : 8;
+#pragma unroll IN_FLIGHT
         for (int p = ch; p < R; p += w) {
           const T qv = qa[p];
           acc0 += qv * vs[p];
@@ -911,8 +915,9 @@ __global__ void __launch_bounds__(256, 4) k_sweep_fused(const FactDesc* __restri
   sh.tv = sh.pj + FS_BUF;
   sh.red = sh.tv + FS_BUF;
   sh.zb = (double*)(((uintptr_t)(sh.red + 256) + 7) & ~(uintptr_t)7);
-  sh.qb = rows <= FS_QROWS ? (T*)(sh.zb + 2 * FS_ZBUF) : nullptr;
-  sh.lmap = (unsigned short*)(sh.qb ? sh.qb + 2 * FS_QBUF : (T*)sh.zb);
+  sh.qcap = fs_qcap(rows);
+  sh.qb = (T*)(sh.zb + (sh.qcap ? 2 * FS_ZBUF : 0));
+  sh.lmap = (unsigned short*)(sh.qb + 2 * sh.qcap);
   const int c = blockIdx.x;
   const int L = Fd->L;
   const int64_t n = Fd->n;
@@ -1042,7 +1047,7 @@ __global__ void __launch_bounds__(256, 4) k_sweep_fused(const FactDesc* __restri
 size_t sweep_fused_smem(int rows, int nrhs, int prec) {
   const size_t esz = prec ? sizeof(float) : sizeof(double);
   return esz * ((size_t)rows * nrhs + 2 * FS_BUF + 256) + 8 +
-         (rows <= FS_QROWS ? 2 * FS_ZBUF * sizeof(double) + 2 * FS_QBUF * esz : 0) +
+         (fs_qcap(rows) ? 2 * FS_ZBUF * sizeof(double) + 2 * fs_qcap(rows) * esz : 0) +
          sizeof(unsigned short) * (size_t)rows;
 }
 
@@ -1148,6 +1153,7 @@ __global__ void __launch_bounds__(256, 2)
   sh.red = sh.tv + FS_BUF;
   sh.zb = nullptr;
   sh.qb = nullptr;
+  sh.qcap = 0;
   sh.lmap = (unsigned short*)(sh.red + 256);
   for (int q = threadIdx.x; q < nleaf; q += blockDim.x) {
     const int s0 = Fd->bnd[bnd_off(L) + q], e0 = Fd->bnd[bnd_off(L) + q + 1];
@@ -1205,28 +1211,46 @@ cudaError_t launch_predict(const HmatDesc* Hd, const FactDesc* Fd, int64_t n, co
 // Fused H-matrix product y = scale (C~ x) + shift x in one cooperative launch
 // of 2^ls CTAs (the fused sweep's decomposition).  CTA c owns the rows [S, E)
 // of level-ls node c: x on them sits in shared memory and each thread keeps
-// the sums for its rows (S + tid + 256 i) in registers.  The leaf blocks and
-// the levels >= ls (whose nodes lie in the CTA) need nothing from other CTAs;
-// each level < ls needs the projection of the partner child, which spans
-// other CTAs: every CTA writes its partial projections for all those levels,
-// passes ONE grid barrier, and sums the partner half's partials.
+// the sums for its rows in registers.  The leaf blocks and the levels >= ls
+// (whose nodes lie in the CTA) need nothing from other CTAs; each level < ls
+// needs the projection of the partner child, which spans other CTAs.  Every CTA
+// hands over its partial projections for all those levels first, works on the
+// leaves and its own levels meanwhile, and then waits once for all CTAs and sums
+// the partner halves' partials.
 //   row p in the left child of a level-l node:  y_p += U_p (V^T x_right)
 //   row p in the right child:                   y_p += V_p (U^T x_left)
 // (U, V share one basis array: row p holds U if p is in the left child.)
+// Bound by the FP64 pipe for large n; for CTAs of few rows by how many threads
+// have work, so `hs` threads share a row (leaf columns and basis columns dealt
+// out between them) when there are at most 160.
 // ---------------------------------------------------------------------------
 #define MV_PROJ_BUF 1024                       // doubles of node projections per batch
 #define MV_PART_STRIDE (FIFA_CAP_MAX * SW_RHS_MAX)  // one CTA's partial of one level
+#define MV_THREADS_MAX 320
+
+// Rows per thread, threads per row (hs) and the distance of a row's threads (rp).
+struct MvShape {
+  int rpt, hs, rp, threads;
+};
+static MvShape mv_shape(int rows) {
+  if (rows <= 64) return {1, 4, 64, 256};
+  if (rows <= 128) return {1, 2, 128, 256};
+  if (rows <= 160) return {1, 2, 160, 320};
+  int rpt = 1;
+  while (rpt * 256 < rows) rpt *= 2;
+  return {rpt, 1, 256, 256};
+}
 
 // BATCH: several H-matrices of one plan in one launch, problem blockIdx.y: its
 // descriptor Hd[blockIdx.y], input xlist[blockIdx.y] and output ylist[...],
-// its partials, barrier and abort flag pstride bytes after the previous
-// problem's (a separate instantiation: re-pointed arguments stay in registers).
+// its partials and its abort flag and counter (bar[0], bar[1], zeroed before)
+// pstride bytes after the previous problem's (a separate instantiation:
+// re-pointed arguments stay in registers).
 template <int RPT, bool BATCH = false>
-__global__ void __launch_bounds__(256, RPT <= 8 ? 4 : 2) k_mv_fused(const HmatDesc* __restrict__ Hd, const double* __restrict__ x, int nrhs,
-                                                  double* __restrict__ y, int ls, int rows, double* __restrict__ part,
-                                                  unsigned int* __restrict__ bar, int* __restrict__ abort_flag,
-                                                  const int* __restrict__ active, const double* const* xlist,
-                                                  double* const* ylist, size_t pstride) {
+__global__ void __launch_bounds__(RPT == 1 ? MV_THREADS_MAX : 256, RPT <= 8 ? 4 : 2)
+    k_mv_fused(const HmatDesc* __restrict__ Hd, const double* __restrict__ x, int nrhs, double* __restrict__ y, int ls,
+               int rows, int hs_arg, int rp, double* __restrict__ part, unsigned int* __restrict__ bar,
+               const int* __restrict__ active, const double* const* xlist, double* const* ylist, size_t pstride) {
   if (active && *active == 0) return;  // a converged iteration: nothing to compute
   if constexpr (BATCH) {
     Hd += blockIdx.y;
@@ -1234,18 +1258,23 @@ __global__ void __launch_bounds__(256, RPT <= 8 ? 4 : 2) k_mv_fused(const HmatDe
     y = ylist[blockIdx.y];
     part = (double*)((char*)part + blockIdx.y * pstride);
     bar = (unsigned int*)((char*)bar + blockIdx.y * pstride);
-    abort_flag = (int*)((char*)abort_flag + blockIdx.y * pstride);
   }
+  const int hs = RPT == 1 ? hs_arg : 1;
   extern __shared__ double sm[];
   double* xs = sm;                                   // nrhs x rows
   double* pj = xs + (size_t)rows * nrhs;             // MV_PROJ_BUF node projections
-  double* red = pj + MV_PROJ_BUF;                    // 256 reduction partials
-  int* lmap = (int*)(red + 256);                     // rows: local leaf of each row
+  double* red = pj + MV_PROJ_BUF;                    // MV_THREADS_MAX reduction partials
+  int* lmap = (int*)(red + MV_THREADS_MAX);          // rows: local leaf of each row
+  __shared__ int rkg[FIFA_LEVELS_MAX];               // rank of this CTA's node at each level < ls
+  __shared__ int arrived;
   const int c = blockIdx.x, C = gridDim.x, tid = threadIdx.x;
   const int L = Hd->L, cap = Hd->cap, Bm = Hd->Bm;
   const int64_t n = Hd->n;
   const int* bnd = Hd->bnd;
   const int S = bnd[bnd_off(ls) + c], E = bnd[bnd_off(ls) + c + 1], R = E - S;
+  const int hsel = RPT == 1 && hs > 1 ? tid / rp : 0;          // which of the row's threads
+  const int row0 = RPT == 1 && hs > 1 ? tid - hsel * rp : tid;  // rows row0 + 256 i
+  if (tid < ls) rkg[tid] = Hd->rank[node_id(tid, c >> (ls - tid))];
   for (int j = 0; j < nrhs; ++j)
     for (int p = tid; p < R; p += blockDim.x) xs[(size_t)j * rows + p] = x[(size_t)j * n + S + p];
   const int nl = 1 << (L - ls), first = c << (L - ls);
@@ -1254,19 +1283,55 @@ __global__ void __launch_bounds__(256, RPT <= 8 ? 4 : 2) k_mv_fused(const HmatDe
     for (int p = s0; p < e0; ++p) lmap[p - S] = q;
   }
   __syncthreads();
+  // levels < ls: partial projections of this CTA's rows, w neighbouring lanes to
+  // a column (few for few rows: a sum over w lanes costs log2 w additions)
+  if (ls > 0) {
+    const int w = R <= 256 ? 8 : (R <= 512 ? 16 : 32), ch = tid & (w - 1), ng = (int)blockDim.x / w;
+    for (int l = 0; l < ls; ++l) {
+      const double* Bl = Hd->bases + (size_t)l * cap * n + S;
+      const int r = rkg[l];
+      for (int a0 = 0; a0 < r; a0 += ng) {
+        const int a = a0 + tid / w;
+        double s0 = 0.0, s1 = 0.0;
+        if (a < r) {
+          const double* b = Bl + (size_t)a * n;
+#pragma unroll 4
+          for (int p = ch; p < R; p += w) {
+            const double bv = b[p];
+            s0 += bv * xs[p];
+            if (nrhs > 1) s1 += bv * xs[rows + p];
+          }
+        }
+        s0 = lanes_sum(s0, w);
+        if (nrhs > 1) s1 = lanes_sum(s1, w);
+        if (ch == 0 && a < r) {
+          double* dst = part + ((size_t)c * ls + l) * MV_PART_STRIDE + a * nrhs;
+          __stcg(dst, s0);
+          if (nrhs > 1) __stcg(dst + 1, s1);
+        }
+      }
+    }
+    __syncthreads();
+    if (tid == 0) {
+      __threadfence();
+      atomicAdd(bar + 1, 1u);
+    }
+  }
   double acc[RPT][SW_RHS_MAX];
 #pragma unroll
   for (int i = 0; i < RPT; ++i) acc[i][0] = acc[i][1] = 0.0;
   // leaf blocks: y_p = sum_k D[p][k] x_k over the leaf of p
 #pragma unroll
   for (int i = 0; i < RPT; ++i) {
-    const int p = S + tid + i * (int)blockDim.x;
+    const int p = S + row0 + i * 256;
     if (p < E) {
       const int q = lmap[p - S], leaf = first + q;
       const int s0 = bnd[bnd_off(L) + leaf], e0 = bnd[bnd_off(L) + leaf + 1];
+      const int per = hs > 1 ? (e0 - s0 + hs - 1) / hs : e0 - s0;  // columns of each of the row's threads
+      const int k0 = s0 + hsel * per, k1 = min(e0, k0 + per);
       const double* D = Hd->leaves + (size_t)leaf * Bm * Bm + (p - s0);
       double a0 = 0.0, a1 = 0.0;
-      for (int k = s0; k < e0; ++k) {
+      for (int k = k0; k < k1; ++k) {
         const double dv = D[(size_t)(k - s0) * Bm];
         a0 += dv * xs[k - S];
         if (nrhs > 1) a1 += dv * xs[rows + k - S];
@@ -1302,7 +1367,7 @@ __global__ void __launch_bounds__(256, RPT <= 8 ? 4 : 2) k_mv_fused(const HmatDe
       // rows of the batch's nodes: y_p += basis_l[p] . proj(partner side)
 #pragma unroll
       for (int i = 0; i < RPT; ++i) {
-        const int p = S + tid + i * (int)blockDim.x;
+        const int p = S + row0 + i * 256;
         if (p < E) {
           const int node = (lmap[p - S] >> (L - l)) - b0;
           if (node >= 0 && node < bn) {
@@ -1313,7 +1378,7 @@ __global__ void __launch_bounds__(256, RPT <= 8 ? 4 : 2) k_mv_fused(const HmatDe
             const int other = p < h0 ? 1 : 0;
             const double* pr = pj + node * per + other * rmax * nrhs;
             double a0 = acc[i][0], a1 = acc[i][1];  // products accumulate onto the row sums
-            for (int cc = 0; cc < r; ++cc) {
+            for (int cc = hsel; cc < r; cc += hs) {
               const double bv = Bl[(size_t)cc * n + p];
               a0 += bv * pr[cc * nrhs];
               if (nrhs > 1) a1 += bv * pr[cc * nrhs + 1];
@@ -1326,68 +1391,99 @@ __global__ void __launch_bounds__(256, RPT <= 8 ? 4 : 2) k_mv_fused(const HmatDe
       __syncthreads();
     }
   }
-  // levels < ls: partial projections of this CTA's rows for every such level
-  for (int l = 0; l < ls; ++l) {
-    const double* Bl = Hd->bases + (size_t)l * cap * n;
-    const int r = Hd->rank[node_id(l, c >> (ls - l))];
-    tile_dots(r * nrhs, Bl, n, xs, rows, S,
-            [&](int o, int& a0, int& a1, int& col, int& j) {
-              a0 = S;
-              a1 = E;
-              col = o / nrhs;
-              j = o % nrhs;
-            },
-            red, pj);
-    for (int k = tid; k < r * nrhs; k += blockDim.x) __stcg(part + ((size_t)c * ls + l) * MV_PART_STRIDE + k, pj[k]);
-    __syncthreads();
-  }
   if (ls > 0) {
-    unsigned int phase = 1;
-    if (!group_barrier(bar, (unsigned)C * phase, Hd->status, abort_flag, Hd->spin)) return;
-  }
-  // levels < ls: the partner half's projection, then the rows' sums
-  for (int l = 0; l < ls; ++l) {
-    const double* Bl = Hd->bases + (size_t)l * cap * n;
-    const int span = ls - l, i = c >> span, side = (c >> (span - 1)) & 1;
-    const int r = Hd->rank[node_id(l, i)];
-    if (r == 0) continue;
-    const int K = r * nrhs, half = 1 << (span - 1);
-    const int c0 = (i << span) + (1 - side) * half;  // first CTA of the partner child
-    const int nch = max(1, (int)blockDim.x / K);
-    if (tid < nch * K) {
-      const int k = tid % K, ch = tid / K;
-      double v = 0.0;
-      for (int q = ch; q < half; q += nch) v += __ldcg(part + ((size_t)(c0 + q) * ls + l) * MV_PART_STRIDE + k);
-      red[ch * K + k] = v;
+    // every CTA's partials are written (a bounded wait; a launch's CTAs are all resident)
+    if (tid == 0) {
+      volatile int* abort_flag = (volatile int*)bar;
+      const unsigned int limit = Hd->spin ? Hd->spin : FIFA_SPIN_LIMIT;
+      unsigned int spins = 0;
+      int ok = 1;
+      while (*((volatile unsigned int*)(bar + 1)) < (unsigned)C) {
+        if (*abort_flag) {
+          ok = 0;
+          break;
+        }
+        if (++spins > limit) {
+          atomicOr(Hd->status, FIFA_DEV_TIMEOUT);
+          *abort_flag = 1;
+          ok = 0;
+          break;
+        }
+        if (spins > 256) __nanosleep(64);
+      }
+      __threadfence();
+      arrived = ok;
     }
     __syncthreads();
-    if (tid < K) {
-      double v = 0.0;
-      for (int ch = 0; ch < nch; ++ch) v += red[ch * K + tid];
-      pj[tid] = v;
+    if (!arrived) return;
+  }
+  // levels < ls, as many at a time as fit pj: the partner halves' projections,
+  // then the rows' sums
+#pragma unroll 1
+  for (int l0 = 0; l0 < ls;) {
+    int l1 = l0, tot = 0;
+    while (l1 < ls && tot + rkg[l1] * nrhs <= MV_PROJ_BUF) tot += rkg[l1++] * nrhs;
+    int off = 0;
+    for (int l = l0; l < l1; ++l) {
+      const int span = ls - l, i = c >> span, side = (c >> (span - 1)) & 1;
+      const int K = rkg[l] * nrhs, half = 1 << (span - 1);
+      const int c0 = (i << span) + (1 - side) * half;  // first CTA of the partner child
+      const int w = min(half, 32), ch = tid & (w - 1), ng = (int)blockDim.x / w;
+      for (int o0 = 0; o0 < K; o0 += ng) {
+        const int k = o0 + tid / w;
+        double v = 0.0;
+        if (k < K) {
+          const double* src = part + ((size_t)c0 * ls + l) * MV_PART_STRIDE + k;
+#pragma unroll 8
+          for (int q = ch; q < half; q += w) v += __ldcg(src + (size_t)q * ls * MV_PART_STRIDE);
+        }
+        v = lanes_sum(v, w);
+        if (ch == 0 && k < K) pj[off + k] = v;
+      }
+      off += K;
     }
     __syncthreads();
 #pragma unroll
     for (int ii = 0; ii < RPT; ++ii) {
-      const int p = S + tid + ii * (int)blockDim.x;
+      const int p = S + row0 + ii * 256;
       if (p < E) {
         double a0 = acc[ii][0], a1 = acc[ii][1];
-        for (int cc = 0; cc < r; ++cc) {
-          const double bv = Bl[(size_t)cc * n + p];
-          a0 += bv * pj[cc * nrhs];
-          if (nrhs > 1) a1 += bv * pj[cc * nrhs + 1];
+        const double* pr = pj;
+        for (int l = l0; l < l1; ++l) {
+          const double* Bl = Hd->bases + (size_t)l * cap * n + p;
+          const int r = rkg[l];
+          for (int cc = hsel; cc < r; cc += hs) {
+            const double bv = Bl[(size_t)cc * n];
+            a0 += bv * pr[cc * nrhs];
+            if (nrhs > 1) a1 += bv * pr[cc * nrhs + 1];
+          }
+          pr += r * nrhs;
         }
         acc[ii][0] = a0;
         acc[ii][1] = a1;
       }
     }
     __syncthreads();
+    l0 = l1;
+  }
+  if (RPT == 1 && hs > 1) {  // the row's threads together, in order
+    if (hsel > 0 && S + row0 < E) {
+      pj[((hsel - 1) * rp + row0) * 2] = acc[0][0];
+      pj[((hsel - 1) * rp + row0) * 2 + 1] = acc[0][1];
+    }
+    __syncthreads();
+    if (hsel > 0) return;
+    if (S + row0 < E)
+      for (int q = 0; q < hs - 1; ++q) {
+        acc[0][0] += pj[(q * rp + row0) * 2];
+        acc[0][1] += pj[(q * rp + row0) * 2 + 1];
+      }
   }
   const double sc = Hd->scale, shf = Hd->shift;
   const double* dg = Hd->diag;
 #pragma unroll
   for (int i = 0; i < RPT; ++i) {
-    const int p = S + tid + i * (int)blockDim.x;
+    const int p = S + row0 + i * 256;
     if (p < E) {
       const bool plain = !dg && shf == 0.0 && sc == 1.0;
       const double sh = dg ? dg[p] : shf;
@@ -1398,7 +1494,7 @@ __global__ void __launch_bounds__(256, RPT <= 8 ? 4 : 2) k_mv_fused(const HmatDe
 }
 
 size_t mv_fused_smem(int rows) {
-  return sizeof(double) * ((size_t)rows * SW_RHS_MAX + MV_PROJ_BUF + 256) + sizeof(int) * (size_t)rows;
+  return sizeof(double) * ((size_t)rows * SW_RHS_MAX + MV_PROJ_BUF + MV_THREADS_MAX) + sizeof(int) * (size_t)rows;
 }
 
 template <int RPT, bool BATCH>
@@ -1409,7 +1505,8 @@ static int mv_fused_per_sm_v(int rows) {
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (smem > (size_t)optin) return 0;
   cudaFuncSetAttribute(k_mv_fused<RPT, BATCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mv_fused<RPT, BATCH>, 256, smem) != cudaSuccess)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mv_fused<RPT, BATCH>, mv_shape(rows).threads, smem) !=
+      cudaSuccess)
     per_sm = 0;
   cudaGetLastError();
   return per_sm;
@@ -1421,17 +1518,11 @@ static int mv_fused_per_sm(int rows) {
   return std::min(mv_fused_per_sm_v<RPT, false>(rows), mv_fused_per_sm_v<RPT, true>(rows));
 }
 
-static int mv_rpt(int rows) {
-  int rpt = 1;
-  while (rpt * 256 < rows) rpt *= 2;
-  return rpt;
-}
-
 int mv_fused_coresident(int rows) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  switch (mv_rpt(rows)) {
+  switch (mv_shape(rows).rpt) {
     case 1: return sms * mv_fused_per_sm<1>(rows);
     case 2: return sms * mv_fused_per_sm<2>(rows);
     case 4: return sms * mv_fused_per_sm<4>(rows);
@@ -1443,14 +1534,15 @@ int mv_fused_coresident(int rows) {
 
 template <int RPT, bool BATCH = false>
 static cudaError_t launch_mv_fused_t(const HmatDesc* Hd, int ls, int rows, const double* x, int nrhs, double* y,
-                                     double* part, unsigned int* bar, int* abort_flag, cudaStream_t st,
-                                     const int* active, const double* const* xlist = nullptr,
-                                     double* const* ylist = nullptr, int nprob = 1, size_t pstride = 0) {
+                                     double* part, unsigned int* bar, cudaStream_t st, const int* active,
+                                     const double* const* xlist = nullptr, double* const* ylist = nullptr,
+                                     int nprob = 1, size_t pstride = 0) {
   const size_t smem = mv_fused_smem(rows);
+  const MvShape sh = mv_shape(rows);
   cudaFuncSetAttribute(k_mv_fused<RPT, BATCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(1u << ls, nprob);
-  cfg.blockDim = dim3(256);
+  cfg.blockDim = dim3(sh.threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
@@ -1458,19 +1550,17 @@ static cudaError_t launch_mv_fused_t(const HmatDesc* Hd, int ls, int rows, const
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_mv_fused<RPT, BATCH>, Hd, x, nrhs, y, ls, rows, part, bar, abort_flag, active,
+  return cudaLaunchKernelEx(&cfg, k_mv_fused<RPT, BATCH>, Hd, x, nrhs, y, ls, rows, sh.hs, sh.rp, part, bar, active,
                             xlist, ylist, pstride);
 }
 
 // nprob H-matrices of one plan (descriptor array Hd), one right-hand side each
 // (xlist[q] -> ylist[q]), in one cooperative launch of 2^ls x nprob CTAs.
 cudaError_t launch_mv_fused_batched(const HmatDesc* Hd, int ls, int rows, const double* const* xlist,
-                                    double* const* ylist, int nprob, double* part, unsigned int* bar, int* abort_flag,
-                                    size_t pstride, cudaStream_t st) {
-#define MVB(R)                                                                                                    \
-  launch_mv_fused_t<R, true>(Hd, ls, rows, nullptr, 1, nullptr, part, bar, abort_flag, st, nullptr, xlist, ylist, \
-                             nprob, pstride)
-  switch (mv_rpt(rows)) {
+                                    double* const* ylist, int nprob, double* part, unsigned int* bar, size_t pstride,
+                                    cudaStream_t st) {
+#define MVB(R) launch_mv_fused_t<R, true>(Hd, ls, rows, nullptr, 1, nullptr, part, bar, st, nullptr, xlist, ylist, nprob, pstride)
+  switch (mv_shape(rows).rpt) {
     case 1: return MVB(1);
     case 2: return MVB(2);
     case 4: return MVB(4);
@@ -1482,13 +1572,13 @@ cudaError_t launch_mv_fused_batched(const HmatDesc* Hd, int ls, int rows, const 
 }
 
 cudaError_t launch_mv_fused(const HmatDesc* Hd, int ls, int rows, const double* x, int nrhs, double* y, double* part,
-                            unsigned int* bar, int* abort_flag, cudaStream_t st, const int* active) {
-  switch (mv_rpt(rows)) {
-    case 1: return launch_mv_fused_t<1>(Hd, ls, rows, x, nrhs, y, part, bar, abort_flag, st, active);
-    case 2: return launch_mv_fused_t<2>(Hd, ls, rows, x, nrhs, y, part, bar, abort_flag, st, active);
-    case 4: return launch_mv_fused_t<4>(Hd, ls, rows, x, nrhs, y, part, bar, abort_flag, st, active);
-    case 8: return launch_mv_fused_t<8>(Hd, ls, rows, x, nrhs, y, part, bar, abort_flag, st, active);
-    case 16: return launch_mv_fused_t<16>(Hd, ls, rows, x, nrhs, y, part, bar, abort_flag, st, active);
+                            unsigned int* bar, cudaStream_t st, const int* active) {
+  switch (mv_shape(rows).rpt) {
+    case 1: return launch_mv_fused_t<1>(Hd, ls, rows, x, nrhs, y, part, bar, st, active);
+    case 2: return launch_mv_fused_t<2>(Hd, ls, rows, x, nrhs, y, part, bar, st, active);
+    case 4: return launch_mv_fused_t<4>(Hd, ls, rows, x, nrhs, y, part, bar, st, active);
+    case 8: return launch_mv_fused_t<8>(Hd, ls, rows, x, nrhs, y, part, bar, st, active);
+    case 16: return launch_mv_fused_t<16>(Hd, ls, rows, x, nrhs, y, part, bar, st, active);
     default: return cudaErrorInvalidValue;
   }
 }
