@@ -99,12 +99,15 @@ __global__ void __launch_bounds__(256, 7)
   load_chunk(0, w0);
   // reciprocals of the pivots: one reciprocal square root per column, products elsewhere
   __shared__ double rinv[FIFA_LEAF_MAX];
-  auto pivot = [&](int k) {  // by one thread
+  auto pivot = [&](int k) {  // by one thread; the diagonal keeps d until the end
     double d = A[k * ld + k];
-    if (!(d > 0.0)) { flag[0] = 1; d = 1.0; }
-    const double rs = rsqrt(d);
-    A[k * ld + k] = d * rs;
-    rinv[k] = rs;
+    const long long bits = __double_as_longlong(d);
+    if (!(bits > 0 && bits <= 0x7ff0000000000000LL)) {  // d > 0, tested on the integer pipe
+      flag[0] = 1;
+      d = 1.0;
+      A[k * ld + k] = d;
+    }
+    rinv[k] = rsqrt_householder(d);
   };
   if (threadIdx.x == 0) flag[0] = 0;
   // column k ready for its step: pivot, column k of L and row k of X scaled
@@ -154,6 +157,8 @@ __global__ void __launch_bounds__(256, 7)
     }
     __syncthreads();
   }
+  for (int k = threadIdx.x; k < m; k += blockDim.x) A[k * ld + k] *= rinv[k];  // sqrt(d) = d / sqrt(d)
+  __syncthreads();
   if (split == 0) {
     double lsum = 0.0;
     for (int k = threadIdx.x; k < m; k += blockDim.x) lsum += log(A[k * ld + k]);
