@@ -86,11 +86,16 @@ static int levels_for(int64_t n, int B) {
   return L;
 }
 
+// Contexts with independent CTAs run the sweeps and products of small problems
+// fused in one cluster (eight CTAs that the hardware schedules together, so no
+// other work can keep one of them waiting) instead of two launches per tree level.
+static bool one_cluster(int64_t n) { return n <= 8192; }
+
 // Partials of the fused sweep: one projection per CTA, level and sweep (a solve
 // has two), for up to min(nleaf, FS_CTAS_MAX) CTAs (none with independent CTAs:
 // no CTA hands anything over).
 static size_t fused_sweep_part_doubles(const Plan* P, const fifa_opts& o) {
-  if (o.independent_ctas) return 1;
+  if (o.independent_ctas && !one_cluster(P->n)) return 1;
   return (size_t)2 * std::max(1, std::min(P->L, 10)) * std::min(P->nleaf, FS_CTAS_MAX) * o.rank_cap * SWEEP_RHS_MAX;
 }
 // Bytes of its abort flag and counters.
@@ -99,7 +104,7 @@ static size_t fused_sweep_bar_bytes(const Plan* P) { return sizeof(unsigned int)
 // Partials of the fused H-matvec: one projection per CTA and level below the
 // CTA level, for up to min(nleaf, FS_CTAS_MAX) CTAs and 10 such levels.
 static size_t fused_mv_part_doubles(const Plan* P, const fifa_opts& o) {
-  if (o.independent_ctas) return 1;
+  if (o.independent_ctas && !one_cluster(P->n)) return 1;
   return (size_t)std::min(P->nleaf, FS_CTAS_MAX) * std::max(1, std::min(P->L, 10)) * FIFA_CAP_MAX * SWEEP_RHS_MAX;
 }
 
@@ -332,6 +337,20 @@ Plan* get_plan(fifa_ctx* ctx, int64_t n, fifa_status* st) {
         break;
       }
     }
+  } else if (one_cluster(n)) {
+    const int k = std::min(P->L, 3);
+    int rows = 0;
+    for (int i = 0; i < (1 << k); ++i)
+      rows = std::max(rows, P->bnd_host[bnd_off(k) + i + 1] - P->bnd_host[bnd_off(k) + i]);
+    if (sweep_fused_coresident(0, rows, ctx->opts.rank_cap) > 0 && sweep_fused_coresident(1, rows, ctx->opts.rank_cap) > 0) {
+      P->fs_ls = k;
+      P->fs_rows = rows;
+    }
+    if (rows <= MV_FUSED_ROWS_MAX && mv_fused_coresident(rows) > 0) {
+      P->mv_ls = k;
+      P->mv_rows = rows;
+    }
+    P->cluster = true;
   }
   char* mem = (char*)ctx->arena.alloc(P->dev_bytes);
   if (!mem) {
@@ -623,6 +642,27 @@ fifa_status hmat_assemble_rest_enqueue(fifa_ctx* ctx, fifa_hmat* H) {
   return FIFA_OK;
 }
 
+// Group sizes for nprob problems' grouped blocks in one launch of at most
+// `cores` CTAs: the plan's, divided.
+static bool aca_groups_for(const Plan* P, int nprob, int cores, AcaGroups* out) {
+  int levels = 0, G[ACA_GROUP_LEVELS];
+  for (int k = 0; k < P->aca_ncoop;) {  // (levels ascending, a level's blocks alike)
+    const int4 w = P->work_host[k];
+    if (levels == ACA_GROUP_LEVELS || w.x != levels) return false;
+    G[levels++] = w.w;
+    k += w.w << w.x;
+  }
+  for (int div = 2; div <= 64; ++div) {
+    int64_t total = 0;
+    for (int l = 0; l < levels; ++l) total += (int64_t)std::max(1, G[l] / div) << l;
+    if (total * nprob > cores) continue;
+    out->levels = levels;
+    for (int l = 0; l < levels; ++l) out->G[l] = std::max(1, G[l] / div);
+    return true;
+  }
+  return false;
+}
+
 fifa_status hmat_assemble_batched(fifa_ctx* ctx, Plan* P, HmatDesc* H0, int nprob, void* scratch0, size_t sstride) {
   void* saved = ctx->active_scratch;
   ctx->active_scratch = scratch0;
@@ -636,6 +676,16 @@ fifa_status hmat_assemble_batched(fifa_ctx* ctx, Plan* P, HmatDesc* H0, int npro
       CK(cudaMemset2DAsync(S.aca_bar, sstride, 0, sizeof(unsigned int) * P->aca_ncoop, nprob, s));
       CK(cudaMemset2DAsync(S.flags, sstride, 0, sizeof(int), nprob, s));
       CK(launch_aca(H0, P->aca_work, P->aca_ncoop, S.aca_part, S.aca_bar, S.flags, s, nprob, sstride));
+    } else if (AcaGroups gr; aca_groups_for(P, nprob, ctx->aca_coresident, &gr)) {
+      // smaller groups, so that all problems' are co-resident: the pivots and
+      // bases do not depend on the group size, and a problem's chain of phases
+      // runs beside the others' (four problems of n = 65536 one after the other
+      // with full groups: 1.62 ms)
+      int ncta = 0;
+      for (int l = 0; l < gr.levels; ++l) ncta += gr.G[l] << l;
+      CK(cudaMemset2DAsync(S.aca_bar, sstride, 0, sizeof(unsigned int) * P->aca_ncoop, nprob, s));
+      CK(cudaMemset2DAsync(S.flags, sstride, 0, sizeof(int), nprob, s));
+      CK(launch_aca(H0, P->aca_work, ncta, S.aca_part, S.aca_bar, S.flags, s, nprob, sstride, &gr));
     } else {
       for (int q = 0; q < nprob; ++q) {  // one grouped launch per problem, each filling the GPU
         const size_t off = (size_t)q * sstride;
@@ -953,7 +1003,7 @@ extern "C" fifa_status fifa_logdet(fifa_ctx* ctx, const fifa_fact* F, double* ou
 // Sweeps, solve, matvec
 // ---------------------------------------------------------------------------
 bool sweep_batch_config(fifa_ctx* ctx, const Plan* P, int nprob, int* ls, int* rows) {
-  if (P->fs_ls < 0 || nprob < 1) return false;
+  if (P->fs_ls < 0 || P->cluster || nprob < 1) return false;
   for (int k = P->fs_ls; k >= 0; --k) {
     int r = 0;
     for (int i = 0; i < (1 << k); ++i) r = std::max(r, P->bnd_host[bnd_off(k) + i + 1] - P->bnd_host[bnd_off(k) + i]);
@@ -986,7 +1036,7 @@ fifa_status sweep_enqueue_desc(fifa_ctx* ctx, Plan* P, const FactDesc* Fdev, int
   if (P->fs_ls >= 0) {
     if (mode != 5) CK(cudaMemsetAsync(S.fs_bar, 0, sizeof(unsigned int) * fs_bar_uints(P->fs_ls), s));
     CK(launch_sweep_fused(Fdev, prec, P->fs_ls, P->fs_rows, ctx->opts.rank_cap, v, nrhs, mode, S.fs_part, S.fs_bar,
-                          (int*)S.fs_bar, s, active));
+                          (int*)S.fs_bar, P->cluster, s, active));
     return FIFA_OK;
   }
   auto level = [&](int l, int zsel, int zt) -> cudaError_t {
@@ -1061,7 +1111,7 @@ fifa_status matvec_enqueue(fifa_ctx* ctx, const fifa_hmat* A, const double* in, 
   Scratch S = carve(ctx, P);
   if (P->mv_ls >= 0) {
     CK(cudaMemsetAsync(S.mv_bar, 0, sizeof(unsigned int) * MV_BAR_UINTS, ctx->stream));
-    CK(launch_mv_fused(A->dev, P->mv_ls, P->mv_rows, in, nrhs, out, S.mv_fpart, S.mv_bar, ctx->stream, active));
+    CK(launch_mv_fused(A->dev, P->mv_ls, P->mv_rows, in, nrhs, out, S.mv_fpart, S.mv_bar, P->cluster, ctx->stream, active));
     return FIFA_OK;
   }
   CK(launch_matvec(A->dev, P->nleaf, P->L, in, nrhs, S.mv_part, S.mv_proj, out, ctx->stream, active));
@@ -1211,7 +1261,7 @@ fifa_status sample_enqueue(fifa_ctx* ctx, const fifa_hmat* C, const fifa_fact* W
 
 bool mv_batch_config(fifa_ctx* ctx, const Plan* P, int nprob, int* ls, int* rows) {
   (void)ctx;
-  if (P->mv_ls < 0 || nprob < 1) return false;
+  if (P->mv_ls < 0 || P->cluster || nprob < 1) return false;
   for (int k = P->mv_ls; k >= 0; --k) {
     int r = 0;
     for (int i = 0; i < (1 << k); ++i) r = std::max(r, P->bnd_host[bnd_off(k) + i + 1] - P->bnd_host[bnd_off(k) + i]);

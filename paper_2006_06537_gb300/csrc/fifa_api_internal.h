@@ -31,6 +31,7 @@ struct Plan {
   int lvl_ctas_max = 1;
   int lvl_grouped = 0;  // levels 0 .. lvl_grouped - 1 have CTA groups
   int fs_ls = -1, fs_rows = 0;  // fused sweep: 2^fs_ls CTAs of fs_rows rows (-1: per-level sweeps)
+  bool cluster = false;  // fused sweep and product launched as one cluster (independent CTAs)
   int mv_ls = -1, mv_rows = 0;  // fused H-matvec: 2^mv_ls CTAs of mv_rows rows (-1: three-pass product)
   size_t scratch_bytes = 0;
 };

@@ -2,7 +2,32 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <stddef.h>
+#include <atomic>
 #include "fifa_common.cuh"
+
+// Let a kernel take all the dynamic shared memory the device allows, once per
+// device: the same value from every thread, so host threads that launch it with
+// different sizes never lower each other's limit between its setting and their
+// launch.  ALLOW_SMEM(kernel) is a cudaError_t.
+inline cudaError_t allow_smem(const void* kernel, std::atomic<unsigned long long>& done) {
+  int dev = 0, optin = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const unsigned long long bit = 1ull << (dev & 63);
+  if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+  cudaFuncAttributes a;
+  e = cudaFuncGetAttributes(&a, kernel);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)a.sharedSizeBytes);
+  if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+  return e;
+}
+#define ALLOW_SMEM(...)                               \
+  ([]() -> cudaError_t {                              \
+    static std::atomic<unsigned long long> done{0};   \
+    return allow_smem((const void*)(__VA_ARGS__), done); \
+  }())
 
 // Assembly launchers take nprob problems of one plan (descriptor arrays,
 // blockIdx.y); the grouped ACA's partials / barriers / abort flags of problem q
@@ -10,9 +35,16 @@
 cudaError_t launch_leaf_assemble(const HmatDesc* Hd, int nleaf, cudaStream_t st, int nprob = 1);
 #define ACA_WARP_MAX 128  // largest side of a block that the warp-per-block ACA takes
 cudaError_t launch_aca_warp(const HmatDesc* Hd, const int4* work, int nwork, cudaStream_t st, int nprob = 1);
-// ncta CTAs of the grouped blocks' work list (a cooperative launch: they wait on each other)
+// Group sizes of the blocks of levels 0 .. levels - 1 (every block of a level alike).
+#define ACA_GROUP_LEVELS 12
+struct AcaGroups {
+  int levels;
+  int G[ACA_GROUP_LEVELS];
+};
+// ncta CTAs of the grouped blocks (a cooperative launch: they wait on each
+// other), by the work list or, with groups, by its group sizes.
 cudaError_t launch_aca(const HmatDesc* Hd, const int4* work, int ncta, ArgMax* part, unsigned int* bar, int* abort_flag,
-                       cudaStream_t st, int nprob = 1, size_t pstride = 0);
+                       cudaStream_t st, int nprob = 1, size_t pstride = 0, const AcaGroups* groups = nullptr);
 // one CTA or cluster per block; span: rows and columns of the largest block
 cudaError_t launch_aca_solo(const HmatDesc* Hd, const int4* work, int nblocks, int span, cudaStream_t st, int nprob = 1);
 int aca_max_coresident_ctas();
@@ -64,8 +96,8 @@ int sweep_fused_coresident(int prec, int rows, int cap);
 // only those levels of the factor), then 6 = its levels < ls.  Arithmetic in
 // the factor's storage precision (prec 1: FP32).
 cudaError_t launch_sweep_fused(const FactDesc* Fd, int prec, int ls, int rows, int cap, double* v, int nrhs,
-                               int mode, double* part, unsigned int* bar, int* abort_flag, cudaStream_t st,
-                               const int* active = nullptr);
+                               int mode, double* part, unsigned int* bar, int* abort_flag, bool cluster,
+                               cudaStream_t st, const int* active = nullptr);
 // nprob FP64 factors of one plan in one launch (one right-hand side each at
 // vlist[q]; per-problem partials / barrier / abort flag pstride bytes apart)
 cudaError_t launch_sweep_fused_batched(const FactDesc* Fd, int ls, int rows, double* const* vlist, int nprob,
@@ -77,7 +109,7 @@ cudaError_t launch_sweep_fused_batched(const FactDesc* Fd, int ls, int rows, dou
 #define MV_BAR_UINTS 2
 int mv_fused_coresident(int rows);
 cudaError_t launch_mv_fused(const HmatDesc* Hd, int ls, int rows, const double* x, int nrhs, double* y, double* part,
-                            unsigned int* bar, cudaStream_t st, const int* active = nullptr);
+                            unsigned int* bar, bool cluster, cudaStream_t st, const int* active = nullptr);
 // nprob H-matrices of one plan in one launch (one right-hand side each:
 // xlist[q] -> ylist[q]; per-problem partials and abort flag / counter pstride
 // bytes apart)

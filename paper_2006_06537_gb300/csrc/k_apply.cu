@@ -1054,7 +1054,7 @@ size_t sweep_fused_smem(int rows, int nrhs, int prec) {
 template <typename T, int NR, bool BATCH = false>
 static int sweep_fused_per_sm(size_t smem) {
   int per_sm = 0;
-  cudaFuncSetAttribute(k_sweep_fused<T, NR, BATCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  ALLOW_SMEM(k_sweep_fused<T, NR, BATCH>);
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep_fused<T, NR, BATCH>, 256, smem) != cudaSuccess)
     per_sm = 0;
   cudaGetLastError();
@@ -1082,8 +1082,9 @@ static cudaError_t launch_sweep_fused_t(cudaLaunchConfig_t& cfg, const FactDesc*
                                         int rows, double* part, unsigned int* bar, int* abort_flag,
                                         const int* active, int prec, double* const* vlist = nullptr,
                                         size_t pstride = 0) {
-  cudaFuncSetAttribute(k_sweep_fused<T, NR, BATCH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)sweep_fused_smem(rows, SW_RHS_MAX, prec));
+  (void)prec;
+  const cudaError_t e = ALLOW_SMEM(k_sweep_fused<T, NR, BATCH>);
+  if (e != cudaSuccess) return e;
   return cudaLaunchKernelEx(&cfg, k_sweep_fused<T, NR, BATCH>, Fd, v, mode, ls, rows, part, bar, abort_flag, active,
                             vlist, pstride);
 }
@@ -1108,8 +1109,8 @@ cudaError_t launch_sweep_fused_batched(const FactDesc* Fd, int ls, int rows, dou
 }
 
 cudaError_t launch_sweep_fused(const FactDesc* Fd, int prec, int ls, int rows, int cap, double* v, int nrhs,
-                               int mode, double* part, unsigned int* bar, int* abort_flag, cudaStream_t st,
-                               const int* active) {
+                               int mode, double* part, unsigned int* bar, int* abort_flag, bool cluster,
+                               cudaStream_t st, const int* active) {
   (void)cap;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(1u << ls);
@@ -1117,8 +1118,15 @@ cudaError_t launch_sweep_fused(const FactDesc* Fd, int prec, int ls, int rows, i
   cfg.dynamicSmemBytes = sweep_fused_smem(rows, nrhs, prec);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = mode == 5 ? 0 : 1;  // mode 5's CTAs never wait on each other
+  if (cluster) {
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 1u << ls;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+  } else {
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = mode == 5 ? 0 : 1;  // mode 5's CTAs never wait on each other
+  }
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   if (prec)
@@ -1201,7 +1209,7 @@ bool predict_many(int64_t n, int64_t nstar) {
 cudaError_t launch_predict(const HmatDesc* Hd, const FactDesc* Fd, int64_t n, const double* x, const double* xstar,
                            int64_t nstar, const double* alpha, double tau2, double* mu, double* var, cudaStream_t st) {
   const size_t smem = predict_smem(n);
-  cudaError_t e = cudaFuncSetAttribute(k_predict, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = ALLOW_SMEM(k_predict);
   if (e != cudaSuccess) return e;
   k_predict<<<(unsigned)std::min<int64_t>(nstar, 1 << 20), 256, smem, st>>>(Hd, Fd, x, xstar, nstar, alpha, tau2, mu, var);
   return cudaGetLastError();
@@ -1504,7 +1512,7 @@ static int mv_fused_per_sm_v(int rows) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (smem > (size_t)optin) return 0;
-  cudaFuncSetAttribute(k_mv_fused<RPT, BATCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  ALLOW_SMEM(k_mv_fused<RPT, BATCH>);
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mv_fused<RPT, BATCH>, mv_shape(rows).threads, smem) !=
       cudaSuccess)
     per_sm = 0;
@@ -1534,20 +1542,28 @@ int mv_fused_coresident(int rows) {
 
 template <int RPT, bool BATCH = false>
 static cudaError_t launch_mv_fused_t(const HmatDesc* Hd, int ls, int rows, const double* x, int nrhs, double* y,
-                                     double* part, unsigned int* bar, cudaStream_t st, const int* active,
-                                     const double* const* xlist = nullptr, double* const* ylist = nullptr,
+                                     double* part, unsigned int* bar, bool cluster, cudaStream_t st,
+                                     const int* active, const double* const* xlist = nullptr, double* const* ylist = nullptr,
                                      int nprob = 1, size_t pstride = 0) {
   const size_t smem = mv_fused_smem(rows);
   const MvShape sh = mv_shape(rows);
-  cudaFuncSetAttribute(k_mv_fused<RPT, BATCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = ALLOW_SMEM(k_mv_fused<RPT, BATCH>);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(1u << ls, nprob);
   cfg.blockDim = dim3(sh.threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
+  if (cluster) {
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 1u << ls;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+  } else {
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+  }
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, k_mv_fused<RPT, BATCH>, Hd, x, nrhs, y, ls, rows, sh.hs, sh.rp, part, bar, active,
@@ -1559,7 +1575,7 @@ static cudaError_t launch_mv_fused_t(const HmatDesc* Hd, int ls, int rows, const
 cudaError_t launch_mv_fused_batched(const HmatDesc* Hd, int ls, int rows, const double* const* xlist,
                                     double* const* ylist, int nprob, double* part, unsigned int* bar, size_t pstride,
                                     cudaStream_t st) {
-#define MVB(R) launch_mv_fused_t<R, true>(Hd, ls, rows, nullptr, 1, nullptr, part, bar, st, nullptr, xlist, ylist, nprob, pstride)
+#define MVB(R) launch_mv_fused_t<R, true>(Hd, ls, rows, nullptr, 1, nullptr, part, bar, false, st, nullptr, xlist, ylist, nprob, pstride)
   switch (mv_shape(rows).rpt) {
     case 1: return MVB(1);
     case 2: return MVB(2);
@@ -1572,13 +1588,13 @@ cudaError_t launch_mv_fused_batched(const HmatDesc* Hd, int ls, int rows, const 
 }
 
 cudaError_t launch_mv_fused(const HmatDesc* Hd, int ls, int rows, const double* x, int nrhs, double* y, double* part,
-                            unsigned int* bar, cudaStream_t st, const int* active) {
+                            unsigned int* bar, bool cluster, cudaStream_t st, const int* active) {
   switch (mv_shape(rows).rpt) {
-    case 1: return launch_mv_fused_t<1>(Hd, ls, rows, x, nrhs, y, part, bar, st, active);
-    case 2: return launch_mv_fused_t<2>(Hd, ls, rows, x, nrhs, y, part, bar, st, active);
-    case 4: return launch_mv_fused_t<4>(Hd, ls, rows, x, nrhs, y, part, bar, st, active);
-    case 8: return launch_mv_fused_t<8>(Hd, ls, rows, x, nrhs, y, part, bar, st, active);
-    case 16: return launch_mv_fused_t<16>(Hd, ls, rows, x, nrhs, y, part, bar, st, active);
+    case 1: return launch_mv_fused_t<1>(Hd, ls, rows, x, nrhs, y, part, bar, cluster, st, active);
+    case 2: return launch_mv_fused_t<2>(Hd, ls, rows, x, nrhs, y, part, bar, cluster, st, active);
+    case 4: return launch_mv_fused_t<4>(Hd, ls, rows, x, nrhs, y, part, bar, cluster, st, active);
+    case 8: return launch_mv_fused_t<8>(Hd, ls, rows, x, nrhs, y, part, bar, cluster, st, active);
+    case 16: return launch_mv_fused_t<16>(Hd, ls, rows, x, nrhs, y, part, bar, cluster, st, active);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -135,6 +135,7 @@ __device__ __forceinline__ AcaBest aca_remote(const AcaBest* p, int rank) {
 
 template <bool CL>
 __global__ void __launch_bounds__(256, 4) k_aca(const HmatDesc* __restrict__ Hd, const int4* __restrict__ work, int C,
+                                              AcaGroups groups,
                                               ArgMax* __restrict__ part, unsigned int* __restrict__ bar,
                                               int* __restrict__ abort_flag, size_t pstride) {
   // problem of a batched launch: its descriptor, its partials, barriers and
@@ -143,8 +144,18 @@ __global__ void __launch_bounds__(256, 4) k_aca(const HmatDesc* __restrict__ Hd,
   part = (ArgMax*)((char*)part + blockIdx.y * pstride);
   bar = (unsigned int*)((char*)bar + blockIdx.y * pstride);
   abort_flag = (int*)((char*)abort_flag + blockIdx.y * pstride);
-  const int4 w = work[CL ? blockIdx.x / C : blockIdx.x];
-  const int lvl = w.x, bi = w.y, g = CL ? blockIdx.x % C : w.z, G = CL ? C : w.w;
+  int lvl, bi, g, G;
+  if (!CL && groups.levels > 0) {  // smaller groups than the work list's: level after level, block after block
+    int b = blockIdx.x;
+    lvl = 0;
+    while (b >= groups.G[lvl] << lvl) b -= groups.G[lvl] << lvl, ++lvl;
+    G = groups.G[lvl];
+    bi = b / G;
+    g = b % G;
+  } else {
+    const int4 w = work[CL ? blockIdx.x / C : blockIdx.x];
+    lvl = w.x, bi = w.y, g = CL ? blockIdx.x % C : w.z, G = CL ? C : w.w;
+  }
   const int base = blockIdx.x - g;
   const int64_t n = Hd->n;
   const int cap = Hd->cap, kind = Hd->kind;
@@ -430,7 +441,7 @@ static cudaError_t launch_aca_cluster(const HmatDesc* Hd, const int4* work, int 
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_aca<true>, Hd, work, C, (ArgMax*)nullptr, (unsigned int*)nullptr, (int*)nullptr,
+  return cudaLaunchKernelEx(&cfg, k_aca<true>, Hd, work, C, AcaGroups{}, (ArgMax*)nullptr, (unsigned int*)nullptr, (int*)nullptr,
                             (size_t)0);
 }
 
@@ -456,7 +467,7 @@ cudaError_t launch_aca_solo(const HmatDesc* Hd, const int4* work, int nblocks, i
 }
 
 cudaError_t launch_aca(const HmatDesc* Hd, const int4* work, int ncta, ArgMax* part, unsigned int* bar, int* abort_flag,
-                       cudaStream_t st, int nprob, size_t pstride) {
+                       cudaStream_t st, int nprob, size_t pstride, const AcaGroups* groups) {
   if (ncta <= 0) return cudaSuccess;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ncta, nprob);
@@ -468,7 +479,7 @@ cudaError_t launch_aca(const HmatDesc* Hd, const int4* work, int ncta, ArgMax* p
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_aca<false>, Hd, work, 1, part, bar, abort_flag, pstride);
+  return cudaLaunchKernelEx(&cfg, k_aca<false>, Hd, work, 1, groups ? *groups : AcaGroups{}, part, bar, abort_flag, pstride);
 }
 
 int aca_max_coresident_ctas() {

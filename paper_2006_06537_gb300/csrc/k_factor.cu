@@ -651,7 +651,7 @@ __device__ void proj_tiled(const T* __restrict__ Qb, T* const* Bp, int w, int64_
 #define LW_RLO 16
 template <typename T>
 __global__ void __launch_bounds__(256, 2)
-    k_level_wide(const FactDesc* __restrict__ Fd, int lvl, int G, double* __restrict__ gpart,
+    k_level_wide(const FactDesc* __restrict__ Fd, int lvl, int nodes, int G, double* __restrict__ gpart,
                  unsigned int* __restrict__ bar, int* __restrict__ abort_flag, size_t sstride) {
   extern __shared__ double sm[];
   // problem of a batched launch: its descriptor, and its scratch sstride bytes on
@@ -660,7 +660,10 @@ __global__ void __launch_bounds__(256, 2)
   gpart = (double*)((char*)gpart + blockIdx.y * sstride);
   bar = (unsigned int*)((char*)bar + blockIdx.y * sstride);
   abort_flag = (int*)((char*)abort_flag + blockIdx.y * sstride);
-  const int bi = blockIdx.x / G, g = blockIdx.x % G, base = blockIdx.x - g;
+  const int g = blockIdx.x % G, base = blockIdx.x - g;
+  // (a group has one node; single CTAs stride over the level, most of whose nodes
+  // are another launch's: a CTA for each took 22 us at 4096 nodes)
+  for (int bi = blockIdx.x / G; bi < nodes; bi += gridDim.x / G) {
   const int nid = node_id(lvl, bi);
   const int cap = Fd->cap, nleaf = Fd->nleaf;
   const int64_t n = Fd->n;
@@ -668,7 +671,8 @@ __global__ void __launch_bounds__(256, 2)
   int s, h, e;
   node_range(bnd, lvl, bi, s, h, e);
   const int r = Fd->rank[nid];
-  if (r <= LW_RLO) return;  // another launch takes this node
+  if (r <= LW_RLO) continue;  // another launch takes this node
+  __syncthreads();            // shared memory is free again
   int* status = Fd->status;
   T* Qall = (T*)Fd->Q;
   T* Qb = Qall + (size_t)lvl * cap * n;
@@ -856,6 +860,7 @@ __global__ void __launch_bounds__(256, 2)
     update_pass<T, W>(Qb, Bp, w, n, r, max(r0, s), min(r1, h), Tm);
     update_pass<T, W>(Qb, Bp, w, n, r, max(r0, h), min(r1, e), Tm + r * W);
     __syncthreads();
+  }
   }
 }
 
@@ -1229,8 +1234,7 @@ template <typename T, int R, int MS, int NPC>
 static cudaError_t launch_level_multi(const FactDesc* Fd, int lvl, int nodes, cudaStream_t st, int nprob) {
   const size_t smem = LmLayout<R, MS, NPC>::bytes(sizeof(T));
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_level_multi<T, R, MS, NPC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    const cudaError_t e = ALLOW_SMEM(k_level_multi<T, R, MS, NPC>);
     if (e != cudaSuccess) return e;
   }
   k_level_multi<T, R, MS, NPC><<<dim3((nodes + NPC - 1) / NPC, nprob), 256, smem, st>>>(Fd, lvl, nodes);
@@ -1290,8 +1294,7 @@ cudaError_t launch_leaf_factor(const HmatDesc* Hd, const FactDesc* Fd, int prec,
   const size_t smem = block ? leaf_block_doubles(Bm) * sizeof(double) : leaf_factor_smem(Bm, L, cap, 0);
   if (smem > (size_t)smem_optin()) return cudaErrorInvalidConfiguration;
   if (smem > 48 * 1024) {
-    cudaError_t e = block ? cudaFuncSetAttribute(k_leaf_factor_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                          : cudaFuncSetAttribute(k_leaf_factor<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = block ? ALLOW_SMEM(k_leaf_factor_block) : ALLOW_SMEM(k_leaf_factor<double>);
     if (e != cudaSuccess) return e;
   }
   const dim3 grid(nleaf * nsplit, nprob);
@@ -1311,10 +1314,10 @@ static cudaError_t launch_level_wide(const FactDesc* Fd, int lvl, int nodes, int
       }
   const size_t smem = level_wide_smem(cap);
   if (smem > (size_t)smem_optin()) return cudaErrorInvalidConfiguration;
-  cudaError_t e = cudaFuncSetAttribute(k_level_wide<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = ALLOW_SMEM(k_level_wide<double>);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(nodes * G, nprob);
+  cfg.gridDim = dim3(G > 1 ? nodes * G : std::min(nodes, 304), nprob);
   cfg.blockDim = dim3(256);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
@@ -1330,7 +1333,7 @@ static cudaError_t launch_level_wide(const FactDesc* Fd, int lvl, int nodes, int
   }
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_level_wide<double>, Fd, lvl, G, part, bar, abort_flag, sstride);
+  return cudaLaunchKernelEx(&cfg, k_level_wide<double>, Fd, lvl, nodes, G, part, bar, abort_flag, sstride);
 }
 
 // CTAs of a cluster for a node of `rows` rows when a launch has `nodes` nodes:
@@ -1380,7 +1383,7 @@ cudaError_t launch_level(const FactDesc* Fd, int prec, int lvl, int nodes, const
 static int level_wide_per_sm(int cap) {
   const size_t smem = level_wide_smem(cap);
   if (smem > (size_t)smem_optin()) return 0;
-  cudaFuncSetAttribute(k_level_wide<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  ALLOW_SMEM(k_level_wide<double>);
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_level_wide<double>, 256, smem) != cudaSuccess) per_sm = 0;
   cudaGetLastError();

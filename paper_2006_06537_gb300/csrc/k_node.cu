@@ -576,8 +576,7 @@ template <int RB, int RLO, bool CL>
 static cudaError_t launch_node_t(const FactDesc* Fd, int lvl, int nodes, int G, double* part, unsigned int* bar,
                                  int* abort_flag, int skip, cudaStream_t st, int nprob, size_t sstride) {
   const size_t smem = NdLayout<RB>::bytes(CL ? G : 1);
-  cudaError_t e = cudaFuncSetAttribute(k_level<RB, RLO, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)NdLayout<RB>::bytes(CL ? 2 : 1));
+  const cudaError_t e = ALLOW_SMEM(k_level<RB, RLO, CL>);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(nodes * G, nprob);
@@ -613,7 +612,7 @@ cudaError_t launch_node(const FactDesc* Fd, int rb, int rlo, bool cluster, int l
 template <int RB, int RLO>
 static int node_per_sm() {
   const size_t smem = NdLayout<RB>::bytes(1);
-  cudaFuncSetAttribute(k_level<RB, RLO, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)NdLayout<RB>::bytes(2));
+  ALLOW_SMEM(k_level<RB, RLO, false>);
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_level<RB, RLO, false>, 256, smem) != cudaSuccess) per_sm = 0;
   cudaGetLastError();
