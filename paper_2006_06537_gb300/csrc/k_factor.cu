@@ -214,21 +214,23 @@ __global__ void __launch_bounds__(256, 7)
 // entry.  The next diagonal block is factored by warp 0 while the other warps
 // update.  The matrix is a packed lower triangle, column after column, so the
 // trailing triangle is one contiguous range and two CTAs of 128-row leaves fit
-// an SM.
-// 1024 leaves of 128 rows with 21 ancestor columns: 3.04 -> 1.66 ms (0.92 ms at
-// the FP64 peak; 1024 leaves are 3.4 waves of two CTAs per SM).  The line at 64
+// an SM: of 16 warps each, since every entry's eight multiply-adds are a chain.
+// 1024 leaves of 128 rows with 21 ancestor columns: 3.04 ms column by column,
+// 1.65 with 8 warps per CTA, 1.46 with 12, 1.38 with 16 (0.92 ms at the FP64
+// peak; 1024 leaves are 3.4 waves of two CTAs per SM).  The line at 64
 // rows: 32 leaves of 64 rows take 84 us either way, 512 leaves of 40 rows 73 us
 // column by column and 81 us in blocks (the chain of diagonal blocks).
 // ---------------------------------------------------------------------------
 #define LB_NB 8
-#define LB_COLS 32  // ancestor columns per pass
+#define LB_COLS 32     // ancestor columns per pass
+#define LB_THREADS 512
 
 __host__ __device__ inline size_t leaf_block_doubles(int Bm) {
   const size_t nblk = (Bm + LB_NB - 1) / LB_NB;
   return (size_t)Bm * (Bm + 1) / 2 + (size_t)LB_COLS * (Bm | 1) + nblk * LB_NB * LB_NB + LB_NB * LB_NB + LB_NB + 40 + Bm;
 }
 
-__global__ void __launch_bounds__(256, 4)
+__global__ void __launch_bounds__(LB_THREADS, 2)
     k_leaf_factor_block(const HmatDesc* __restrict__ Hd, const FactDesc* __restrict__ Fd, int nsplit) {
   extern __shared__ double sm[];
   Hd += blockIdx.y;  // problem of a batched launch (descriptor arrays)
@@ -1298,7 +1300,7 @@ cudaError_t launch_leaf_factor(const HmatDesc* Hd, const FactDesc* Fd, int prec,
     if (e != cudaSuccess) return e;
   }
   const dim3 grid(nleaf * nsplit, nprob);
-  if (block) k_leaf_factor_block<<<grid, 256, smem, st>>>(Hd, Fd, nsplit);
+  if (block) k_leaf_factor_block<<<grid, LB_THREADS, smem, st>>>(Hd, Fd, nsplit);
   else k_leaf_factor<double><<<grid, 256, smem, st>>>(Hd, Fd, nsplit);
   return cudaGetLastError();
 }
