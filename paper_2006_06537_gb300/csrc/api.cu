@@ -628,8 +628,8 @@ static int aca_solo_span(const Plan* P) {
   return P->bnd_host[bnd_off(w.x) + w.y + 1] - P->bnd_host[bnd_off(w.x) + w.y];
 }
 
-// Second part (after the first in stream order): dense leaves, one-CTA and
-// one-warp ACA blocks; independent CTAs only.
+// Second part (after the first in stream order): dense leaves and the ACA
+// blocks without a group; independent CTAs and clusters only.
 fifa_status hmat_assemble_rest_enqueue(fifa_ctx* ctx, fifa_hmat* H) {
   Plan* P = H->plan;
   fifa_status st = ensure_scratch(ctx, P);
@@ -637,8 +637,7 @@ fifa_status hmat_assemble_rest_enqueue(fifa_ctx* ctx, fifa_hmat* H) {
   Scratch S = carve(ctx, P);
   cudaStream_t s = ctx->stream;
   CK(launch_leaf_assemble(H->dev, P->nleaf, s));
-  CK(launch_aca_solo(H->dev, P->aca_work + P->aca_ncoop, P->aca_nsolo, aca_solo_span(P), s));
-  if (P->aca_nwarp > 0) CK(launch_aca_warp(H->dev, P->aca_work + P->aca_ncoop + P->aca_nsolo, P->aca_nwarp, s));
+  CK(launch_aca_blocks(H->dev, P->aca_work + P->aca_ncoop, P->aca_nsolo, P->aca_nwarp, aca_solo_span(P), s));
   return FIFA_OK;
 }
 
@@ -697,8 +696,7 @@ fifa_status hmat_assemble_batched(fifa_ctx* ctx, Plan* P, HmatDesc* H0, int npro
       }
     }
   }
-  CK(launch_aca_solo(H0, P->aca_work + P->aca_ncoop, P->aca_nsolo, aca_solo_span(P), s, nprob));
-  if (P->aca_nwarp > 0) CK(launch_aca_warp(H0, P->aca_work + P->aca_ncoop + P->aca_nsolo, P->aca_nwarp, s, nprob));
+  CK(launch_aca_blocks(H0, P->aca_work + P->aca_ncoop, P->aca_nsolo, P->aca_nwarp, aca_solo_span(P), s, nprob));
   return FIFA_OK;
 }
 

@@ -34,7 +34,6 @@ inline cudaError_t allow_smem(const void* kernel, std::atomic<unsigned long long
 // sit q * pstride bytes after problem 0's.
 cudaError_t launch_leaf_assemble(const HmatDesc* Hd, int nleaf, cudaStream_t st, int nprob = 1);
 #define ACA_WARP_MAX 128  // largest side of a block that the warp-per-block ACA takes
-cudaError_t launch_aca_warp(const HmatDesc* Hd, const int4* work, int nwork, cudaStream_t st, int nprob = 1);
 // Group sizes of the blocks of levels 0 .. levels - 1 (every block of a level alike).
 #define ACA_GROUP_LEVELS 12
 struct AcaGroups {
@@ -46,7 +45,8 @@ struct AcaGroups {
 cudaError_t launch_aca(const HmatDesc* Hd, const int4* work, int ncta, ArgMax* part, unsigned int* bar, int* abort_flag,
                        cudaStream_t st, int nprob = 1, size_t pstride = 0, const AcaGroups* groups = nullptr);
 // one CTA or cluster per block; span: rows and columns of the largest block
-cudaError_t launch_aca_solo(const HmatDesc* Hd, const int4* work, int nblocks, int span, cudaStream_t st, int nprob = 1);
+cudaError_t launch_aca_blocks(const HmatDesc* Hd, const int4* work, int nsolo, int nwarp, int span, cudaStream_t st,
+                              int nprob = 1);
 int aca_max_coresident_ctas();
 
 size_t leaf_factor_smem(int Bm, int L, int cap, int prec);

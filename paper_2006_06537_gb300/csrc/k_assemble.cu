@@ -445,25 +445,33 @@ static cudaError_t launch_aca_cluster(const HmatDesc* Hd, const int4* work, int 
                             (size_t)0);
 }
 
-// Small blocks: one warp each when there are enough to fill the GPU, else a CTA
-// or a cluster each (the same bases either way: 15 blocks of n = 500 took one
-// warp each 278 us).
-cudaError_t launch_aca_warp(const HmatDesc* Hd, const int4* work, int nwork, cudaStream_t st, int nprob) {
-  if (nwork <= 0) return cudaSuccess;
-  if ((int64_t)nwork * nprob <= 608)
-    return launch_aca_cluster(Hd, work, nwork, aca_cluster((int64_t)nwork * nprob, 2 * ACA_WARP_MAX), st, nprob);
-  k_aca_warp<<<dim3((nwork + 7) / 8, nprob), 256, 0, st>>>(Hd, work, nwork);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_leaf_assemble(const HmatDesc* Hd, int nleaf, cudaStream_t st, int nprob) {
   k_leaf_assemble<<<dim3(nleaf, nprob), 256, 0, st>>>(Hd);
   return cudaGetLastError();
 }
 
-cudaError_t launch_aca_solo(const HmatDesc* Hd, const int4* work, int nblocks, int span, cudaStream_t st, int nprob) {
-  if (nblocks <= 0) return cudaSuccess;
-  return launch_aca_cluster(Hd, work, nblocks, aca_cluster((int64_t)nblocks * nprob, span), st, nprob);
+// The blocks without a group: work[0, nsolo) the larger ones (span: rows and
+// columns of the largest), work[nsolo, nsolo + nwarp) those of at most
+// ACA_WARP_MAX rows a side.  Small blocks take one warp each when there are
+// enough to fill the GPU, else a cluster each like the larger ones (15 blocks of
+// n = 500 took one warp each 278 us), in the same launch if that leaves the
+// largest block at most 512 rows and columns to a CTA, two entries of a phase to
+// a thread: the two launches of n = 500 took 98 and 87 us one after the other.
+cudaError_t launch_aca_blocks(const HmatDesc* Hd, const int4* work, int nsolo, int nwarp, int span, cudaStream_t st,
+                              int nprob) {
+  const bool small_warps = (int64_t)nwarp * nprob > 608;
+  const int together = aca_cluster((int64_t)(nsolo + nwarp) * nprob, span);
+  if (!small_warps && nsolo > 0 && nwarp > 0 && span <= 1024 * together)
+    return launch_aca_cluster(Hd, work, nsolo + nwarp, together, st, nprob);
+  if (nsolo > 0) {
+    const cudaError_t e = launch_aca_cluster(Hd, work, nsolo, aca_cluster((int64_t)nsolo * nprob, span), st, nprob);
+    if (e != cudaSuccess) return e;
+  }
+  if (nwarp <= 0) return cudaSuccess;
+  if (!small_warps)
+    return launch_aca_cluster(Hd, work + nsolo, nwarp, aca_cluster((int64_t)nwarp * nprob, 2 * ACA_WARP_MAX), st, nprob);
+  k_aca_warp<<<dim3((nwarp + 7) / 8, nprob), 256, 0, st>>>(Hd, work + nsolo, nwarp);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_aca(const HmatDesc* Hd, const int4* work, int ncta, ArgMax* part, unsigned int* bar, int* abort_flag,

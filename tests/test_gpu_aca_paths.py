@@ -21,6 +21,7 @@ CASES = [
     (257, 16, 1, 0.1, 1e-10, 32, "sine"),      # warp-sized blocks by clusters, one of 128 x 129 by a solo launch
     (1500, 40, 0, 0.3, 1e-14, 6, "sine"),      # the rank cap stops every large block
     (3000, 2, 0, 0.05, 1e-10, 16, "sine"),     # more small blocks than the GPU holds CTAs: one warp each
+    (3500, 32, 0, 0.05, 1e-10, 32, "sine"),    # large and small blocks in one launch, clusters of four
     (6001, 100, 1, 0.02, 1e-10, 32, "cluster"),  # groups at the top, clusters below
     (9000, 64, 0, 0.002, 1e-12, 40, "sine"),   # many steps: U and V beyond the kept ones
 ]
