@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(256) k_sweep_leaf(const FactDesc* __restrict__
 // ones wait for the CTAs of their own node only (a counter per node).
 //
 // What bounds it: up to n ~ 2^17 the chain of levels < ls (a barrier of the
-// whole grid and loads behind it cost ~17 us per level; now ~4), beyond that
+// whole grid and loads behind it cost ~17 us per level; now 5 to 8), beyond that
 // the FP64 pipe.  So a level's basis rows and its block of Z are copied to
 // shared memory while the level before runs (as far as they fit, fs_qcap), and
 // sums go over lanes that share an output, not over one thread's chain: a lone
@@ -347,12 +347,6 @@ __device__ __forceinline__ void prefetch_cols_l2(const T* __restrict__ Qb, int64
     const int a = t / nl, li = first + t % nl;
     prefetch_l2(Qb + (size_t)a * n + (size_t)li * PER);
   }
-}
-
-template <typename T>
-__device__ __forceinline__ T warp_sum_t(T v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  return v;
 }
 
 // Sum over rows [a0, a1) of Bl[col][p] * xs[j][p - S] for K outputs
