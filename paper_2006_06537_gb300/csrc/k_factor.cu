@@ -1340,23 +1340,30 @@ static cudaError_t launch_level_wide(const FactDesc* Fd, int lvl, int nodes, int
 
 // CTAs of a cluster for a node of `rows` rows when a launch has `nodes` nodes:
 // up to eight while they fill at most two CTAs per SM of 152 and keep 12 rows
-// each.
+// each; sixteen (not portable, so asked for first) while they fill at most one
+// and keep 32: a node of 2048 rows and rank 14 spends a third of its 80 us on
+// its CTAs' row work (Gibbs iteration at n = 2048: 727 -> 705 us).
 static int level_cluster(int64_t nodes, int64_t rows) {
   int c = 1;
   while (c < 8 && 2 * c * nodes <= 304 && rows / (2 * c) >= 12) c *= 2;
+  if (c == 8 && 16 * nodes <= 152 && rows >= 512 && node_cluster_max() == 16) c = 16;
   return c;
 }
 
 // Ranks <= 16: nodes of at most LEVEL_CLUSTER_ROWS rows by a cluster each (its
 // CTAs are scheduled together by the hardware, so no cooperative launch and no
-// waiting on other launches), larger ones by groups of G CTAs.  Ranks above 16:
+// waiting on other launches), larger ones by groups of G CTAs, or by a cluster
+// where there are no groups (contexts with independent CTAs took one CTA per
+// node there: a factorization of n = 8191 2.81 -> 0.67 ms, of n = 20000 5.76 ->
+// 0.99 ms, with all the level kernels' changes).  Ranks above 16:
 // groups of G[2] CTAs, a cluster of them for the small nodes.
 cudaError_t launch_level(const FactDesc* Fd, int prec, int lvl, int nodes, const int* G, int cap, double* part,
                          unsigned int* bar, int bar_stride, int* abort_flag, int side_max, cudaStream_t st, int nprob,
                          size_t sstride) {
   if (prec != 0) return cudaErrorInvalidValue;
   cudaError_t e = cudaSuccess;
-  const bool cluster = level_clustered(side_max);
+  const int cl = level_cluster((int64_t)nodes * nprob, 2 * (int64_t)side_max);
+  const bool cluster = level_clustered(side_max) || (G[0] == 1 && G[1] == 1 && cl > 1);
   int skip = -1;
   if (side_max <= 128) {
     // small nodes of rank <= 4: several nodes per CTA
@@ -1365,7 +1372,6 @@ cudaError_t launch_level(const FactDesc* Fd, int prec, int lvl, int nodes, const
                          : launch_level_multi<double, 4, 128, 1>(Fd, lvl, nodes, st, nprob);
     skip = 4;
   }
-  const int cl = level_cluster((int64_t)nodes * nprob, 2 * (int64_t)side_max);
   const int Gn[2] = {cluster ? cl : G[0], cluster ? cl : G[1]};
   // a level of few nodes often has ranks of both buckets: one launch for every
   // rank <= 16 instead of two that would each leave the other's CTAs idle

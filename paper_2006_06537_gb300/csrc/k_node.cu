@@ -296,15 +296,19 @@ __global__ void __launch_bounds__(256, RB == 4 ? 4 : 3)
       const double* mine = slot();
       cluster_sync_all();
       for (int t = tid; t < count; t += blockDim.x) {
-        double v[8];
+        double sum = 0.0;
+        for (int q0 = 0; q0 < G; q0 += 8) {
+          double v[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) v[q] = q < G ? ld_cluster(mine + t, q) : 0.0;
+          for (int q = 0; q < 8; ++q) v[q] = q0 + q < G ? ld_cluster(mine + t, q0 + q) : 0.0;
 #pragma unroll
-        for (int o = 4; o > 0; o >>= 1)
+          for (int o = 4; o > 0; o >>= 1)
 #pragma unroll
-          for (int q = 0; q < 4; ++q)
-            if (q < o) v[q] += v[q + o];
-        xs[t] = v[0];
+            for (int q = 0; q < 4; ++q)
+              if (q < o) v[q] += v[q + o];
+          sum += v[0];
+        }
+        xs[t] = sum;
       }
       ++phase;
       __syncthreads();
@@ -607,6 +611,34 @@ cudaError_t launch_node(const FactDesc* Fd, int rb, int rlo, bool cluster, int l
   if (rlo >= 4) ND_GO(16, 4);
   ND_GO(16, -1);
 #undef ND_GO
+}
+
+// Largest cluster of the level kernels: 16 CTAs, beyond the portable eight,
+// where the GPU can hold one.
+template <int RB, int RLO>
+static bool node_cluster16() {
+  const size_t smem = NdLayout<RB>::bytes(16);
+  if (ALLOW_SMEM(k_level<RB, RLO, true>) != cudaSuccess ||
+      cudaFuncSetAttribute(k_level<RB, RLO, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+    return false;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(16);
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 16;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int held = 0;
+  return cudaOccupancyMaxActiveClusters(&held, k_level<RB, RLO, true>, &cfg) == cudaSuccess && held > 0;
+}
+int node_cluster_max() {
+  static const int c = node_cluster16<4, -1>() && node_cluster16<16, 4>() && node_cluster16<16, -1>() ? 16 : 8;
+  cudaGetLastError();
+  return c;
 }
 
 template <int RB, int RLO>
