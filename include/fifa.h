@@ -75,12 +75,13 @@ typedef struct {
   int refine_max;     /* MIXED: conjugate-gradient steps captured per solve (fixed; once every system
                          has converged the remaining steps' launches return at once) */
   int independent_ctas; /* 1: no kernel splits a tree node over a group of CTAs that wait on each
-                           other (every CTA runs independently).  0: groups fill the GPU (or the
+                           other (every CTA runs independently, or in a thread-block cluster that the
+                           hardware schedules as one).  0: groups fill the GPU (or the
                            context's coresident_share of it) for the top levels.  Several
                            contexts that launch work concurrently on one GPU need 1, or 0 with
                            coresident_share >= the number of such contexts. */
   int wait_polls;     /* a CTA waiting for the rest of its group gives up after this many polls
-                         (each followed by a 64 ns sleep), sets FIFA_ERR_TIMEOUT in the object's
+                         (each followed by a 64 ns sleep after the first 256), sets FIFA_ERR_TIMEOUT in the object's
                          status and makes the whole launch return; 0: the default 2^26 polls
                          (seconds).  Objects take the value of the context that created them. */
   int coresident_share; /* 0 or 1: a launch whose CTAs wait on each other may use every CTA the
@@ -404,7 +405,7 @@ void fifa_destroy_tensor(fifa_ctx* ctx, fifa_tensor* model);
  * among those a worker may run, when that worker is idle and the budget can
  * hold its chain (fifa_chain_bytes plus its input and result buffers);
  * admitted requests run concurrently and their kernels overlap on the GPU.
- * Narrow workers use independent CTAs (opts.independent_ctas forced to 1).
+ * Narrow workers use independent CTAs and clusters (opts.independent_ctas forced to 1).
  * With wide_min_n > 0, the wide workers run the requests with n >= wide_min_n,
  * with CTA groups and fused sweeps (the only streams whose kernels' CTAs wait
  * on each other), each sized to 1 / wide_workers of the CTAs the GPU holds at

@@ -320,7 +320,8 @@ __global__ void __launch_bounds__(256) k_sweep_leaf(const FactDesc* __restrict__
 // the FP64 pipe.  So a level's basis rows and its block of Z are copied to
 // shared memory while the level before runs (as far as they fit, fs_qcap), and
 // sums go over lanes that share an output, not over one thread's chain: a lone
-// warp takes 64 cycles per FP64 instruction.
+// warp takes 64 cycles per FP64 instruction.  One W^-1 of n = 2^20 to two
+// vectors 1.06 -> 0.83 ms; a solve of n = 500 129 -> 61 us.
 // ---------------------------------------------------------------------------
 #define FS_WARPS 8
 // Entries of a level's basis rows staged ahead, by the CTA's rows: as many as
@@ -1224,7 +1225,8 @@ cudaError_t launch_predict(const HmatDesc* Hd, const FactDesc* Fd, int64_t n, co
 // (U, V share one basis array: row p holds U if p is in the left child.)
 // Bound by the FP64 pipe for large n; for CTAs of few rows by how many threads
 // have work, so `hs` threads share a row (leaf columns and basis columns dealt
-// out between them) when there are at most 160.
+// out between them) when there are at most 160: n = 20011, one vector, 100 -> 49
+// us; n = 1000003 670 -> 626 us (0.47 ms at the FP64 peak).
 // ---------------------------------------------------------------------------
 #define MV_PROJ_BUF 1024                       // doubles of node projections per batch
 #define MV_PART_STRIDE (FIFA_CAP_MAX * SW_RHS_MAX)  // one CTA's partial of one level
