@@ -73,7 +73,7 @@ cudaError_t launch_level(const FactDesc* Fd, int prec, int lvl, int nodes, const
 cudaError_t launch_node(const FactDesc* Fd, int rb, int rlo, bool cluster, int lvl, int nodes, int G, double* part,
                         unsigned int* bar, int* abort_flag, int skip, cudaStream_t st, int nprob, size_t sstride);
 int node_ctas_per_sm(int rb);
-int node_cluster_max();  // CTAs of the level kernels' largest cluster: 16 or 8
+int node_cluster_max();  // CTAs of the level kernels' largest cluster on the current device: 16 or 8
 // Co-resident CTAs of the level kernel of rank bucket b (0: <= 4, 1: 5..16, 2: > 16).
 int level_bucket_coresident(int prec, int b, int cap);
 cudaError_t launch_logdet_reduce(const FactDesc* Fd, cudaStream_t st, int nprob = 1);

@@ -30,6 +30,7 @@
 // us; one factorization of n = 2^20 (clustered inputs, ranks 2 to 7) 11.8 -> 10.6
 // ms with the leaf factor's changes, its levels at 46-67% of the FP64 peak.
 #include <algorithm>
+#include <atomic>
 
 #include "fifa_common.cuh"
 #include "fifa_launch.h"
@@ -639,10 +640,19 @@ static bool node_cluster16() {
   int held = 0;
   return cudaOccupancyMaxActiveClusters(&held, k_level<RB, RLO, true>, &cfg) == cudaSuccess && held > 0;
 }
+// (for the current device: the permission that node_cluster16 sets is the
+// device's own, as is the answer)
 int node_cluster_max() {
-  static const int c = node_cluster16<4, -1>() && node_cluster16<16, 4>() && node_cluster16<16, -1>() ? 16 : 8;
-  cudaGetLastError();
-  return c;
+  static std::atomic<unsigned long long> asked{0}, sixteen{0};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 8;
+  const unsigned long long bit = 1ull << (dev & 63);
+  if (!(asked.load(std::memory_order_acquire) & bit)) {
+    if (node_cluster16<4, -1>() && node_cluster16<16, 4>() && node_cluster16<16, -1>()) sixteen.fetch_or(bit);
+    cudaGetLastError();
+    asked.fetch_or(bit, std::memory_order_release);
+  }
+  return sixteen.load(std::memory_order_relaxed) & bit ? 16 : 8;
 }
 
 template <int RB, int RLO>
