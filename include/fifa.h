@@ -76,7 +76,8 @@ typedef struct {
                          has converged the remaining steps' launches return at once) */
   int independent_ctas; /* 1: no kernel splits a tree node over a group of CTAs that wait on each
                            other (every CTA runs independently, or in a thread-block cluster that the
-                           hardware schedules as one).  0: groups fill the GPU (or the
+                           hardware schedules as one and that meets at its hardware barrier: nothing
+                           polls, and wait_polls does not apply).  0: groups fill the GPU (or the
                            context's coresident_share of it) for the top levels.  Several
                            contexts that launch work concurrently on one GPU need 1, or 0 with
                            coresident_share >= the number of such contexts. */

@@ -87,8 +87,9 @@ static int levels_for(int64_t n, int B) {
 }
 
 // Contexts with independent CTAs run the sweeps and products of small problems
-// fused in one cluster (eight CTAs that the hardware schedules together, so no
-// other work can keep one of them waiting) instead of two launches per tree level.
+// fused in one cluster (eight CTAs that the hardware schedules together and that
+// meet at its barrier, so nothing polls and opts.wait_polls does not apply) instead
+// of two launches per tree level.
 static bool one_cluster(int64_t n) { return n <= 8192; }
 
 // Partials of the fused sweep: one projection per CTA, level and sweep (a solve
@@ -1032,7 +1033,7 @@ fifa_status sweep_enqueue_desc(fifa_ctx* ctx, Plan* P, const FactDesc* Fdev, int
   Scratch S = carve(ctx, P);
   cudaStream_t s = ctx->stream;
   if (P->fs_ls >= 0) {
-    if (mode != 5) CK(cudaMemsetAsync(S.fs_bar, 0, sizeof(unsigned int) * fs_bar_uints(P->fs_ls), s));
+    if (mode != 5 && !P->cluster) CK(cudaMemsetAsync(S.fs_bar, 0, sizeof(unsigned int) * fs_bar_uints(P->fs_ls), s));
     CK(launch_sweep_fused(Fdev, prec, P->fs_ls, P->fs_rows, ctx->opts.rank_cap, v, nrhs, mode, S.fs_part, S.fs_bar,
                           (int*)S.fs_bar, P->cluster, s, active));
     return FIFA_OK;
@@ -1108,7 +1109,7 @@ fifa_status matvec_enqueue(fifa_ctx* ctx, const fifa_hmat* A, const double* in, 
   Plan* P = A->plan;
   Scratch S = carve(ctx, P);
   if (P->mv_ls >= 0) {
-    CK(cudaMemsetAsync(S.mv_bar, 0, sizeof(unsigned int) * MV_BAR_UINTS, ctx->stream));
+    if (!P->cluster) CK(cudaMemsetAsync(S.mv_bar, 0, sizeof(unsigned int) * MV_BAR_UINTS, ctx->stream));
     CK(launch_mv_fused(A->dev, P->mv_ls, P->mv_rows, in, nrhs, out, S.mv_fpart, S.mv_bar, P->cluster, ctx->stream, active));
     return FIFA_OK;
   }

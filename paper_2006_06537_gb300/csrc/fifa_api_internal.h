@@ -48,9 +48,9 @@ struct Scratch {
   double* red;  // 512 doubles of reduction partials
   int* flags;
   double* fs_part;        // fused sweep partials
-  unsigned int* fs_bar;   // fused sweep: abort flag, counters
+  unsigned int* fs_bar;   // fused sweep: abort flag, counters (not used by a cluster)
   double* mv_fpart;       // fused H-matvec partials
-  unsigned int* mv_bar;   // fused H-matvec grid barrier
+  unsigned int* mv_bar;   // fused H-matvec: abort flag, counter (not used by a cluster)
   double* pcg;            // PCG_SCRATCH_DOUBLES: partial sums and state of a mixed-precision solve
 };
 

@@ -273,6 +273,18 @@ __device__ inline void blk_triinv_lower(const double* Lm, int ldl, double* Li, i
 
 template <typename T> __device__ __forceinline__ double to_d(T v) { return (double)v; }
 
+// Hardware barrier of the CTAs of a thread-block cluster, in two halves: what a
+// CTA wrote before its arrival, in shared or global memory, is visible to the
+// others after their wait.  Every thread takes both, its warp converged.
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync_all() {
+  cluster_arrive();
+  cluster_wait();
+}
+
 // Bounded spin barrier among the G blocks of one group (counter monotone).
 // Returns false (in every thread) if the wait gave up; *err then has the
 // TIMEOUT bit set.

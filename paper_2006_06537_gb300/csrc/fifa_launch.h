@@ -86,7 +86,8 @@ cudaError_t launch_sweep_level(const FactDesc* Fd, int prec, int lvl, int nodes,
 // Fused sweep (one cooperative launch of 2^ls CTAs; rows >= the longest
 // level-ls node).  part: 2 ls slots of 2^ls x cap x SWEEP_RHS_MAX doubles; bar,
 // zeroed before: the abort flag, then a counter per node of the levels < ls for
-// each of two sweeps.
+// each of two sweeps.  cluster (2^ls <= 8): one cluster instead, which meets at its
+// hardware barrier and uses no bar.
 #define FS_BAR_COUNTERS 16
 inline size_t fs_bar_uints(int ls) { return FS_BAR_COUNTERS + ((size_t)2 << ls); }
 #define FS_CTAS_MAX 1024
@@ -105,7 +106,8 @@ cudaError_t launch_sweep_fused_batched(const FactDesc* Fd, int ls, int rows, dou
                                        int mode, double* part, unsigned int* bar, int* abort_flag, size_t pstride,
                                        cudaStream_t st);
 // Fused H-matrix product (one cooperative launch of 2^ls CTAs, rows <= 4096).
-// part: 2^ls * ls * MV_PART_STRIDE doubles; bar, zeroed before: abort flag and counter.
+// part: 2^ls * ls * MV_PART_STRIDE doubles; bar, zeroed before: abort flag and counter
+// (cluster: not used).
 #define MV_FUSED_ROWS_MAX 4096
 #define MV_BAR_UINTS 2
 int mv_fused_coresident(int rows);

@@ -313,7 +313,9 @@ __global__ void __launch_bounds__(256) k_sweep_leaf(const FactDesc* __restrict__
 // without its zeros: Z = [0 0; K Y] (the capacitance's factor is [I 0; M^T L2]),
 // so t is zero on the left side for Z, and Z^T takes p from the right side
 // alone.  A CTA left of the split hands over its partial and goes on; the right
-// ones wait for the CTAs of their own node only (a counter per node).
+// ones wait for the CTAs of their own node only (a counter per node).  Launched as
+// one cluster (contexts with independent CTAs), nothing polls: every CTA passes
+// one hardware barrier of the cluster per level.
 //
 // What bounds it: up to n ~ 2^17 the chain of levels < ls (a barrier of the
 // whole grid and loads behind it cost ~17 us per level; now 5 to 8), beyond that
@@ -552,11 +554,13 @@ __device__ __forceinline__ int lanes_for(int K) {
 // one child (side).  The CTAs hand over their partial projections in FP64
 // (`part`, this level's slots) and count themselves in at their node's counter.
 // What the level needs is in buffer `buf` (fs_stage, the oldest group of
-// copies) or still in global memory.  Returns false if the wait gave up.
+// copies) or still in global memory.  cluster: the launch's CTAs are one cluster
+// and meet at its barrier instead, all of them at every level.  Returns false if
+// the wait gave up.
 template <typename T, int NR>
 __device__ bool fs_global_level(const FactDesc* __restrict__ Fd, int l, int ls, int c, int r, T* vs, int rows, int S,
                                 int E, int zsel, int zt, double* __restrict__ part, int buf, unsigned int* counter,
-                                int* abort_flag, FsShared<T>& sh) {
+                                int* abort_flag, bool cluster, FsShared<T>& sh) {
   constexpr int nrhs = NR;
   const int tid = threadIdx.x, R = E - S;
   const int cap = Fd->cap, ld2 = 2 * cap, pstr = cap * SW_RHS_MAX;
@@ -566,7 +570,10 @@ __device__ bool fs_global_level(const FactDesc* __restrict__ Fd, int l, int ls, 
   const bool staged = r * R <= sh.qcap && 2 * r * r <= FS_ZBUF;
   asm volatile("cp.async.wait_group 1;" ::: "memory");  // this level's copies; the next level's may be in flight
   __syncthreads();                                       // ... every thread's, and v is up to date
-  if (r == 0) return true;                               // (for every CTA of the node: none waits)
+  if (r == 0) {                                          // (for every CTA of the node: none waits)
+    if (cluster) cluster_sync_all();                     // (other nodes of the level may have a rank)
+    return true;
+  }
   const T* Qb = (const T*)Fd->Q + (size_t)l * cap * n;
   const T* q = staged ? sh.qb + buf * sh.qcap : Qb + S;  // column a at q + a * qs, from row S
   const size_t qs = staged ? (size_t)R : (size_t)n;
@@ -597,16 +604,22 @@ __device__ bool fs_global_level(const FactDesc* __restrict__ Fd, int l, int ls, 
         if (nrhs > 1) __stcg(part + (size_t)c * pstr + a * nrhs + 1, (double)acc1);
       }
     }
-    __syncthreads();
-    if (tid == 0) {
-      __threadfence();
-      atomicAdd(counter, 1u);
+    if (!cluster) {
+      __syncthreads();
+      if (tid == 0) {
+        __threadfence();
+        atomicAdd(counter, 1u);
+      }
     }
+  }
+  if (cluster) {
+    __syncthreads();
+    cluster_sync_all();
   }
   if (!zt && !side) return true;  // the left rows keep their values
   // wait for the CTAs that hand over: both halves, or the right one
   __shared__ int arrived;
-  if (tid == 0) {
+  if (tid == 0 && !cluster) {
     const unsigned int target = zt ? half : 2 * half;
     const unsigned int limit = Fd->spin ? Fd->spin : FIFA_SPIN_LIMIT;
     unsigned int spins = 0;
@@ -627,8 +640,10 @@ __device__ bool fs_global_level(const FactDesc* __restrict__ Fd, int l, int ls, 
     __threadfence();
     arrived = ok;
   }
-  __syncthreads();
-  if (!arrived) return false;
+  if (!cluster) {
+    __syncthreads();
+    if (!arrived) return false;
+  }
   // p (left entries, then right ones; right ones alone for Z^T)
   {
     const int K2 = zt ? K : 2 * K, w = lanes_for(K2), ch = tid & (w - 1);
@@ -885,13 +900,14 @@ __device__ void fw_block_level(const FactDesc* __restrict__ Fd, int l, int lw, i
 // longest level-ls node), then the FsShared arrays.  vlist (nullable): several
 // factors of one plan in one launch, problem blockIdx.y: its descriptor
 // Fd[blockIdx.y], its vector vlist[blockIdx.y], its partials, barrier and
-// abort flag pstride bytes after the previous problem's.
+// abort flag pstride bytes after the previous problem's.  cluster: the grid is one
+// cluster (bar and abort_flag are not used then).
 template <typename T, int NR, bool BATCH = false>
 __global__ void __launch_bounds__(256, 4) k_sweep_fused(const FactDesc* __restrict__ Fd, double* __restrict__ v,
                                                         int mode, int ls, int rows, double* __restrict__ part,
                                                         unsigned int* __restrict__ bar, int* __restrict__ abort_flag,
                                                         const int* __restrict__ active, double* const* vlist,
-                                                        size_t pstride) {
+                                                        size_t pstride, bool cluster) {
   constexpr int nrhs = NR;
   if (active && *active == 0) return;
   // (a separate instantiation: re-pointed arguments live in registers for the
@@ -1004,7 +1020,8 @@ __global__ void __launch_bounds__(256, 4) k_sweep_fused(const FactDesc* __restri
       else asm volatile("cp.async.commit_group;" ::: "memory");
       ok = fs_global_level<T, NR>(Fd, l, ls, c, rkg[l], vs, rows, S, E, zsel, zt,
                                   part + (size_t)(pass * ls + l) * gridDim.x * pstr, buf,
-                                  bar + FS_BAR_COUNTERS + (pass << ls) + node_id(l, c >> (ls - l)), abort_flag, sh);
+                                  bar + FS_BAR_COUNTERS + (pass << ls) + node_id(l, c >> (ls - l)), abort_flag, cluster,
+                                  sh);
       buf ^= 1;
     }
     __syncthreads();
@@ -1075,13 +1092,12 @@ int sweep_fused_coresident(int prec, int rows, int cap) {
 template <typename T, int NR, bool BATCH = false>
 static cudaError_t launch_sweep_fused_t(cudaLaunchConfig_t& cfg, const FactDesc* Fd, double* v, int mode, int ls,
                                         int rows, double* part, unsigned int* bar, int* abort_flag,
-                                        const int* active, int prec, double* const* vlist = nullptr,
+                                        const int* active, bool cluster, double* const* vlist = nullptr,
                                         size_t pstride = 0) {
-  (void)prec;
   const cudaError_t e = ALLOW_SMEM(k_sweep_fused<T, NR, BATCH>);
   if (e != cudaSuccess) return e;
   return cudaLaunchKernelEx(&cfg, k_sweep_fused<T, NR, BATCH>, Fd, v, mode, ls, rows, part, bar, abort_flag, active,
-                            vlist, pstride);
+                            vlist, pstride, cluster);
 }
 
 // nprob FP64 factors of one plan (descriptor array Fd), one right-hand side
@@ -1099,8 +1115,8 @@ cudaError_t launch_sweep_fused_batched(const FactDesc* Fd, int ls, int rows, dou
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return launch_sweep_fused_t<double, 1, true>(cfg, Fd, nullptr, mode, ls, rows, part, bar, abort_flag, nullptr, 0,
-                                               vlist, pstride);
+  return launch_sweep_fused_t<double, 1, true>(cfg, Fd, nullptr, mode, ls, rows, part, bar, abort_flag, nullptr,
+                                               false, vlist, pstride);
 }
 
 cudaError_t launch_sweep_fused(const FactDesc* Fd, int prec, int ls, int rows, int cap, double* v, int nrhs,
@@ -1125,10 +1141,10 @@ cudaError_t launch_sweep_fused(const FactDesc* Fd, int prec, int ls, int rows, i
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   if (prec)
-    return nrhs > 1 ? launch_sweep_fused_t<float, 2>(cfg, Fd, v, mode, ls, rows, part, bar, abort_flag, active, prec)
-                    : launch_sweep_fused_t<float, 1>(cfg, Fd, v, mode, ls, rows, part, bar, abort_flag, active, prec);
-  return nrhs > 1 ? launch_sweep_fused_t<double, 2>(cfg, Fd, v, mode, ls, rows, part, bar, abort_flag, active, prec)
-                  : launch_sweep_fused_t<double, 1>(cfg, Fd, v, mode, ls, rows, part, bar, abort_flag, active, prec);
+    return nrhs > 1 ? launch_sweep_fused_t<float, 2>(cfg, Fd, v, mode, ls, rows, part, bar, abort_flag, active, cluster)
+                    : launch_sweep_fused_t<float, 1>(cfg, Fd, v, mode, ls, rows, part, bar, abort_flag, active, cluster);
+  return nrhs > 1 ? launch_sweep_fused_t<double, 2>(cfg, Fd, v, mode, ls, rows, part, bar, abort_flag, active, cluster)
+                  : launch_sweep_fused_t<double, 1>(cfg, Fd, v, mode, ls, rows, part, bar, abort_flag, active, cluster);
 }
 
 // ---------------------------------------------------------------------------
@@ -1218,7 +1234,8 @@ cudaError_t launch_predict(const HmatDesc* Hd, const FactDesc* Fd, int64_t n, co
 // (whose nodes lie in the CTA) need nothing from other CTAs; each level < ls
 // needs the projection of the partner child, which spans other CTAs.  Every CTA
 // hands over its partial projections for all those levels first, works on the
-// leaves and its own levels meanwhile, and then waits once for all CTAs and sums
+// leaves and its own levels meanwhile, and then waits once for all CTAs (at a
+// counter, or, launched as one cluster, at the cluster's hardware barrier) and sums
 // the partner halves' partials.
 //   row p in the left child of a level-l node:  y_p += U_p (V^T x_right)
 //   row p in the right child:                   y_p += V_p (U^T x_left)
@@ -1254,7 +1271,8 @@ template <int RPT, bool BATCH = false>
 __global__ void __launch_bounds__(RPT == 1 ? MV_THREADS_MAX : 256, RPT <= 8 ? 4 : 2)
     k_mv_fused(const HmatDesc* __restrict__ Hd, const double* __restrict__ x, int nrhs, double* __restrict__ y, int ls,
                int rows, int hs_arg, int rp, double* __restrict__ part, unsigned int* __restrict__ bar,
-               const int* __restrict__ active, const double* const* xlist, double* const* ylist, size_t pstride) {
+               const int* __restrict__ active, const double* const* xlist, double* const* ylist, size_t pstride,
+               bool cluster) {
   if (active && *active == 0) return;  // a converged iteration: nothing to compute
   if constexpr (BATCH) {
     Hd += blockIdx.y;
@@ -1316,7 +1334,9 @@ __global__ void __launch_bounds__(RPT == 1 ? MV_THREADS_MAX : 256, RPT <= 8 ? 4 
       }
     }
     __syncthreads();
-    if (tid == 0) {
+    if (cluster) {
+      cluster_arrive();
+    } else if (tid == 0) {
       __threadfence();
       atomicAdd(bar + 1, 1u);
     }
@@ -1397,7 +1417,10 @@ __global__ void __launch_bounds__(RPT == 1 ? MV_THREADS_MAX : 256, RPT <= 8 ? 4 
   }
   if (ls > 0) {
     // every CTA's partials are written (a bounded wait; a launch's CTAs are all resident)
-    if (tid == 0) {
+    if (cluster) {
+      __syncthreads();
+      cluster_wait();
+    } else if (tid == 0) {
       volatile int* abort_flag = (volatile int*)bar;
       const unsigned int limit = Hd->spin ? Hd->spin : FIFA_SPIN_LIMIT;
       unsigned int spins = 0;
@@ -1418,8 +1441,10 @@ __global__ void __launch_bounds__(RPT == 1 ? MV_THREADS_MAX : 256, RPT <= 8 ? 4 
       __threadfence();
       arrived = ok;
     }
-    __syncthreads();
-    if (!arrived) return;
+    if (!cluster) {
+      __syncthreads();
+      if (!arrived) return;
+    }
   }
   // levels < ls, as many at a time as fit pj: the partner halves' projections,
   // then the rows' sums
@@ -1563,7 +1588,7 @@ static cudaError_t launch_mv_fused_t(const HmatDesc* Hd, int ls, int rows, const
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, k_mv_fused<RPT, BATCH>, Hd, x, nrhs, y, ls, rows, sh.hs, sh.rp, part, bar, active,
-                            xlist, ylist, pstride);
+                            xlist, ylist, pstride, cluster);
 }
 
 // nprob H-matrices of one plan (descriptor array Hd), one right-hand side each

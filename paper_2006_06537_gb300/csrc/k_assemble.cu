@@ -121,9 +121,6 @@ __device__ __forceinline__ double aca_value(const AcaBest& a) {
   return __longlong_as_double(a.v | ((long long)(a.p & 1) << 63));
 }
 
-__device__ __forceinline__ void aca_cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-}
 __device__ __forceinline__ AcaBest aca_remote(const AcaBest* p, int rank) {
   const unsigned a = (unsigned)__cvta_generic_to_shared(p);
   unsigned r;
@@ -193,7 +190,7 @@ __global__ void __launch_bounds__(256, 4) k_aca(const HmatDesc* __restrict__ Hd,
     if (G > 1) {
       if constexpr (CL) {
         if (tid == 0) cbest[phase & 1u] = a;
-        aca_cluster_sync();
+        cluster_sync_all();
         a = aca_remote(&cbest[phase & 1u], min(lane & 7, G - 1));
         aca_shuffle<4>(a);
       } else {
@@ -297,7 +294,7 @@ __global__ void __launch_bounds__(256, 4) k_aca(const HmatDesc* __restrict__ Hd,
       if (nb.v < 0) break;
       i = nb.p >> 1;
     }
-  if (CL && G > 1) aca_cluster_sync();  // no CTA leaves while another may still read its maxima
+  if (CL && G > 1) cluster_sync_all();  // no CTA leaves while another may still read its maxima
   if (g == 0 && threadIdx.x == 0) {
     Hd->rank[nid] = k;
     for (int l = 0; l < cap; ++l) {

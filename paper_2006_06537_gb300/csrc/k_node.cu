@@ -53,9 +53,6 @@ struct NdLayout {
   }
 };
 
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-}
 // Load a double of the same shared-memory variable in CTA `rank` of the cluster.
 __device__ __forceinline__ double ld_cluster(const double* p, int rank) {
   unsigned a = (unsigned)__cvta_generic_to_shared(p), r;
