@@ -91,22 +91,33 @@ static int levels_for(int64_t n, int B) {
 // meet at its barrier, so nothing polls and opts.wait_polls does not apply) instead
 // of two launches per tree level.
 static bool one_cluster(int64_t n) { return n <= 8192; }
+#define FUSED_CLUSTER_LEVELS 3  // eight CTAs
+
+// CTAs and levels above them of the largest fused launch of a plan (0 CTAs: none,
+// no CTA hands anything over).
+struct FusedMax {
+  int ctas, levels;
+};
+static FusedMax fused_max(const Plan* P, const fifa_opts& o) {
+  if (!o.independent_ctas) return {std::min(P->nleaf, FS_CTAS_MAX), std::max(1, std::min(P->L, 10))};
+  if (!one_cluster(P->n)) return {0, 0};
+  return {std::min(P->nleaf, 1 << FUSED_CLUSTER_LEVELS), std::max(1, std::min(P->L, FUSED_CLUSTER_LEVELS))};
+}
 
 // Partials of the fused sweep: one projection per CTA, level and sweep (a solve
-// has two), for up to min(nleaf, FS_CTAS_MAX) CTAs (none with independent CTAs:
-// no CTA hands anything over).
+// has two).
 static size_t fused_sweep_part_doubles(const Plan* P, const fifa_opts& o) {
-  if (o.independent_ctas && !one_cluster(P->n)) return 1;
-  return (size_t)2 * std::max(1, std::min(P->L, 10)) * std::min(P->nleaf, FS_CTAS_MAX) * o.rank_cap * SWEEP_RHS_MAX;
+  const FusedMax f = fused_max(P, o);
+  return (size_t)2 * f.levels * f.ctas * o.rank_cap * SWEEP_RHS_MAX + 1;
 }
 // Bytes of its abort flag and counters.
 static size_t fused_sweep_bar_bytes(const Plan* P) { return sizeof(unsigned int) * fs_bar_uints(std::min(P->L, 10)); }
 
 // Partials of the fused H-matvec: one projection per CTA and level below the
-// CTA level, for up to min(nleaf, FS_CTAS_MAX) CTAs and 10 such levels.
+// CTA level.
 static size_t fused_mv_part_doubles(const Plan* P, const fifa_opts& o) {
-  if (o.independent_ctas && !one_cluster(P->n)) return 1;
-  return (size_t)std::min(P->nleaf, FS_CTAS_MAX) * std::max(1, std::min(P->L, 10)) * FIFA_CAP_MAX * SWEEP_RHS_MAX;
+  const FusedMax f = fused_max(P, o);
+  return (size_t)f.ctas * f.levels * FIFA_CAP_MAX * SWEEP_RHS_MAX + 1;
 }
 
 // Level barriers: one set per rank bucket of every level with CTA groups, so one
@@ -230,7 +241,8 @@ static Plan* plan_build(int64_t n, const fifa_opts& o, int aca_cores, const int*
   add(sizeof(unsigned int) * std::max(1, P->aca_ncoop));         // ACA barriers
   int64_t lvl_ctas = 1, sweep_ctas = 1;
   for (int l = 0; l < P->L; ++l) {
-    for (int b = 0; b < LEVEL_BUCKETS; ++b) lvl_ctas = std::max<int64_t>(lvl_ctas, ((int64_t)1 << l) * P->lvl_G[b][l]);
+    for (int b = 0; b < LEVEL_BUCKETS; ++b)  // (only the CTAs of groups exchange through partials and barriers)
+      if (P->lvl_G[b][l] > 1) lvl_ctas = std::max<int64_t>(lvl_ctas, ((int64_t)1 << l) * P->lvl_G[b][l]);
     sweep_ctas = std::max<int64_t>(sweep_ctas, ((int64_t)1 << l) * P->sweep_G[l]);
   }
   P->lvl_ctas_max = (int)lvl_ctas;
@@ -339,7 +351,7 @@ Plan* get_plan(fifa_ctx* ctx, int64_t n, fifa_status* st) {
       }
     }
   } else if (one_cluster(n)) {
-    const int k = std::min(P->L, 3);
+    const int k = std::min(P->L, FUSED_CLUSTER_LEVELS);
     int rows = 0;
     for (int i = 0; i < (1 << k); ++i)
       rows = std::max(rows, P->bnd_host[bnd_off(k) + i + 1] - P->bnd_host[bnd_off(k) + i]);

@@ -28,7 +28,7 @@ struct Plan {
   std::vector<int4> work_host;
   size_t work_off = 0, dev_bytes = 0;  // device block: bounds, then the work list at work_off
   std::vector<int> lvl_G[3], sweep_G;  // lvl_G[b]: group size of the level kernel of rank bucket b
-  int lvl_ctas_max = 1;
+  int lvl_ctas_max = 1;  // most CTAs of a level whose nodes have groups
   int lvl_grouped = 0;  // levels 0 .. lvl_grouped - 1 have CTA groups
   int fs_ls = -1, fs_rows = 0;  // fused sweep: 2^fs_ls CTAs of fs_rows rows (-1: per-level sweeps)
   bool cluster = false;  // fused sweep and product launched as one cluster (independent CTAs)
