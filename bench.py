@@ -737,7 +737,8 @@ def additive_leg(fifa, torch, sweeps, leaf, n=65536, d=4):
 def factor_work(n, leaf, ranks):
     """Algorithmic FP64 flops of one HODLR factorization (per level too), from
     the per-node ranks (heap order): leaf m^3/3 + m^2 C_anc, levels 4 r^2 m
-    (CholeskyQR2) + 4 r C_anc m (ancestor update)."""
+    (CholeskyQR2) + 3 r C_anc m (projection of the ancestor columns, update of
+    the right half's rows: the inverse node factor leaves the left half's)."""
     L = 0
     while (n + (1 << L) - 1) >> L > leaf:
         L += 1
@@ -763,7 +764,7 @@ def factor_work(n, leaf, ranks):
         canc = np.zeros_like(r_l)
         for j in range(l):
             canc += np.repeat(ranks[(1 << j) - 1:(1 << (j + 1)) - 1], 1 << (l - j))
-        f = float(np.sum(4.0 * r_l * r_l * m + 4.0 * r_l * canc * m))
+        f = float(np.sum(4.0 * r_l * r_l * m + 3.0 * r_l * canc * m))
         lv.append(f)
         flops += f
     per_level += lv[::-1]
@@ -791,9 +792,10 @@ def apply_work(n, leaves_m, ranks, L, nrhs=2):
 
 def sweep_flops(n, leaves_m, ranks, L, nrhs=2):
     """FP64 flops of one W^-1 sweep: the leaf triangular solves (m^2 each) and
-    per level the projection and the update (2 r flops per row each)."""
+    per level the projection (2 r flops per row) and the update of the right
+    half's rows."""
     rank_rows = n * float(sum(ranks[(1 << l) - 1:(1 << (l + 1)) - 1].mean() for l in range(L)))
-    return float((np.sum(leaves_m ** 2) + 4 * rank_rows) * nrhs)
+    return float((np.sum(leaves_m ** 2) + 3 * rank_rows) * nrhs)
 
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum, summed over the 41
