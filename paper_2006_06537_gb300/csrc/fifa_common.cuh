@@ -259,18 +259,6 @@ __device__ inline void blk_triinv_upper(const double* R, int ldr, double* Ri, in
   __syncthreads();
 }
 
-// Li = L^-1 for lower-triangular L (r x r); one thread per column.
-__device__ inline void blk_triinv_lower(const double* Lm, int ldl, double* Li, int ldi, int r) {
-  for (int j = threadIdx.x; j < r; j += blockDim.x) {
-    for (int i = 0; i < r; ++i) {
-      double acc = (i == j) ? 1.0 : 0.0;
-      for (int k = j; k < i; ++k) acc -= Lm[i * ldl + k] * Li[k * ldi + j];
-      Li[i * ldi + j] = (i >= j) ? acc / Lm[i * ldl + i] : 0.0;
-    }
-  }
-  __syncthreads();
-}
-
 template <typename T> __device__ __forceinline__ double to_d(T v) { return (double)v; }
 
 // Hardware barrier of the CTAs of a thread-block cluster, in two halves: what a

@@ -24,10 +24,10 @@
 #include "fifa_launch.h"
 #include "fifa_level.cuh"
 
-// Ancestor columns per right-hand-side chunk of the leaf TRSM: the first chunk
-// is eliminated together with the Cholesky steps, later chunks (more ancestor
-// columns than this) by a separate triangular solve.
-__host__ __device__ inline int lf_nch(int Bm) { return Bm <= 64 ? 64 : 32; }
+// Leaves of up to 64 rows.  Ancestor columns per right-hand-side chunk of the leaf
+// TRSM: the first chunk is eliminated together with the Cholesky steps, later
+// chunks (more ancestor columns than this) by a separate triangular solve.
+#define LF_NCH 64
 
 template <typename T>
 __global__ void __launch_bounds__(256, 7)
@@ -42,7 +42,8 @@ __global__ void __launch_bounds__(256, 7)
   const double sc = Hd->scale, shf = Hd->shift;
   const int* bnd = Fd->bnd;
   const int s = bnd[bnd_off(L) + leaf], e = bnd[bnd_off(L) + leaf + 1], m = e - s;
-  const int ld = Bm + 1, NCH = lf_nch(Bm);
+  constexpr int NCH = LF_NCH;
+  const int ld = Bm + 1;
   double* A = sm;                          // FP64 Cholesky, column-major A[j*ld + i]
   T* La = sizeof(T) == sizeof(double) ? (T*)A : (T*)(A + (size_t)Bm * ld);  // L in the TRSM precision
   T* X = (T*)(A + (size_t)Bm * ld + (sizeof(T) == sizeof(double) ? 0 : ((size_t)Bm * ld + 1) / 2));
@@ -689,9 +690,8 @@ __global__ void __launch_bounds__(256, 2)
   double* Ri2 = Ri + cc2;                 // the packed Gram entries of both sides span them)
   double* RU = Ri2 + cc2;                 // R1, then R = R2 R1 of the left side
   double* RV = RU + cc2;                  // ... of the right side
-  double* rvs = RV + cc2;                 // 2 x 8 reciprocal pivots (serial small factorizations)
   const int tbuf = (ldm + W) * LV_TRP;    // doubles per row tile
-  double* tile = rvs + 16;                // two (ldm + W) x LV_TRP row tiles
+  double* tile = RV + cc2;                // two (ldm + W) x LV_TRP row tiles
   double* part = tile + 2 * tbuf;         // 256 group partial sums
   double* tmp = part + 256;               // LV_RED
   double* Pm = tmp + LV_RED;              // 2ldm x W
@@ -709,7 +709,6 @@ __global__ void __launch_bounds__(256, 2)
   // while the other side is factored
   const int npk = r * (r + 1) / 2;
   const int sa0 = max(r0, s), sa1 = min(r1, h), sb0 = max(r0, h), sb1 = min(r1, e);
-  if (threadIdx.x == 0) iflag[2] = 0;
   for (int pass = 0; pass < 2; ++pass) {
     gram_tiled<T>(Qb, n, r, sa0, sa1, tile, tbuf, part, Ri);
     gram_tiled<T>(Qb, n, r, sb0, sb1, tile, tbuf, part, Ri + npk);
@@ -738,7 +737,6 @@ __global__ void __launch_bounds__(256, 2)
     rowmul_pass<T>(Qb, n, r, sa0, sa1, Ri, ldm);
     rowmul_pass<T>(Qb, n, r, sb0, sb1, Ri2, ldm);
   }
-  ok = ok && iflag[2] == 0;
   if (!ok && g == 0 && threadIdx.x == 0) atomicOr(status, FIFA_DEV_NOT_SPD);
 
   // capacitance: S = I + R X R^T, L_S = chol(S) (computed by the group's first CTA)
@@ -1260,13 +1258,13 @@ size_t leaf_factor_smem(int Bm, int L, int cap, int prec) {
   const size_t ld = Bm + 1;
   size_t b = (size_t)Bm * ld * sizeof(double);                   // FP64 Cholesky
   if (prec) b += ((size_t)Bm * ld + 1) / 2 * sizeof(double);      // FP32 copy of L
-  b += (size_t)lf_nch(Bm) * ld * (prec ? sizeof(float) : sizeof(double));  // right-hand sides
+  b += (size_t)LF_NCH * ld * (prec ? sizeof(float) : sizeof(double));  // right-hand sides
   b += 16 + 40 * sizeof(double) + (4 + (size_t)L * cap) * sizeof(int);
   return b;
 }
 static size_t level_wide_smem(int cap) {
   const size_t W = LEVEL_W, ldm = cap;
-  return ((size_t)6 * ldm * ldm + 16 + 2 * (size_t)(ldm + W) * LV_TRP + 256 + LV_RED + 4 * (size_t)ldm * W) * sizeof(double) +
+  return ((size_t)6 * ldm * ldm + 2 * (size_t)(ldm + W) * LV_TRP + 256 + LV_RED + 4 * (size_t)ldm * W) * sizeof(double) +
          W * sizeof(void*) + (4 + (size_t)FIFA_LEVELS_MAX * cap) * sizeof(int);
 }
 
