@@ -307,6 +307,11 @@ extern "C" fifa_status fifa_plan_describe(const fifa_opts* opts, int64_t n, int 
 // 43/37/40 us; n = 65537 114/111/127, 250/250/299, 70/65/78 us; n = 131072 (Matern)
 // 203/160/167, 500/460/486, 153/111/111 us; n = 300007 388/299/275, 861/644/630,
 // 262/176/145 us; n = 8192 at 2^6, 2^7, 2^8: 59/58/66, 114/111/137, 35/29/31 us.
+// Between 2^17 and 2^18, at 2^8 / 2^9 CTAs (the latter of 257 to 512 rows, which
+// are co-resident only if none are staged), W^-1 (two vectors), FP32 solve (one) and
+// product (one, two): n = 160000 223/220, 173/202, 100/102, 137/149; n = 200000
+// 253/259, 221/232, 117/112, 163/172; n = 262143 290/283, 221/210, 147/138, 202/212
+// us: the crossing is near the line.
 static int fused_ctas(int64_t n, int small) {
   if (n >= (int64_t)1 << 18) return FS_CTAS_MAX;
   const int64_t most = n < 32768 ? small : 256;
