@@ -100,6 +100,9 @@ int sweep_fused_coresident(int prec, int rows, int cap);
 cudaError_t launch_sweep_fused(const FactDesc* Fd, int prec, int ls, int rows, int cap, double* v, int nrhs,
                                int mode, double* part, unsigned int* bar, int* abort_flag, bool cluster,
                                cudaStream_t st, const int* active = nullptr);
+// (k_apply_cluster.cu) the same as one cluster of 2^ls <= 8 CTAs
+cudaError_t launch_sweep_cluster(const FactDesc* Fd, int prec, int ls, int rows, double* v, int nrhs, int mode,
+                                 double* part, cudaStream_t st, const int* active = nullptr);
 // nprob FP64 factors of one plan in one launch (one right-hand side each at
 // vlist[q]; per-problem partials / barrier / abort flag pstride bytes apart)
 cudaError_t launch_sweep_fused_batched(const FactDesc* Fd, int ls, int rows, double* const* vlist, int nprob,
@@ -113,6 +116,9 @@ cudaError_t launch_sweep_fused_batched(const FactDesc* Fd, int ls, int rows, dou
 int mv_fused_coresident(int rows);
 cudaError_t launch_mv_fused(const HmatDesc* Hd, int ls, int rows, const double* x, int nrhs, double* y, double* part,
                             unsigned int* bar, bool cluster, cudaStream_t st, const int* active = nullptr);
+// (k_apply_cluster.cu) the same as one cluster of 2^ls <= 8 CTAs, rows <= 1024
+cudaError_t launch_mv_cluster(const HmatDesc* Hd, int ls, int rows, const double* x, int nrhs, double* y, double* part,
+                              cudaStream_t st, const int* active = nullptr);
 // nprob H-matrices of one plan in one launch (one right-hand side each:
 // xlist[q] -> ylist[q]; per-problem partials and abort flag / counter pstride
 // bytes apart)

@@ -7,7 +7,7 @@
 //              factor.  W32 W32^T is then a symmetric positive definite
 //              preconditioner whose relative distance to the factored matrix is
 //              about sqrt(kappa) u32 (W is only as ill-conditioned as the square
-//              root of M~), applied by the FP32 sweeps of k_apply.cu.
+//              root of M~), applied by the FP32 sweeps of fifa_apply.cuh.
 //  k_pcg_*     conjugate gradients preconditioned by W32 W32^T on the FP64
 //              operator M~ (the current one; the factor may belong to an
 //              earlier M~ of the chain), for up to two right-hand sides, with

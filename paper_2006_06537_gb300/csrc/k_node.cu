@@ -28,7 +28,7 @@
 // Against three exchanges and more per level, one-thread algebra and an update of
 // both sides: a level of n = 2048 (64-row leaves, ranks to 14) 128-189 -> 33-80
 // us; one factorization of n = 2^20 (clustered inputs, ranks 2 to 7) 11.8 -> 10.6
-// ms with the leaf factor's changes, its levels at 46-67% of the FP64 peak.
+// ms with the leaf factor's changes, its levels at 45-68% of the FP64 peak.
 #include <algorithm>
 #include <atomic>
 
