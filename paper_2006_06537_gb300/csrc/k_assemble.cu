@@ -198,12 +198,19 @@ __global__ void __launch_bounds__(256, 4) k_aca(const HmatDesc* __restrict__ Hd,
         ArgMax* mine = part + 2 * (base + g) + (phase & 1u);
         if (tid == 0) *mine = ArgMax{__longlong_as_double(a.v), a.p, __longlong_as_double(a.u)};
         if (!group_barrier(bar + base, G * (phase + 1), Hd->status, abort_flag, Hd->spin)) dead = true;
+        // a slot to a thread (every warp reading all of them moved 8 times as much
+        // out of L2: 3 us a phase for 589 CTAs), then as above; wb is free again
+        // since the barrier
         a = aca_none();
-        for (int q = lane; q < G && !dead; q += 32) {
+        for (int q = tid; q < G && !dead; q += blockDim.x) {
           const ArgMax* pq = part + 2 * (base + q) + (phase & 1u);
           aca_take(a, AcaBest{__double_as_longlong(__ldcg(&pq->v)), __double_as_longlong(__ldcg(&pq->sv)), __ldcg(&pq->i)});
         }
         aca_shuffle<16>(a);
+        if (lane == 0) wb[warp] = a;
+        __syncthreads();
+        a = wb[lane & 7];
+        aca_shuffle<4>(a);
       }
     }
     ++phase;
