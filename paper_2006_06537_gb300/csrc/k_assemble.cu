@@ -86,8 +86,9 @@ __global__ void __launch_bounds__(256) k_leaf_assemble(const HmatDesc* __restric
 // memory as far as they fit (ACA_KEEP doubles), the pivot row's U entries come
 // in one load, and a reduction is one shuffle tree per warp, one exchange in
 // shared memory and a second tree in every warp: n = 500, 15 blocks, 400 us in
-// two launches -> 98 in one; 0.94 -> 0.92 ms for the grouped blocks of n = 300007,
-// which the FP64 pipe bounds.
+// two launches -> 98 in one; 0.94 -> 0.91 ms for the grouped blocks of n = 200000,
+// which the FP64 pipe bounds.  KEEP = false keeps nothing and leaves that memory to
+// the L1 cache.
 // ---------------------------------------------------------------------------
 #define ACA_KEEP 5632  // doubles of U and V kept per CTA (four CTAs per SM)
 
@@ -132,7 +133,7 @@ __device__ __forceinline__ AcaBest aca_remote(const AcaBest* p, int rank) {
   return b;
 }
 
-template <bool CL>
+template <bool CL, bool KEEP>
 __global__ void __launch_bounds__(256, 4) k_aca(const HmatDesc* __restrict__ Hd, const int4* __restrict__ work, int C,
                                               AcaGroups groups,
                                               ArgMax* __restrict__ part, unsigned int* __restrict__ bar,
@@ -174,7 +175,7 @@ __global__ void __launch_bounds__(256, 4) k_aca(const HmatDesc* __restrict__ Hd,
   __shared__ int rowp[FIFA_CAP_MAX], colp[FIFA_CAP_MAX];
   __shared__ double piv_row[FIFA_CAP_MAX];  // the pivot row's U entries, then the pivot column's V entries
   __shared__ AcaBest wbest[2][8], cbest[2];
-  const int kl = min(cap, ACA_KEEP / (rc + cc)), kstep = rc + cc;
+  const int kl = KEEP ? min(cap, ACA_KEEP / (rc + cc)) : 0, kstep = rc + cc;
   unsigned int phase = 0;
 
   // reduce over the node's CTAs; two buffers in turn, each written again only
@@ -218,10 +219,12 @@ __global__ void __launch_bounds__(256, 4) k_aca(const HmatDesc* __restrict__ Hd,
   };
   // acc - sum_{l < k} piv_row[l] (this CTA's entry q of V or U in step l)
   auto residual = [&](double acc, int k, const double* kp, const double* gp) {
-    const int k1 = min(k, kl);
     int l = 0;
+    if constexpr (KEEP) {
+      const int k1 = min(k, kl);
 #pragma unroll 4
-    for (; l < k1; ++l) acc = __fma_rn(-piv_row[l], kp[l * kstep], acc);
+      for (; l < k1; ++l) acc = __fma_rn(-piv_row[l], kp[l * kstep], acc);
+    }
 #pragma unroll 4
     for (; l < k; ++l) acc = __fma_rn(-piv_row[l], gp[(size_t)l * n], acc);
     return acc;
@@ -242,7 +245,7 @@ __global__ void __launch_bounds__(256, 4) k_aca(const HmatDesc* __restrict__ Hd,
       for (int j = c0 + tid; j < c1; j += blockDim.x) {
         const double en = j == c0 + tid ? first : kern_entry(kind, kc, xi, x[h + j]);
         const double acc = residual(en, k, keep + (j - c0), Bs + h + j);
-        if (k < kl) keep[k * kstep + (j - c0)] = acc;
+        if (KEEP && k < kl) keep[k * kstep + (j - c0)] = acc;
         else Bs[(size_t)k * n + h + j] = acc;
         // an entry that would win is checked against the used columns (the
         // check runs only then: same result as checking every entry)
@@ -267,7 +270,7 @@ __global__ void __launch_bounds__(256, 4) k_aca(const HmatDesc* __restrict__ Hd,
       if (r0 + tid < r1) first = kern_entry(kind, kc, x[s + r0 + tid], xj);
       for (int j = c0 + tid; j < c1; j += blockDim.x) {
         double* vp = Bs + (size_t)k * n + h + j;
-        if (k < kl) *vp = keep[k * kstep + (j - c0)] = __dmul_rn(keep[k * kstep + (j - c0)], rpiv);
+        if (KEEP && k < kl) *vp = keep[k * kstep + (j - c0)] = __dmul_rn(keep[k * kstep + (j - c0)], rpiv);
         else *vp = __dmul_rn(*vp, rpiv);
       }
       __syncthreads();
@@ -276,7 +279,7 @@ __global__ void __launch_bounds__(256, 4) k_aca(const HmatDesc* __restrict__ Hd,
       for (int ii = r0 + tid; ii < r1; ii += blockDim.x) {
         const double en = ii == r0 + tid ? first : kern_entry(kind, kc, x[s + ii], xj);
         const double acc = residual(en, k, keep + cc + (ii - r0), Bs + s + ii);
-        if (k < kl) keep[k * kstep + cc + (ii - r0)] = acc;
+        if (KEEP && k < kl) keep[k * kstep + cc + (ii - r0)] = acc;
         Bs[(size_t)k * n + s + ii] = acc;
         const AcaBest cand{__double_as_longlong(fabs(acc)), 0, 2 * ii + (__double2hiint(acc) < 0)};
         if (cand.v > nb.u) nb.u = cand.v;
@@ -433,12 +436,19 @@ static int aca_cluster(int64_t blocks, int span) {
   return c;
 }
 
-static cudaError_t launch_aca_cluster(const HmatDesc* Hd, const int4* work, int blocks, int C, cudaStream_t st,
+// Largest slice of U and V (rows and columns of a CTA) of which steps are kept: with
+// fewer than three of them in ACA_KEEP the L1 cache does better.  One assembly, kept /
+// not: 312 entries to a CTA 517/566 us, 1000 533/544, 2000 1180/1190, 2500 761/752,
+// 3125 1607/1561, 131072 14.85/14.14 ms.
+#define ACA_KEEP_SPAN 2048
+
+static cudaError_t launch_aca_cluster(const HmatDesc* Hd, const int4* work, int blocks, int C, int span, cudaStream_t st,
                                       int nprob) {
+  const bool keep = span <= ACA_KEEP_SPAN * C;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(blocks * C, nprob);
   cfg.blockDim = dim3(256);
-  cfg.dynamicSmemBytes = ACA_KEEP * sizeof(double);
+  cfg.dynamicSmemBytes = keep ? ACA_KEEP * sizeof(double) : 0;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -447,8 +457,8 @@ static cudaError_t launch_aca_cluster(const HmatDesc* Hd, const int4* work, int 
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_aca<true>, Hd, work, C, AcaGroups{}, (ArgMax*)nullptr, (unsigned int*)nullptr, (int*)nullptr,
-                            (size_t)0);
+  return cudaLaunchKernelEx(&cfg, keep ? k_aca<true, true> : k_aca<true, false>, Hd, work, C, AcaGroups{},
+                            (ArgMax*)nullptr, (unsigned int*)nullptr, (int*)nullptr, (size_t)0);
 }
 
 cudaError_t launch_leaf_assemble(const HmatDesc* Hd, int nleaf, cudaStream_t st, int nprob) {
@@ -468,14 +478,15 @@ cudaError_t launch_aca_blocks(const HmatDesc* Hd, const int4* work, int nsolo, i
   const bool small_warps = (int64_t)nwarp * nprob > 608;
   const int together = aca_cluster((int64_t)(nsolo + nwarp) * nprob, span);
   if (!small_warps && nsolo > 0 && nwarp > 0 && span <= 1024 * together)
-    return launch_aca_cluster(Hd, work, nsolo + nwarp, together, st, nprob);
+    return launch_aca_cluster(Hd, work, nsolo + nwarp, together, span, st, nprob);
   if (nsolo > 0) {
-    const cudaError_t e = launch_aca_cluster(Hd, work, nsolo, aca_cluster((int64_t)nsolo * nprob, span), st, nprob);
+    const cudaError_t e = launch_aca_cluster(Hd, work, nsolo, aca_cluster((int64_t)nsolo * nprob, span), span, st, nprob);
     if (e != cudaSuccess) return e;
   }
   if (nwarp <= 0) return cudaSuccess;
   if (!small_warps)
-    return launch_aca_cluster(Hd, work + nsolo, nwarp, aca_cluster((int64_t)nwarp * nprob, 2 * ACA_WARP_MAX), st, nprob);
+    return launch_aca_cluster(Hd, work + nsolo, nwarp, aca_cluster((int64_t)nwarp * nprob, 2 * ACA_WARP_MAX),
+                              2 * ACA_WARP_MAX, st, nprob);
   k_aca_warp<<<dim3((nwarp + 7) / 8, nprob), 256, 0, st>>>(Hd, work + nsolo, nwarp);
   return cudaGetLastError();
 }
@@ -493,14 +504,14 @@ cudaError_t launch_aca(const HmatDesc* Hd, const int4* work, int ncta, ArgMax* p
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_aca<false>, Hd, work, 1, groups ? *groups : AcaGroups{}, part, bar, abort_flag, pstride);
+  return cudaLaunchKernelEx(&cfg, k_aca<false, true>, Hd, work, 1, groups ? *groups : AcaGroups{}, part, bar, abort_flag, pstride);
 }
 
 int aca_max_coresident_ctas() {
   int dev = 0, sms = 0, per_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_aca<false>, 256, ACA_KEEP * sizeof(double)) != cudaSuccess)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_aca<false, true>, 256, ACA_KEEP * sizeof(double)) != cudaSuccess)
     per_sm = 1;
   return sms * per_sm;
 }
