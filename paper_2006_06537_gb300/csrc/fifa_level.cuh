@@ -112,14 +112,25 @@ __device__ __forceinline__ void tile_walk(double* tile, int tbuf, int ncol, int 
   }
 }
 
+// 1 / sqrt(d), d > 0: the hardware's approximation y refined by one step of
+// Householder's method of third order, y + y e (1/2 + 3/8 e) with e = 1 - d y^2
+// (what remains, about e^3, is far below the rounding): five FP64 instructions.
+// Where the approximation would flush a subnormal or d y overflow, the library's.
+__device__ __forceinline__ double rsqrt_householder(double d) {
+  const int ex = (__double2hiint(d) >> 20) & 0x7ff;
+  if (ex < 100 || ex > 1900) return rsqrt(d);
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+  const double e = fma(-(d * y), y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
 // One warp, in place: M (r x r symmetric, r <= 16, rows ld apart, upper triangle
 // read) = R^T R.  Leaves R above the diagonal of M, its diagonal in Rd, and
 // R^-T below and on the diagonal of M (1 / R_kk there).  Left-looking, lane =
 // column: row k of R (lanes > k) and of R^-T (lanes < k) are one dot product
 // each.  A warp issues an FP64 instruction every 64 cycles (its quarter of the
-// SM's FP64 pipe), so what counts is their number: a reciprocal square root (the
-// library's; one of five FP64 instructions written out here was no faster, 222 us
-// against 218 for a factorization of n = 500) and k + 2 products for pivot k; the
+// SM's FP64 pipe), so what counts is their number, 7 + k for pivot k; the
 // diagonal of R is left to one product at the end.  A pivot that is not positive
 // is taken as 1 and reported.
 static __device__ __noinline__ bool warp_chol_inv(double* M, int ld, int r, double* Rd, int lane) {
@@ -133,7 +144,7 @@ static __device__ __noinline__ bool warp_chol_inv(double* M, int ld, int r, doub
       ok = false;
       d = 1.0;
     }
-    const double rs = rsqrt(d);
+    const double rs = rsqrt_householder(d);
     const double own = lane == k ? rs : acc * rs;
     if (lane == k) Rd[k] = d;
     if (lane < r) M[k * ld + lane] = own;

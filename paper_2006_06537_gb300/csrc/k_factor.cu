@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(256, 7)
       d = 1.0;
       A[k * ld + k] = d;
     }
-    rinv[k] = rsqrt(d);
+    rinv[k] = rsqrt_householder(d);
   };
   if (threadIdx.x == 0) flag[0] = 0;
   // column k ready for its step: pivot, column k of L and row k of X scaled
